@@ -17,6 +17,7 @@
 #include "adam.cuh"
 #include "common.cuh"
 #include "gemm_apply.cuh"
+#include "gemm_fma.cuh"
 #include "gemm_split.cuh"
 #include "gemm_tc.cuh"
 #include "refresh.cuh"
@@ -118,7 +119,7 @@ struct galore_layer {
   int q_block;
   int64_t nblk;
   int block;             // columns of the refresh block
-  int proj_splits;       // K slices of the projection on the path of split operands
+  int proj_splits;       // K slices of the projection on the fp32 path
   int tc_splits;         // K slices of the projection on the tensor-core path
   int64_t ld_part, ld_n; // padded row pitches of the R partials and of N
   int p_planes;          // bf16 planes the projector is split into for the weight update, 0: it is used where it lies
@@ -155,6 +156,9 @@ struct Sizes {
   size_t off_vrow, off_vcol;
   size_t off_status, off_R, off_N, off_Pp, off_af, off_refresh, ws_bytes;
 };
+
+// Layers whose W and G are both fp32 keep one order of the projection's sums (gemm_fma.cu says why).
+bool fma_projection(const galore_config_t& c) { return c.w_dtype == GALORE_F32 && c.g_dtype == GALORE_F32; }
 
 galore_status_t resolve(const galore_config_t* c, Sizes* s) {
   if (!c || !s) return GALORE_ERR_INVALID_ARG;
@@ -200,8 +204,7 @@ galore_status_t resolve(const galore_config_t* c, Sizes* s) {
   s->block = (int)std::min<int64_t>(s->d, (int64_t)r + over);
 
   // K slices of the projection
-  s->proj_splits = s->left ? split_choose_slices(r, c->n, c->m)
-                           : split_choose_slices(c->m, r, c->n);
+  s->proj_splits = fma_projection(*c) ? fma_choose_slices(s->srows, s->scols, s->d) : split_choose_slices(s->srows, s->scols, s->d);
   s->tc_splits = s->tensor_path ? tensor_proj_splits(*c, s->left) : 0;
   s->ld_part = (s->scols + 7) / 8 * 8;     // 32-byte rows for whole-sector vector stores
   s->ld_n = (s->scols + 15) / 16 * 16;     // 32-byte bf16 rows: TMA needs 16, the epilogue that writes N stores 32 at a time
@@ -250,17 +253,50 @@ galore_status_t convert_copy(const TS* src, TD* dst, int64_t count, cudaStream_t
   return GALORE_OK;
 }
 
-// ---- the two projections with split operands (fp32 tensors, or rows TMA cannot address) -------------
+// ---- the two projections of the fp32 path (fp32 tensors, or rows TMA cannot address) -------------
 
-// R (r x n) = P^T G (left) resp. R (m x r) = G Q into `part`
-galore_status_t split_add_project(SplitGroup& g, const galore_layer* l, const void* G, int64_t ldg, float* part, int splits) {
-  const galore_config_t& c = l->cfg;
-  const int64_t stride = l->srows * l->ld_part;
-  if (l->left)
-    return split_group_add_store(g, c.rank, (int)c.n, (int)c.m, split_operand(l->P, c.p_dtype, 1, c.rank),
-                                 split_operand(G, c.g_dtype, 1, ldg), splits, part, l->ld_part, stride, l->status);
-  return split_group_add_store(g, (int)c.m, c.rank, (int)c.n, split_operand(G, c.g_dtype, ldg, 1),
-                               split_operand(l->P, c.p_dtype, 1, c.rank), splits, part, l->ld_part, stride, l->status);
+// R (r x n) = P^T G (left) resp. R (m x r) = G Q of one layer into `part`
+struct ProjectJob {
+  const galore_layer* l;
+  const void* G;
+  int64_t ldg;
+  float* part;
+  int splits;
+};
+// All layers have the types of the first; layers of both sides only where P and G have one type.
+galore_status_t launch_projections(const ProjectJob* jobs, int count, bool early, cudaStream_t st) {
+  const galore_config_t& kind = jobs[0].l->cfg;
+  const int32_t a_dtype = jobs[0].l->left ? kind.p_dtype : kind.g_dtype, b_dtype = jobs[0].l->left ? kind.g_dtype : kind.p_dtype;
+  if (fma_projection(kind)) {
+    FmaGroup g;
+    g.count = 0;
+    for (int i = 0; i < count; ++i) {
+      const ProjectJob& j = jobs[i];
+      const galore_config_t& c = j.l->cfg;
+      const int64_t r = c.rank;
+      FmaProblem p = {};
+      if (j.l->left) p = FmaProblem{c.rank, (int)c.n, (int)c.m, j.l->P, j.G, 1, r, j.ldg, 1};
+      else p = FmaProblem{(int)c.m, c.rank, (int)c.n, j.G, j.l->P, j.ldg, 1, r, 1};
+      p.C = j.part; p.ldc = j.l->ld_part; p.split_stride = j.l->srows * j.l->ld_part;
+      GALORE_TRY(fma_group_add(g, p, j.splits));
+    }
+    return launch_fma_group(g, a_dtype, b_dtype, early, st);
+  }
+  SplitGroup g;
+  g.count = 0;
+  for (int i = 0; i < count; ++i) {
+    const ProjectJob& j = jobs[i];
+    const galore_layer* l = j.l;
+    const galore_config_t& c = l->cfg;
+    const int64_t stride = l->srows * l->ld_part;
+    if (l->left)
+      GALORE_TRY(split_group_add_store(g, c.rank, (int)c.n, (int)c.m, split_operand(l->P, c.p_dtype, 1, c.rank),
+                                       split_operand(j.G, c.g_dtype, 1, j.ldg), j.splits, j.part, l->ld_part, stride, l->status));
+    else
+      GALORE_TRY(split_group_add_store(g, (int)c.m, c.rank, (int)c.n, split_operand(j.G, c.g_dtype, j.ldg, 1),
+                                       split_operand(l->P, c.p_dtype, 1, c.rank), j.splits, j.part, l->ld_part, stride, l->status));
+  }
+  return launch_split_store(g, a_dtype, b_dtype, early, st);
 }
 // W <- keep W - scale P N (left) resp. N Q^T: N in n_planes bf16 planes, P where it lies or in the planes at `pp`
 ApplyItem apply_item(const galore_layer* l, const __nv_bfloat16* N, int n_planes, const __nv_bfloat16* pp, void* W, int64_t ldw, float lr) {
@@ -280,10 +316,6 @@ PlaneSplit projector_split(const galore_layer* l, __nv_bfloat16* pp) {
   PlaneSplit s = {};
   if (l->p_planes) s = PlaneSplit{l->P, pp, l->cfg.p_dtype, (int)l->d, l->cfg.rank, (int)l->ld_p, l->p_planes};
   return s;
-}
-galore_status_t split_launch_project(const SplitGroup& g, const galore_layer* kind, bool early, cudaStream_t st) {
-  const galore_config_t& c = kind->cfg;
-  return kind->left ? launch_split_store(g, c.p_dtype, c.g_dtype, early, st) : launch_split_store(g, c.g_dtype, c.p_dtype, early, st);
 }
 // the layer's share of an Adam launch: R partials in `part`, N to `nbuf`
 AdamItem adam_item(const galore_layer* l, const float* part, int splits, __nv_bfloat16* nbuf, const AdamParams& ap) {
@@ -328,10 +360,8 @@ galore_status_t step_split(galore_layer* l, void* W, int64_t ldw, const void* G,
                            const AdamParams& ap, cudaStream_t st) {
   {
     PhaseTimer pt(0, st);
-    SplitGroup g;
-    g.count = 0;
-    GALORE_TRY(split_add_project(g, l, G, ldg, l->Rpart, l->proj_splits));
-    GALORE_TRY(split_launch_project(g, l, true, st));     // early: see step_tensor
+    const ProjectJob job{l, G, ldg, l->Rpart, l->proj_splits};
+    GALORE_TRY(launch_projections(&job, 1, true, st));     // early: see step_tensor
   }
   {
     PhaseTimer pt(1, st);
@@ -1072,10 +1102,9 @@ galore_status_t galore_step_batch(galore_layer_t* const* layers, void* const* W,
     const bool early = short_group(fgroups[gi]);
     {
       PhaseTimer pt(0, st);
-      SplitGroup g;
-      g.count = 0;
-      for (const SplitMember& q : ps) GALORE_TRY(split_add_project(g, q.l, q.G, q.ldg, q.part(), q.splits));
-      GALORE_TRY(split_launch_project(g, first, early && (gi > 0 || !groups.empty()), st));
+      std::vector<ProjectJob> jobs;
+      for (const SplitMember& q : ps) jobs.push_back(ProjectJob{q.l, q.G, q.ldg, q.part(), q.splits});
+      GALORE_TRY(launch_projections(jobs.data(), (int)jobs.size(), early && (gi > 0 || !groups.empty()), st));
     }
     {
       scratch.adam->count = 0;

@@ -1,0 +1,188 @@
+// Products with fp32 FMA.
+//
+// Why they stand beside the faster split products (gemm_split.cuh), whose sums are nearer to the exact ones: with both moments
+// young, Eq. 15 is N = r / (|r| + eps), and an r that the sum over K all but cancels hands its rounding to N undamped.  An
+// fp32 W shows that: for 512 x 1376 at rank 128 two sums that differ in their last bits gave weights 8.5e-5 apart in 1 of 40
+// runs (each 1.6e-5 to 6.9e-5 from those of a product in 64 bits).  Such layers therefore keep one fixed order of their
+// sums: fmaf over k, slice after slice.  Where W or G is bf16 its rounding hides the difference, and the split products
+// carry the projection.
+//
+// What bounds it: the FMA rate of a 128 x 128 tile of 256 threads for large matrices; for small ones the latency of the K loop,
+// 16 k at a time with the next ones on their way.
+#include "gemm_fma.cuh"
+
+#include <algorithm>
+
+#include "launch.cuh"
+#include "tc_ptx.cuh"
+
+namespace galore {
+
+namespace {
+
+constexpr int kBK = 16;
+constexpr int kThreads = 256;
+
+// BM x BN tile, TM x TN elements a thread in groups of four
+template <typename TA, typename TB, int BM, int BN, int TM, int TN, int CAP>
+__global__ void __launch_bounds__(kThreads) gemm_fma_kernel(const __grid_constant__ FmaArgs<CAP> g) {
+  static_assert((BM / TM) * (BN / TN) == kThreads, "one micro-tile a thread");
+  constexpr int LA = BM * kBK / kThreads, LB = BN * kBK / kThreads;      // elements of a tile each thread fetches
+  __shared__ float As[kBK][BM + 4];
+  __shared__ float Bs[kBK][BN + 4];
+  grid_dependency_wait();
+  grid_launch_dependents();
+  GroupCursor cursor;
+  int local = cursor.seek<CAP>(g, (int)blockIdx.x);
+  const FmaProblem& p = g.p[cursor.pi];
+  const int tiles_n = (p.N + BN - 1) / BN, tiles_m = (p.M + BM - 1) / BM;
+  const int n0 = (local % tiles_n) * BN;
+  local /= tiles_n;
+  const int m0 = (local % tiles_m) * BM, slice = local / tiles_m;
+  const int k_begin = slice * p.kchunk, k_end = min(p.K, k_begin + p.kchunk);
+  const TA* A = (const TA*)p.A;
+  const TB* B = (const TB*)p.B;
+  const int64_t sAi = p.sAi, sAk = p.sAk, sBk = p.sBk, sBj = p.sBj;
+  const int M = p.M, N = p.N;
+
+  const int tid = threadIdx.x;
+  const int tx = tid % (BN / TN), ty = tid / (BN / TN);
+  const bool a_kfast = (sAk == 1);   // consecutive threads walk the contiguous direction
+  const bool b_kfast = (sBk == 1);
+
+  float acc[TM][TN];
+#pragma unroll
+  for (int u = 0; u < TM; ++u)
+#pragma unroll
+    for (int v = 0; v < TN; ++v) acc[u][v] = 0.f;
+
+  float ra[LA], rb[LB];
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int e = 0; e < LA; ++e) {
+      const int idx = tid + e * kThreads;
+      const int i = a_kfast ? idx / kBK : idx % BM;
+      const int k = a_kfast ? idx % kBK : idx / BM;
+      const int gi = m0 + i, gk = k0 + k;
+      ra[e] = (gi < M && gk < k_end) ? cvt<float>(A[(int64_t)gi * sAi + (int64_t)gk * sAk]) : 0.f;
+    }
+#pragma unroll
+    for (int e = 0; e < LB; ++e) {
+      const int idx = tid + e * kThreads;
+      const int j = b_kfast ? idx / kBK : idx % BN;
+      const int k = b_kfast ? idx % kBK : idx / BN;
+      const int gj = n0 + j, gk = k0 + k;
+      rb[e] = (gj < N && gk < k_end) ? cvt<float>(B[(int64_t)gk * sBk + (int64_t)gj * sBj]) : 0.f;
+    }
+  };
+  auto stash = [&]() {
+#pragma unroll
+    for (int e = 0; e < LA; ++e) {
+      const int idx = tid + e * kThreads;
+      As[a_kfast ? idx % kBK : idx / BM][a_kfast ? idx / kBK : idx % BM] = ra[e];
+    }
+#pragma unroll
+    for (int e = 0; e < LB; ++e) {
+      const int idx = tid + e * kThreads;
+      Bs[b_kfast ? idx % kBK : idx / BN][b_kfast ? idx / kBK : idx % BN] = rb[e];
+    }
+  };
+
+  if (k_begin < k_end) fetch(k_begin);
+  for (int k0 = k_begin; k0 < k_end; k0 += kBK) {
+    __syncthreads();
+    stash();
+    __syncthreads();
+    if (k0 + kBK < k_end) fetch(k0 + kBK);
+#pragma unroll
+    for (int k = 0; k < kBK; ++k) {
+      float a[TM], b[TN];
+#pragma unroll
+      for (int u = 0; u < TM; ++u) a[u] = As[k][(u / 4) * (BM / (TM / 4)) + ty * 4 + (u % 4)];
+#pragma unroll
+      for (int v = 0; v < TN; ++v) b[v] = Bs[k][(v / 4) * (BN / (TN / 4)) + tx * 4 + (v % 4)];
+#pragma unroll
+      for (int u = 0; u < TM; ++u)
+#pragma unroll
+        for (int v = 0; v < TN; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
+    }
+  }
+  // a thread's columns come in runs of four: one 16-byte store where the rows allow it
+  float* const C = p.C + (int64_t)slice * p.split_stride;
+  const bool vec = (((uintptr_t)C & 15) == 0) && (p.ldc % 4) == 0;
+#pragma unroll
+  for (int u = 0; u < TM; ++u) {
+    const int i = m0 + (u / 4) * (BM / (TM / 4)) + ty * 4 + (u % 4);
+    if (i >= M) continue;
+#pragma unroll
+    for (int vg = 0; vg < TN / 4; ++vg) {
+      const int j = n0 + vg * (BN / (TN / 4)) + tx * 4;
+      float* dst = C + (int64_t)i * p.ldc + j;
+      if (j + 3 < N && vec) {
+        *reinterpret_cast<float4*>(dst) = make_float4(acc[u][4 * vg], acc[u][4 * vg + 1], acc[u][4 * vg + 2], acc[u][4 * vg + 3]);
+      } else {
+#pragma unroll
+        for (int v = 0; v < 4; ++v)
+          if (j + v < N) dst[v] = acc[u][4 * vg + v];
+      }
+    }
+  }
+}
+
+// Results below 96 tiles of 128 x 128 are cut into 64 x 64.
+bool small_result(int64_t M, int64_t N) { return M * N < (int64_t)128 * 128 * 96; }
+
+template <typename TA, typename TB>
+galore_status_t launch_typed(const FmaGroup& g, bool early, cudaStream_t st) {
+  if (g.count > 1)
+    return launch_kernel(gemm_fma_kernel<TA, TB, 128, 128, 8, 8, kFmaGroup>, dim3((unsigned)g.unit_end[g.count - 1]), kThreads, 0, 1, early, st, g);
+  FmaArgs<1> one;
+  const FmaProblem& p = one.p[0] = g.p[0];
+  one.count = 1;
+  const bool small = small_result(p.M, p.N);
+  const int64_t t = small ? 64 : 128;
+  one.unit_end[0] = (int)(ceil_div(p.M, t) * ceil_div(p.N, t) * p.splits);
+  const dim3 grid((unsigned)one.unit_end[0]);
+  if (small) return launch_kernel(gemm_fma_kernel<TA, TB, 64, 64, 4, 4, 1>, grid, kThreads, 0, 1, early, st, one);
+  return launch_kernel(gemm_fma_kernel<TA, TB, 128, 128, 8, 8, 1>, grid, kThreads, 0, 1, early, st, one);
+}
+
+int chunk_of(int64_t K, int slices) { return (int)(std::max<int64_t>(1, ceil_div(ceil_div(K, std::max(1, slices)), kBK)) * kBK); }
+
+}  // namespace
+
+int fma_effective_slices(int64_t K, int slices) { return (int)ceil_div(std::max<int64_t>(1, K), chunk_of(K, slices)); }
+
+int fma_choose_slices(int64_t M, int64_t N, int64_t K) {
+  const int64_t t = small_result(M, N) ? 64 : 128;
+  const int64_t tiles = ceil_div(M, t) * ceil_div(N, t);
+  int64_t want = std::min<int64_t>(16, std::max<int64_t>(1, ceil_div(2 * 148, tiles)));
+  want = std::min<int64_t>(want, std::max<int64_t>(1, K / 64));
+  return fma_effective_slices(K, (int)want);
+}
+
+galore_status_t fma_group_add(FmaGroup& g, const FmaProblem& problem, int slices) {
+  if (g.count >= kFmaGroup) return GALORE_ERR_BUFFER_TOO_SMALL;
+  FmaProblem p = problem;
+  if (p.M <= 0 || p.N <= 0 || p.K <= 0) return GALORE_ERR_SHAPE;
+  p.kchunk = chunk_of(p.K, slices);
+  p.splits = fma_effective_slices(p.K, slices);
+  const int64_t ctas = ceil_div(p.M, 128) * ceil_div(p.N, 128) * p.splits;
+  const int64_t before = g.count ? g.unit_end[g.count - 1] : 0;
+  if (before + 4 * ctas >= ((int64_t)1 << 31)) return GALORE_ERR_SHAPE;
+  g.p[g.count] = p;
+  g.unit_end[g.count] = (int)(before + ctas);
+  g.count += 1;
+  return GALORE_OK;
+}
+
+galore_status_t launch_fma_group(const FmaGroup& g, int32_t a_dtype, int32_t b_dtype, bool early, cudaStream_t st) {
+  if (g.count < 1) return GALORE_OK;
+  const bool ab = a_dtype == GALORE_BF16, bb = b_dtype == GALORE_BF16;
+  if (ab && bb) return GALORE_ERR_INVALID_ARG;       // the split products are as exact
+  if (ab) return launch_typed<__nv_bfloat16, float>(g, early, st);
+  if (bb) return launch_typed<float, __nv_bfloat16>(g, early, st);
+  return launch_typed<float, float>(g, early, st);
+}
+
+}  // namespace galore

@@ -21,7 +21,7 @@
 #include "adam.cuh"
 #include "common.cuh"
 #include "gemm_apply.cuh"
-#include "gemm_split.cuh"
+#include "gemm_fma.cuh"
 #include "gemm_tc.cuh"
 
 namespace galore {
@@ -107,8 +107,8 @@ extern "C" galore_status_t galore_step_static(int64_t m, int64_t n, int32_t rank
 
   // The step is independent along the wide side: where the array does not hold the intermediates of the whole matrix it
   // is done in strips.  Layout inside the array: [status words 256 B][R partials][planes of N][planes of P, whole or a
-  // range of rows].  The K slices are those of the regular fp32 path (results agree bit for bit), fewer where they do
-  // not fit.
+  // range of rows].  The K slices are those that the regular path gives the whole matrix, so that the moments agree bit for
+  // bit; fewer where even the narrowest strip would not hold them.
   const AdamParams ap = make_adam_params(beta1, beta2, eps, (double)(completed_steps + 1));
   const float scale = lr * alpha;
   const int64_t d = left ? m : n, ldp = ((int64_t)r + 7) / 8 * 8;
@@ -119,11 +119,15 @@ extern "C" galore_status_t galore_step_static(int64_t m, int64_t n, int32_t rank
   auto rows_of = [&](int64_t w) { return left ? (int64_t)r : w; };
   auto cols_of = [&](int64_t w) { return left ? w : (int64_t)r; };
   auto need = [&](int64_t w, int splits) { return r_bytes(rows_of(w), cols_of(w), splits) + n_bytes(rows_of(w), cols_of(w)) + p_least; };
-  int64_t strip = wide;
-  for (int64_t parts = 2; strip > 256 && need(strip, 1) > room; ++parts) strip = align_up(ceil_div(wide, parts), 256);
-  if (need(strip, 1) > room) return GALORE_ERR_BUFFER_TOO_SMALL;
-  int splits = left ? split_choose_slices(r, strip, m) : split_choose_slices(strip, r, n);
-  while (splits > 1 && need(strip, splits) > room) splits = split_effective_slices(d, splits - 1);
+  auto strip_of = [&](int splits) {
+    int64_t strip = wide;
+    for (int64_t parts = 2; strip > 256 && need(strip, splits) > room; ++parts) strip = align_up(ceil_div(wide, parts), 256);
+    return strip;
+  };
+  int splits = fma_choose_slices(rows_of(wide), cols_of(wide), d);
+  while (splits > 1 && need(strip_of(splits), splits) > room) splits = fma_effective_slices(d, splits - 1);
+  const int64_t strip = strip_of(splits);
+  if (need(strip, splits) > room) return GALORE_ERR_BUFFER_TOO_SMALL;
   float* const Rpart = (float*)((char*)base + 256);
   __nv_bfloat16* const Nbuf = (__nv_bfloat16*)((char*)Rpart + r_bytes(rows_of(strip), cols_of(strip), splits));
   __nv_bfloat16* const planes = (__nv_bfloat16*)((char*)Nbuf + n_bytes(rows_of(strip), cols_of(strip)));
@@ -139,15 +143,12 @@ extern "C" galore_status_t galore_step_static(int64_t m, int64_t n, int32_t rank
       const float* Gs = left ? G + w0 : G + w0 * ldg;
       float* Ws = left ? W + w0 : W + w0 * ldw;
       const int64_t state_at = left ? w0 : w0 * scols_all;
-      SplitGroup g;
+      FmaProblem proj = left ? FmaProblem{r, (int)w, (int)m, P, Gs, 1, r, ldg, 1} : FmaProblem{(int)w, r, (int)n, Gs, P, ldg, 1, r, 1};
+      proj.C = Rpart; proj.ldc = ld; proj.split_stride = srows * ld;
+      FmaGroup g;
       g.count = 0;
-      if (left)
-        GALORE_TRY(split_group_add_store(g, r, (int)w, (int)m, split_operand(P, GALORE_F32, 1, r), split_operand(Gs, GALORE_F32, 1, ldg),
-                                         splits, Rpart, ld, srows * ld, status));
-      else
-        GALORE_TRY(split_group_add_store(g, (int)w, r, (int)n, split_operand(Gs, GALORE_F32, ldg, 1), split_operand(P, GALORE_F32, 1, r),
-                                         splits, Rpart, ld, srows * ld, status));
-      GALORE_TRY(launch_split_store(g, GALORE_F32, GALORE_F32, false, st));
+      GALORE_TRY(fma_group_add(g, proj, splits));
+      GALORE_TRY(launch_fma_group(g, GALORE_F32, GALORE_F32, false, st));
 
       AdamItem item = {};
       item.Rpart = Rpart; item.splits = g.p[0].splits; item.split_stride = srows * ld;

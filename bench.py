@@ -11,7 +11,8 @@ N > 1 (under torch.distributed.run) runs N independent replicas of the same
 workload, one per GPU: the path has no exchange step, so nothing is sharded
 and no collective is on the data path; only the timing is reduced over ranks.
 `--impl reference` times the CPU oracle on the host cores on a bounded sample.
-Prints ONE JSON line on rank 0.
+Prints ONE JSON line on rank 0; the full record (the refresh of every shape, the other workloads' own rooflines) goes to
+standard error as another.
 """
 from __future__ import annotations
 
@@ -115,6 +116,24 @@ def kernel_costs(w, shapes):
         back["flops"] += 2 * m * n * r
         back["bytes"] += 2 * m * n * elem_bytes(w.w_dtype) + p_bytes + nel * n_b
     return proj, adam, back
+
+
+def summary(res):
+    """What the line on standard output holds: readers keep a few thousand characters of it.  The parts of a record that only
+    explain its figures (per-shape refresh phases, the other workloads' kernels) are left to the full record."""
+    def short(x):
+        if isinstance(x, float):
+            return float(f"{x:.7g}")
+        if isinstance(x, dict):
+            return {k: short(v) for k, v in x.items()}
+        return [short(v) for v in x] if isinstance(x, (list, tuple)) else x
+
+    out = {k: short(v) for k, v in res.items() if k not in ("refresh", "refresh_set", "refresh_amortised", "other_workloads")}
+    if "other_workloads" in res:
+        out["other_workloads"] = [
+            {"workload": x["config"]["workload"], "rank": x["config"]["rank"], "state_fmt": x["config"]["state_fmt"],
+             "value": short(x["value"]), "ms_per_step": short(x["ms_per_step"])} for x in res["other_workloads"]]
+    return out
 
 
 def max_over_ranks(value: float, dist, device) -> float:
@@ -350,7 +369,8 @@ def main():
                 extras.append(time_workload(wl.WORKLOADS[name], args, dev, None, 1, 0, full=False))
         if extras:
             res["other_workloads"] = extras
-        print(json.dumps(res), flush=True)
+        print(json.dumps(res), file=sys.stderr, flush=True)
+        print(json.dumps(summary(res)), flush=True)
     if dist is not None:
         dist.barrier()
         dist.destroy_process_group()

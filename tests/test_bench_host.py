@@ -72,3 +72,28 @@ def test_clock_sampler_tolerates_a_missing_nvidia_smi():
     s.start()
     res = s.stop()
     assert set(res) >= {"sm_mhz", "sm_max_mhz", "reasons"}
+
+
+def test_the_printed_line_keeps_the_figures_and_stays_short():
+    """A line of every workload's full record was cut off by its readers."""
+    phase = {"ms_per_step": 13.066239953041076, "launches_per_step": 1.0, "tflops": 1413.4410082145796, "gbs": 818.5579966722333,
+             "roof_ms": 0.133789911422776, "frac_of_own_roof": 1.0239358216564616}
+    refresh = [{"shape": [4096, 11008], "count": 64, "ms": 128.64598083496094, "iterations": 18, "residual": 6.749436290840305e-06}] * 3
+    config = {"workload": "llama_7b_q8", "rank": 1024, "state_fmt": "q8", "l2": "inputs larger than L2 (whole layer set streamed each step)"}
+    gaps = {str(t): 43726525071.28677 for t in (50, 200, 1000)}
+    record = {"metric": bench.METRIC, "value": 226123456789.12345, "unit": bench.UNIT, "n_gpus": 1, "steps": 20, "warmup": 5,
+              "ms_per_step": 28.612345678901234, "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "bf16",
+              "data": "synthetic", "config": config, "clocks": {"sm_mhz": 1507.0, "sm_max_mhz": 1965.0, "reasons": ["sw_power_cap"], "samples": 6},
+              "gpu_launches": 420, "roofline": {"bound": "tensor", "frac": 0.6904188076514539, "kernels": {k: phase for k in "abc"},
+                                                "traffic": {k: 3645065883.062857 for k in "abc"}, "refresh_amortised": {"by_gap": gaps}},
+              "refresh": refresh, "refresh_set": {"ms": 6000.0}, "refresh_amortised": {"by_gap": gaps},
+              "e2e": {"value": 11544679720.197325, "unit": bench.UNIT, "h2d_bytes_per_step": 1, "d2h_bytes_per_step": 2}, "device_status": 0}
+    record["other_workloads"] = [{k: record[k] for k in ("value", "ms_per_step", "config", "roofline", "refresh", "clocks")} for _ in range(16)]
+    line = json.dumps(bench.summary(record))
+    assert len(line) < 5000 < len(json.dumps(record))
+    got = json.loads(line)
+    for key in ("metric", "unit", "n_gpus", "steps", "warmup", "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "config", "clocks",
+                "gpu_launches"):
+        assert got[key] == record[key]
+    assert abs(got["value"] / record["value"] - 1) < 1e-6 and abs(got["ms_per_step"] / record["ms_per_step"] - 1) < 1e-6
+    assert got["e2e"]["h2d_bytes_per_step"] == 1 and len(got["other_workloads"]) == 16

@@ -33,6 +33,8 @@
  *     each needs a whole SM's tensor memory and shared memory, so they would
  *     not overlap anyway, and runs that kept several streams of them in flight
  *     stalled on the test machines for a reason that was not found.
+ *   - A step (of one layer, of a batch, static) may be captured into a CUDA graph on any stream; a
+ *     call inside a capture is neither chained behind earlier calls nor are later ones behind it.
  *   - Every entry point returns a galore_status_t: 0 ok, > 0 warning, < 0
  *     error.  Nothing throws or aborts across this boundary.  Conditions
  *     detected on the device (non-finite values, a bounded wait that ran out)
@@ -272,8 +274,8 @@ galore_status_t galore_free(galore_layer_t* layer);
  *     GALORE_ERR_BUFFER_TOO_SMALL and nothing is launched.
  *   - The first call on each device looks up the array's device address (with that device
  *     current).  Make that first call outside of any stream capture.
- *   - `stream` must belong to the current device (checked: GALORE_ERR_INVALID_ARG otherwise); the
- *     array that is used is the current device's.
+ *   - `stream` must belong to the current device (checked outside of a capture:
+ *     GALORE_ERR_INVALID_ARG otherwise); the array that is used is the current device's.
  *   - All calls on a device share the array, and it keeps the previous call's contents.  The call
  *     clears the status word it needs at zero; everything else it reads it has written first.
  *     Calls whose GPU work can overlap (two streams, two threads) race on the array: serialise

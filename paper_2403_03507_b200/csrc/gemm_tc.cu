@@ -33,7 +33,6 @@
 #include <algorithm>
 #include <atomic>
 #include <memory>
-#include <mutex>
 #include <new>
 
 namespace galore {
@@ -766,42 +765,28 @@ int tensor_sm_count() {
   return sms;
 }
 
-namespace {
-
-// Launches of these kernels given on different streams are chained with an event, in the order of
-// the calls.  One CTA takes a whole SM's tensor memory and nearly all of its shared memory, so two
-// of them never share an SM and little is lost; runs that kept several streams of them in flight
-// did not finish on the test machines, and no cause was found in the code.
-struct StreamChain {
-  std::mutex mutex;
-  cudaStream_t last[64] = {};
-  cudaEvent_t done[64] = {};
-  bool used[64] = {};
-};
-StreamChain g_chain;
-
-galore_status_t chain_before(cudaStream_t st, int dev) {
-  if (g_chain.used[dev] && g_chain.last[dev] != st) GALORE_CUDA_TRY(cudaStreamWaitEvent(st, g_chain.done[dev], 0));
+galore_status_t CudaOrder::capturing(cudaStream_t st, bool* on) {
+  cudaStreamCaptureStatus c = cudaStreamCaptureStatusNone;
+  GALORE_CUDA_TRY(cudaStreamIsCapturing(st, &c));
+  *on = c != cudaStreamCaptureStatusNone;
   return GALORE_OK;
 }
-galore_status_t chain_after(cudaStream_t st, int dev) {
-  if (!g_chain.done[dev]) GALORE_CUDA_TRY(cudaEventCreateWithFlags(&g_chain.done[dev], cudaEventDisableTiming));
-  GALORE_CUDA_TRY(cudaEventRecord(g_chain.done[dev], st));
-  g_chain.last[dev] = st;
-  g_chain.used[dev] = true;
+galore_status_t CudaOrder::wait(cudaStream_t st, cudaEvent_t e) {
+  GALORE_CUDA_TRY(cudaStreamWaitEvent(st, e, 0));
+  return GALORE_OK;
+}
+galore_status_t CudaOrder::create(cudaEvent_t* e) {
+  GALORE_CUDA_TRY(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+  return GALORE_OK;
+}
+galore_status_t CudaOrder::record(cudaEvent_t e, cudaStream_t st) {
+  GALORE_CUDA_TRY(cudaEventRecord(e, st));
   return GALORE_OK;
 }
 
-}  // namespace
-
-galore_status_t tensor_launch_in_order(cudaStream_t st, const std::function<galore_status_t()>& launch) {
-  int dev = 0;
-  GALORE_CUDA_TRY(cudaGetDevice(&dev));
-  if (dev < 0 || dev >= 64) return GALORE_ERR_INVALID_ARG;
-  std::lock_guard<std::mutex> lock(g_chain.mutex);
-  GALORE_TRY(chain_before(st, dev));
-  GALORE_TRY(launch());
-  return chain_after(st, dev);
+LaunchOrder<CudaOrder>& launch_order() {
+  static LaunchOrder<CudaOrder> order;
+  return order;
 }
 
 namespace {

@@ -3,9 +3,10 @@
 
 #include <cuda.h>
 
-#include <functional>
+#include <utility>
 
 #include "common.cuh"
+#include "launch_order.h"
 #include "q8_code.cuh"
 
 namespace galore {
@@ -62,10 +63,25 @@ galore_status_t tensor_group_add_gemm(TensorGroup* t, const void* A, int64_t lda
                                       int b_mn, int M, int N, int K, float* C, int64_t ldc, int32_t* status);
 galore_status_t tensor_group_launch_project(TensorGroup* t, bool early, cudaStream_t st);
 
-
+struct CudaOrder {
+  using Status = galore_status_t;
+  using Stream = cudaStream_t;
+  using Event = cudaEvent_t;
+  static Status capturing(Stream st, bool* on);
+  static Status wait(Stream st, Event e);
+  static Status create(Event* e);
+  static Status record(Event e, Stream st);
+};
+LaunchOrder<CudaOrder>& launch_order();
 // Runs `launch` (which queues kernels that allocate tensor memory on st) after every such kernel queued before it,
-// whatever their streams; see the note at its definition.  The entry points call it, once around all their launches.
-galore_status_t tensor_launch_in_order(cudaStream_t st, const std::function<galore_status_t()>& launch);
+// whatever their streams; see launch_order.h.  The entry points call it, once around all their launches.
+template <class F>
+galore_status_t tensor_launch_in_order(cudaStream_t st, F&& launch) {
+  int dev = 0;
+  GALORE_CUDA_TRY(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= LaunchOrder<CudaOrder>::kDevices) return GALORE_ERR_INVALID_ARG;
+  return launch_order().run(dev, st, std::forward<F>(launch));
+}
 int tensor_sm_count();
 // a matrix of rows x cols elements (cols contiguous) with boxes of box_rows x box_cols, 128-byte swizzle
 galore_status_t tensor_encode(CUtensorMap* map, const void* base, int32_t dtype, int64_t rows, int64_t cols, int64_t ld,

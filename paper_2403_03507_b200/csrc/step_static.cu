@@ -58,6 +58,9 @@ __global__ void fold_status_kernel(int32_t* words) {
 // the stream, if one is given, must live on the device whose array is about to be used
 static galore_status_t check_stream_device(cudaStream_t st) {
   if (!st || st == cudaStreamLegacy || st == cudaStreamPerThread) return GALORE_OK;
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  GALORE_CUDA_TRY(cudaStreamIsCapturing(st, &capture));
+  if (capture != cudaStreamCaptureStatusNone) return GALORE_OK;      // a captured stream does not tell its device
   int cur = 0, dev = 0;
   GALORE_CUDA_TRY(cudaGetDevice(&cur));
   GALORE_CUDA_TRY(cudaStreamGetDevice(st, &dev));

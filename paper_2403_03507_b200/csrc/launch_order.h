@@ -39,8 +39,8 @@ class LaunchOrder {
       if (w < 0) return w;
     }
     const Status l = launch();
-    if (l < 0) return l;
-    return after(d, st);
+    const Status r = after(d, st);      // also behind a call that failed half-way: what it had queued runs
+    return l < 0 ? l : r;
   }
 
  private:

@@ -25,3 +25,9 @@ def test_a_captured_call_neither_waits_nor_records(check):
     assert got[3:5] == ["launch stream 2", "status 0"]
     # the calls after it are chained to the last one outside the capture
     assert got[5:] == ["wait stream 3 event 1", "launch stream 3", "record event 1 stream 3", "status 0"]
+
+
+def test_a_call_that_failed_half_way_is_waited_for(check):
+    # the kernels it had queued before the error are on the stream
+    assert check("fail 1 call 2") == ["launch stream 1", "record event 1 stream 1", "status -5",
+                                      "wait stream 2 event 1", "launch stream 2", "record event 1 stream 2", "status 0"]

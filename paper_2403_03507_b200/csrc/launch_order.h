@@ -32,8 +32,8 @@ class LaunchOrder {
     const Status s = Api::capturing(st, &captured);
     if (s < 0) return s;
     if (captured) return launch();
-    std::lock_guard<std::mutex> lock(mutex_);
     Device& d = devices_[dev];
+    std::lock_guard<std::mutex> lock(d.mutex);      // for the whole call: its kernels follow one another on the stream
     if (d.used && d.last != st) {
       const Status w = Api::wait(st, d.done);
       if (w < 0) return w;
@@ -45,6 +45,7 @@ class LaunchOrder {
 
  private:
   struct Device {
+    std::mutex mutex;
     bool used = false;
     Stream last = {};
     Event done = {};
@@ -60,7 +61,6 @@ class LaunchOrder {
     d.used = true;
     return r;
   }
-  std::mutex mutex_;
   Device devices_[kDevices];
 };
 

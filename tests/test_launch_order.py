@@ -31,3 +31,8 @@ def test_a_call_that_failed_half_way_is_waited_for(check):
     # the kernels it had queued before the error are on the stream
     assert check("fail 1 call 2") == ["launch stream 1", "record event 1 stream 1", "status -5",
                                       "wait stream 2 event 1", "launch stream 2", "record event 1 stream 2", "status 0"]
+
+
+def test_devices_do_not_wait_for_each_other(check):
+    # the launch on one device waits (up to ten seconds) for one on the other to begin, in another thread
+    assert check("both 0 both 1") == ["both launches at once"] * 2

@@ -12,8 +12,8 @@
 // step); otherwise a launch before it leaves them in T, the L_i in the part above the diagonal.
 //
 // What bounds it: for a few blocks the chain of launches, two thirds of each the 64 x 64 factorisation (a step in
-// fp64: 46 thousand cycles, of them 30 the factorisation, 9 the two products, 5 the loads; 73 before the pivots' chain was
-// freed of branches and the products went to the MMA unit); for many the FMA rate.
+// fp64, before the pivots took the library's rsqrt: 46 thousand cycles, of them 30 the factorisation, 9 the two products, 5 the
+// loads; a refresh of 512 x 1376 at rank 128 takes 4.08 ms with it, 3.92 without); for many the FMA rate.
 #include "cholesky.cuh"
 
 #include <algorithm>
@@ -39,18 +39,6 @@ using Tile = S (*)[kLd<S>];
 template <typename S>
 constexpr int chol_smem(int tiles) { return tiles * kB * kLd<S> * (int)sizeof(S); }
 
-// x^-1/2 of a normal number.  It stands in the chain of the 64 pivots: from an approximation with error d, one step of third
-// order (e = 1 - x y^2 = 2 d; y (1 + e / 2 + 3 e^2 / 8), error 5 e^3 / 16) is shorter than two of Newton's.
-__device__ __forceinline__ double pivot_rsqrt(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  const double e = fma(-x * y, y, 1.0);
-  return fma(y * e, fma(e, 0.375, 0.5), y);
-}
-__device__ __forceinline__ float pivot_rsqrt(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double smallest_pivot(double) { return 2.3e-308; }
-__device__ __forceinline__ float smallest_pivot(float) { return 0.0f; }
-
 // ---- factor and inverse of one 64 x 64 block ---------------------------------------------------------
 // A (lower triangle, rows of kLdF) <- L, X (rows of kLdF) <- L^-1 with zeros above the diagonal; W: 32 x 33 of scratch,
 // rdiag: 64 values.  By sub-blocks of 16: one warp factors the diagonal sub-block with its rows in the lanes'
@@ -72,7 +60,7 @@ __device__ __forceinline__ void factor_block(S (*A)[kLdF], S (*X)[kLdF], S (*W)[
       S piv = __shfl_sync(0xffffffffu, r[0], 0);
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
-        const bool unusable = !(piv > smallest_pivot(S(0)));       // not positive definite: go on with a usable pivot, latch the fact
+        const bool unusable = !(piv > S(0));       // not positive definite: go on with a usable pivot, latch the fact
         bad |= unusable;
         piv = unusable ? (S)fabs(piv) + S(1e-30) : piv;
         S raw = S(0), next = S(1);
@@ -80,7 +68,7 @@ __device__ __forceinline__ void factor_block(S (*A)[kLdF], S (*X)[kLdF], S (*W)[
           raw = __shfl_sync(0xffffffffu, r[j], j + 1);
           next = __shfl_sync(0xffffffffu, r[j + 1], j + 1);
         }
-        const S rs = pivot_rsqrt(piv);
+        const S rs = rsqrt(piv);
         const S l = (i == j ? piv : (i > j ? r[j] : S(0))) * rs;
         const S l1 = raw * rs;
         r[j] = l;

@@ -60,7 +60,7 @@ __device__ __forceinline__ BlockPair block_pair(int pair, int round, int nblk) {
 }
 
 // part[(pair * chunks + chunk)] (64 x 64) = rows(pair)[:, chunk] rows(pair)[:, chunk]^T
-__global__ void __launch_bounds__(128) jb_gram_kernel(const double* __restrict__ X, int b, int nblk, int round, int chunks,
+__global__ void __launch_bounds__(128) jb_gram_kernel(const double* X, int b, int nblk, int round, int chunks,
                                                       double* __restrict__ part, const SlotList slots) {
   grid_dependency_wait();
   grid_launch_dependents();
@@ -288,7 +288,7 @@ __device__ __forceinline__ double2 jacobi_rotation(double app, double aqq, doubl
   return turn ? make_double2(c * fix, s * fix) : make_double2(1.0, 0.0);
 }
 
-__global__ void __launch_bounds__(kSweepThreads, 2) jb_sweep_kernel(const double* __restrict__ part, int chunks, int b, int nblk,
+__global__ void __launch_bounds__(kSweepThreads, 2) jb_sweep_kernel(const double* part, int chunks, int b, int nblk,
                                                                  int round, double tol, double* __restrict__ rot_out,
                                                                  int* __restrict__ flags, int* __restrict__ rotations,
                                                                  const SlotList slots) {
@@ -479,7 +479,7 @@ __global__ void __launch_bounds__(kSweepThreads, 2) jb_sweep_kernel(const double
 // is already on its way from global memory into registers, and with one half in shared memory three CTAs
 // fit on an SM.  Warp (wy, wx) forms rows 32 wy .. + 32, columns 16 wx .. + 16 of a half.
 __global__ void __launch_bounds__(256) jb_apply_kernel(double* __restrict__ X, double* __restrict__ Vt, int b, int nblk, int round,
-                                                       const double* __restrict__ rot, const int* __restrict__ flags,
+                                                       const double* rot, const int* flags,
                                                        const SlotList slots, int matrices) {
   grid_dependency_wait();
   grid_launch_dependents();

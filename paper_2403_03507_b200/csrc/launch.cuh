@@ -11,6 +11,8 @@ namespace galore {
 // Device side of programmatic dependent launch.  A kernel that was launched "early" may run beside the end of the kernel
 // before it: nothing that kernel wrote may be read, and nothing it reads may be written, before the wait.  Every kernel
 // of a step waits before it lets its own successor start, so whatever came before its predecessor is complete.
+// Inputs of such a kernel are no `const T* __restrict__` parameters: the compiler would read them as memory that does not
+// change while the kernel runs (ld.global.nc), and until the wait the kernel before it may still write them.
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

@@ -98,8 +98,8 @@ __device__ __forceinline__ double block_sum_256(double v, double* red) {
 // part[blockIdx.x] = this CTA's share of the sum of squares (fixed grid, so the total is reproducible)
 constexpr int kSumsqBlocks = 592;
 // Ynew += delta * Yold,  delta = max(1e-4 * rms column norm of Ynew, 1e-30)
-__global__ void __launch_bounds__(256) shift_kernel(float* __restrict__ Ynew, const float* __restrict__ Yold, int64_t count,
-                                                    int cols, const double* __restrict__ part) {
+__global__ void __launch_bounds__(256) shift_kernel(float* __restrict__ Ynew, const float* Yold, int64_t count,
+                                                    int cols, const double* part) {
   grid_dependency_wait();
   grid_launch_dependents();
   __shared__ double red[8];
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(256) sum_slices_kernel(const Slices s, int64_t
 }
 
 // out = x0 + x1 (+ x2); optionally stored as fp32 and always as a hi/lo pair
-__global__ void sum_split_kernel(const float* __restrict__ x0, const float* __restrict__ x1, const float* __restrict__ x2,
+__global__ void sum_split_kernel(const float* x0, const float* x1, const float* x2,
                                  float* __restrict__ out, __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
                                  int64_t count) {
   grid_dependency_wait();
@@ -175,8 +175,8 @@ __global__ void __launch_bounds__(256) add_sumsq_kernel(const Slices x, int64_t 
 // Ynew += delta * Yold, then the hi/lo pair of Ynew.  delta = 1e-2 x rms column norm here (1e-4 on
 // the fp32 path): the pair carries about 16 bits, so directions kept alive only by the shift must
 // stay well above 2^-16 of the dominant ones for the Gram matrix to remain positive definite.
-__global__ void __launch_bounds__(256) shift_split_kernel(float* __restrict__ Ynew, const float* __restrict__ Yold,
-                                                          int64_t count, int cols, const double* __restrict__ part,
+__global__ void __launch_bounds__(256) shift_split_kernel(float* __restrict__ Ynew, const float* Yold,
+                                                          int64_t count, int cols, const double* part,
                                                           __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo) {
   grid_dependency_wait();
   grid_launch_dependents();
@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(256) shift_split_kernel(float* __restrict__ Yn
 // first step Y1 = (B Y0 - c Y0) / c, second step Y2 = 2 (B Y1 - c Y1) / c - Y0 = T_2((B - c) / c) Y0.
 // The slices add up to the product B y; v = s (B y - c y) - z (z: the block two steps back, or null),
 // stored in x[0] and, where wanted, as a hi/lo pair.
-__global__ void __launch_bounds__(256) cheb_split_kernel(const Slices x, const float* __restrict__ y, const float* __restrict__ z,
+__global__ void __launch_bounds__(256) cheb_split_kernel(const Slices x, const float* y, const float* z,
                                                          float c, float s, int64_t count, __nv_bfloat16* __restrict__ hi,
                                                          __nv_bfloat16* __restrict__ lo) {
   grid_dependency_wait();
@@ -247,7 +247,7 @@ __global__ void gram_sum_kernel(const Slices g, float* __restrict__ C, int64_t c
   }
 }
 
-__global__ void split_kernel(const float* __restrict__ x, __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
+__global__ void split_kernel(const float* x, __nv_bfloat16* __restrict__ hi, __nv_bfloat16* __restrict__ lo,
                              int64_t count) {
   grid_dependency_wait();
   grid_launch_dependents();

@@ -489,7 +489,10 @@ galore_status_t launch_split_variant(const SplitArgs<CAP>& g, bool early, cudaSt
   }
   // setmaxnreg moves registers inside what the CTA was launched with: less than kLaunchRegs would leave it waiting, more
   // would make a step the wrong way
-  if (registers.load(std::memory_order_relaxed) != kLaunchRegs) return GALORE_ERR_CUDA;
+  if (registers.load(std::memory_order_relaxed) != kLaunchRegs) {
+    note_cuda_error(cudaErrorInvalidConfiguration, "gemm_split_kernel: its register split needs a build with 72 registers a thread");
+    return GALORE_ERR_CUDA;
+  }
   GALORE_TRY(allow_smem(configured, (const void*)kern, kSmemBytes));
   return launch_kernel(kern, dim3((unsigned)std::min(units, tensor_sm_count())), kThreads, kSmemBytes, 1, early, st, g);
 }

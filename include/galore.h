@@ -36,7 +36,8 @@
  *   - A step (of one layer, of a batch, static) may be captured into a CUDA graph on any stream; a
  *     call inside a capture is neither chained behind earlier calls nor are later ones behind it.
  *   - Every entry point returns a galore_status_t: 0 ok, > 0 warning, < 0
- *     error.  Nothing throws or aborts across this boundary.  Conditions
+ *     error.  Nothing throws or aborts across this boundary (host memory that
+ *     runs out: GALORE_ERR_INVALID_ARG).  Conditions
  *     detected on the device (non-finite values, a bounded wait that ran out)
  *     are latched in a status word read by galore_device_status().
  */

@@ -514,7 +514,7 @@ galore_status_t galore_query_bytes(const galore_config_t* cfg, size_t* state_byt
 }
 
 galore_status_t galore_init_layer(const galore_config_t* cfg, void* state_buf, size_t state_bytes, void* workspace,
-                                  size_t workspace_bytes, void* stream, galore_layer_t** out) {
+                                  size_t workspace_bytes, void* stream, galore_layer_t** out) try {
   if (!out) return GALORE_ERR_INVALID_ARG;
   *out = nullptr;
   Sizes s;
@@ -589,14 +589,14 @@ galore_status_t galore_init_layer(const galore_config_t* cfg, void* state_buf, s
   }
   *out = l;
   return GALORE_OK;
-}
+} GALORE_CATCH
 
 galore_status_t galore_refresh_projector(galore_layer_t* l, const void* G, int64_t ldg, void* stream,
-                                         galore_refresh_info_t* info) {
+                                         galore_refresh_info_t* info) try {
   if (!l || !G) return GALORE_ERR_INVALID_ARG;
   if (ldg < l->cfg.n) return GALORE_ERR_INVALID_ARG;
   return do_refresh(l, G, ldg, (cudaStream_t)stream, info);
-}
+} GALORE_CATCH
 
 galore_status_t galore_refresh_query_bytes(const galore_layer_t* l, size_t* bytes) {
   if (!l || !bytes) return GALORE_ERR_INVALID_ARG;
@@ -605,7 +605,7 @@ galore_status_t galore_refresh_query_bytes(const galore_layer_t* l, size_t* byte
 }
 
 galore_status_t galore_refresh_batch(galore_layer_t* const* layers, const void* const* G, const int64_t* ldg, int32_t count,
-                                     void* workspace, size_t workspace_bytes, void* stream, galore_refresh_info_t* infos) {
+                                     void* workspace, size_t workspace_bytes, void* stream, galore_refresh_info_t* infos) try {
   if (count < 0 || (count > 0 && (!layers || !G || !ldg || !workspace))) return GALORE_ERR_INVALID_ARG;
   if ((uintptr_t)workspace & 255) return GALORE_ERR_INVALID_ARG;
   for (int i = 0; i < count; ++i) {
@@ -640,9 +640,9 @@ galore_status_t galore_refresh_batch(galore_layer_t* const* layers, const void* 
     i += n;
   }
   return warn;
-}
+} GALORE_CATCH
 
-galore_status_t galore_step(galore_layer_t* l, void* W, int64_t ldw, const void* G, int64_t ldg, float lr, void* stream) {
+galore_status_t galore_step(galore_layer_t* l, void* W, int64_t ldw, const void* G, int64_t ldg, float lr, void* stream) try {
   if (!l || !W || !G) return GALORE_ERR_INVALID_ARG;
   if (ldw < l->cfg.n || ldg < l->cfg.n) return GALORE_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
@@ -663,10 +663,10 @@ galore_status_t galore_step(galore_layer_t* l, void* W, int64_t ldw, const void*
   if (s < 0) return s;
   l->k += 1;
   return warn;
-}
+} GALORE_CATCH
 
 galore_status_t galore_step_host(galore_layer_t* l, void* W_host, const void* G_host, void* W_dev, void* G_dev, float lr,
-                                 void* stream) {
+                                 void* stream) try {
   if (!l || !W_host || !G_host || !W_dev || !G_dev) return GALORE_ERR_INVALID_ARG;
   cudaStream_t st = (cudaStream_t)stream;
   const size_t wb = (size_t)l->cfg.m * l->cfg.n * dtype_size(l->cfg.w_dtype);
@@ -677,7 +677,7 @@ galore_status_t galore_step_host(galore_layer_t* l, void* W_host, const void* G_
   if (s < 0) return s;
   GALORE_CUDA_TRY(cudaMemcpyAsync(W_host, W_dev, wb, cudaMemcpyDeviceToHost, st));
   return s;
-}
+} GALORE_CATCH
 
 // ---- pipelined step for host-resident W and G -------------------------------------------------------
 namespace {
@@ -756,7 +756,7 @@ galore_status_t galore_host_batch_query_bytes(galore_layer_t* const* layers, int
 
 galore_status_t galore_step_host_batch(galore_layer_t* const* layers, void* const* W_host, const void* const* G_host,
                                        int32_t count, float lr, void* staging, size_t staging_bytes, int32_t slots,
-                                       void* stream) {
+                                       void* stream) try {
   if (count < 0 || slots < 1 || (count > 0 && (!layers || !W_host || !G_host || !staging))) return GALORE_ERR_INVALID_ARG;
   if (count == 0) return GALORE_OK;
   if ((uintptr_t)staging & 255) return GALORE_ERR_INVALID_ARG;
@@ -824,7 +824,7 @@ galore_status_t galore_step_host_batch(galore_layer_t* const* layers, void* cons
   }
   for (int j = 0; j < std::min<int>(slots, count); ++j) GALORE_CUDA_TRY(cudaStreamWaitEvent(st, hp.drained[j], 0));
   return warn;
-}
+} GALORE_CATCH
 
 // ---- batched step --------------------------------------------------------------------------------
 namespace {
@@ -873,7 +873,7 @@ struct BatchMember {
 
 }  // namespace
 
-galore_status_t galore_batch_query_bytes(galore_layer_t* const* layers, int32_t count, size_t* bytes) {
+galore_status_t galore_batch_query_bytes(galore_layer_t* const* layers, int32_t count, size_t* bytes) try {
   if (!bytes || count < 0 || (count > 0 && !layers)) return GALORE_ERR_INVALID_ARG;
   int eligible = 0;
   for (int32_t i = 0; i < count; ++i) {
@@ -908,11 +908,11 @@ galore_status_t galore_batch_query_bytes(galore_layer_t* const* layers, int32_t 
   }
   *bytes = std::max(*bytes, best);
   return GALORE_OK;
-}
+} GALORE_CATCH
 
 galore_status_t galore_step_batch(galore_layer_t* const* layers, void* const* W, const int64_t* ldw, const void* const* G,
                                   const int64_t* ldg, int32_t count, float lr, void* batch_ws, size_t batch_ws_bytes,
-                                  void* stream) {
+                                  void* stream) try {
   if (count < 0 || (count > 0 && (!layers || !W || !ldw || !G || !ldg))) return GALORE_ERR_INVALID_ARG;
   if (batch_ws && ((uintptr_t)batch_ws & 255)) return GALORE_ERR_ALIGNMENT;
   cudaStream_t st = (cudaStream_t)stream;
@@ -1138,7 +1138,7 @@ galore_status_t galore_step_batch(galore_layer_t* const* layers, void* const* W,
     return GALORE_OK;
   }));
   return worst;
-}
+} GALORE_CATCH
 
 galore_status_t galore_free(galore_layer_t* l) {
   if (!l) return GALORE_ERR_INVALID_ARG;
@@ -1332,23 +1332,23 @@ galore_status_t galore_import_state(galore_layer_t* l, const void* src_host, siz
   return GALORE_OK;
 }
 
-galore_status_t galore_q8_codebook(int32_t is_signed, float* out256_host) {
+galore_status_t galore_q8_codebook(int32_t is_signed, float* out256_host) try {
   if (!out256_host) return GALORE_ERR_INVALID_ARG;
   q8_host_codebook(is_signed != 0, out256_host);
   return GALORE_OK;
-}
+} GALORE_CATCH
 
 galore_status_t galore_q8_quantize(const float* x, int64_t rows, int64_t cols, int32_t is_signed, int32_t tile_rows,
-                                   int32_t tile_cols, uint8_t* codes, float* absmax, void* stream) {
+                                   int32_t tile_cols, uint8_t* codes, float* absmax, void* stream) try {
   if (rows < 0 || cols < 0 || (rows > 0 && cols > 0 && (!x || !codes || !absmax))) return GALORE_ERR_INVALID_ARG;
   return launch_q8_quantize(x, rows, cols, cols, is_signed, tile_rows, tile_cols, codes, cols, absmax, (cudaStream_t)stream);
-}
+} GALORE_CATCH
 
 galore_status_t galore_q8_dequantize(const uint8_t* codes, const float* absmax, int64_t rows, int64_t cols,
-                                     int32_t is_signed, int32_t tile_rows, int32_t tile_cols, float* out, void* stream) {
+                                     int32_t is_signed, int32_t tile_rows, int32_t tile_cols, float* out, void* stream) try {
   if (rows < 0 || cols < 0 || (rows > 0 && cols > 0 && (!codes || !absmax || !out))) return GALORE_ERR_INVALID_ARG;
   return launch_q8_dequantize(codes, cols, absmax, rows, cols, is_signed, tile_rows, tile_cols, out, cols, (cudaStream_t)stream);
-}
+} GALORE_CATCH
 
 const char* galore_status_string(galore_status_t s) {
   switch (s) {
@@ -1382,7 +1382,7 @@ galore_status_t galore_profile_enable(int32_t on) {
   return GALORE_OK;
 }
 
-galore_status_t galore_profile_read(double* ms3, int64_t* count3) {
+galore_status_t galore_profile_read(double* ms3, int64_t* count3) try {
   if (!ms3 || !count3) return GALORE_ERR_INVALID_ARG;
   std::vector<PhaseEvent> evs;
   {
@@ -1405,6 +1405,6 @@ galore_status_t galore_profile_read(double* ms3, int64_t* count3) {
     cudaEventDestroy(e.b);
   }
   return rc;
-}
+} GALORE_CATCH
 
 }  // extern "C"

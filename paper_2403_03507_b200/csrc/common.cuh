@@ -7,6 +7,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <new>
+
 #include "../../include/galore.h"
 
 namespace galore {
@@ -29,6 +31,12 @@ void count_launch(int n = 1);
     galore_status_t s__ = (expr);                 \
     if (s__ < 0) return s__;                      \
   } while (0)
+
+// behind the body of an entry point that keeps lists in host memory (`... try { ... } GALORE_CATCH`): nothing throws to the caller
+#define GALORE_CATCH                  \
+  catch (const std::bad_alloc&) {     \
+    return GALORE_ERR_INVALID_ARG;    \
+  }
 
 // after a kernel launch: counts it and converts a launch failure into a status
 #define GALORE_LAUNCH_CHECK()                                   \

@@ -157,8 +157,10 @@ struct Sizes {
   size_t off_status, off_R, off_N, off_Pp, off_af, off_refresh, ws_bytes;
 };
 
-// Layers whose W and G are both fp32 keep one order of the projection's sums (gemm_fma.cu says why).
-bool fma_projection(const galore_config_t& c) { return c.w_dtype == GALORE_F32 && c.g_dtype == GALORE_F32; }
+// fp32 W and G under fp32 Adam moments keep one order of the projection's sums (gemm_fma.cu says why).
+bool fma_projection(const galore_config_t& c) {
+  return c.w_dtype == GALORE_F32 && c.g_dtype == GALORE_F32 && c.state_fmt == GALORE_STATE_F32;
+}
 
 galore_status_t resolve(const galore_config_t* c, Sizes* s) {
   if (!c || !s) return GALORE_ERR_INVALID_ARG;

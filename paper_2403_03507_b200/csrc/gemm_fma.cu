@@ -4,8 +4,8 @@
 // young, Eq. 15 is N = r / (|r| + eps), and an r that the sum over K all but cancels hands its rounding to N undamped.  An
 // fp32 W shows that: for 512 x 1376 at rank 128 two sums that differ in their last bits gave weights 8.5e-5 apart in 1 of 40
 // runs (each 1.6e-5 to 6.9e-5 from those of a product in 64 bits).  Such layers therefore keep one fixed order of their
-// sums: fmaf over k, slice after slice.  Where W or G is bf16 its rounding hides the difference, and the split products
-// carry the projection.
+// sums: fmaf over k, slice after slice.  A bf16 W or 8-bit moments round far above the difference, and Adafactor's
+// factored second moment does not vanish with a single r: there the split products carry the projection.
 //
 // What bounds it: the FMA rate of a 128 x 128 tile of 256 threads for large matrices; for small ones the latency of the K loop,
 // 16 k at a time with the next ones on their way.

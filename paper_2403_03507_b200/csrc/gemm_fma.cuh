@@ -1,4 +1,4 @@
-// Products with fp32 FMA: the projection of layers whose W and G are both fp32.  Interface.
+// Products with fp32 FMA: the projection of layers with fp32 W, G and Adam moments.  Interface.
 //
 // C(i, j) = sum_k A(i, k) * B(k, j),  A(i, k) = A[i * sAi + k * sAk],  B(k, j) = B[k * sBk + j * sBj], any leading
 // dimension and either storage order.  Every element of a K slice is one chain of fmaf in the order of k, whatever the tile.

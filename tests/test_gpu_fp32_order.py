@@ -1,4 +1,4 @@
-"""Layers with fp32 W and fp32 G: the projection is one chain of fused multiply-adds over k (slice after slice), bit for bit,
+"""Layers with fp32 W, G and Adam moments: the projection is one chain of fused multiply-adds over k (slice after slice), bit for bit,
 on every entry point, so that a run repeats what earlier releases of the library gave."""
 import pytest
 import torch

@@ -23,8 +23,7 @@ def test_strips_equal_the_regular_step(m, n, r, side):
     assert gb.galore_step_static(P, M, V, W, G, 1e-2, completed_steps=0, side=side) == 0
     layer.galore_step(W_ref, G, 1e-2)
     M_ref, V_ref = layer.get_moments()
-    # the two sum the K blocks in another order: fp32 sums of at most 4100 terms, about 2^-24 sqrt(4100) of their size
-    assert float((M - M_ref).norm() / M_ref.norm()) <= 4e-6
-    assert float((V - V_ref).norm() / V_ref.norm()) <= 8e-6
-    # N = R / |R| at the first step: only an R that rounds to the other side of zero could differ by more than rounding
-    assert float((W - W_ref).norm() / (W_ref - W0).norm()) <= 1e-3
+    # the K slices of the regular step, whatever the strips: the same bits
+    assert torch.equal(M, M_ref) and torch.equal(V, V_ref)
+    # the same N through other tiles of the update: fp32 sums of at most 1000 terms
+    assert float((W - W_ref).norm() / (W_ref - W0).norm()) <= 4e-6

@@ -15,6 +15,7 @@
 
 #include <algorithm>
 
+#include "gemm_dmma.cuh"
 #include "launch.cuh"
 
 namespace galore {
@@ -31,14 +32,6 @@ constexpr int kGramLd = 36;       // shared-memory row strides, all = 4 mod 16 d
 constexpr int kRotLd = 68;        // fragments of the fp64 MMA then fall on distinct banks
 constexpr int kApplyHalf = 64;    // columns in shared memory at a time
 constexpr int kHalfLd = 68;
-
-// D (8 x 8) += A (8 x 4, row) B (4 x 8, col), fp64.  Lane l holds A[l / 4][l % 4], B[l % 4][l / 4]
-// and D[l / 4][2 (l % 4) + {0, 1}].
-__device__ __forceinline__ void dmma(double (&d)[2], double a, double b) {
-  asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};\n"
-               : "+d"(d[0]), "+d"(d[1])
-               : "d"(a), "d"(b));
-}
 
 // Round-robin tournament of n players (n even): in `round`, position k meets position n - 1 - k.
 __host__ __device__ __forceinline__ int rr_player(int pos, int round, int n) {
@@ -138,7 +131,7 @@ __global__ void __launch_bounds__(128) jb_gram_kernel(const double* X, int b, in
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int j = i; j < 4; ++j) dmma(acc[i][j], a[i], bb[j]);
+          for (int j = i; j < 4; ++j) dmma_m8n8k4(acc[i][j], a[i], bb[j]);
       }
     } else {                   // two of the four tile columns of the off-diagonal quadrant (kept in acc[.][0..1])
 #pragma unroll
@@ -151,7 +144,7 @@ __global__ void __launch_bounds__(128) jb_gram_kernel(const double* X, int b, in
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
-          for (int j = 0; j < 2; ++j) dmma(acc[i][j], a[i], bb[j]);
+          for (int j = 0; j < 2; ++j) dmma_m8n8k4(acc[i][j], a[i], bb[j]);
       }
     }
     if (tile + 1 < tiles) stash(buf ^ 1);
@@ -558,7 +551,7 @@ __global__ void __launch_bounds__(256) jb_apply_kernel(double* __restrict__ X, d
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) dmma(acc[i][j], a[i], bb[j]);
+        for (int j = 0; j < 2; ++j) dmma_m8n8k4(acc[i][j], a[i], bb[j]);
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) {

@@ -1,18 +1,18 @@
 // Products with fp32 operands (or bf16 operands whose rows TMA cannot address) on the 5th-generation
 // tensor cores.
 //
-// x = hi + mid + lo with three bf16 numbers holds every fp32 value exactly (24 significand bits), so
+// x = hi + mid + lo with three bf16 numbers holds an fp32 value exactly (24 significand bits; gemm_split.cuh has the range), so
 //   a b = ah bh + (ah bm + am bh) + (ah bl + am bm + al bh) + O(2^-26) |a b|
 // and six tcgen05 products of bf16 operands replace one fp32 product (three when one operand is bf16
 // already, one when both are).  The dropped terms lie below fp32's own rounding of a product.
 //
 // Accumulation: the leading products go to one TMEM accumulator, all smaller ones to a second, and
-// after every few k-blocks both are added to an fp32 sum in the epilogue warps' registers.  The
+// after every k-block (kChunk) both are added to an fp32 sum in the epilogue warps' registers.  The
 // tensor core's accumulator rounds towards zero: the short chains keep that below the rounding of an
 // ordinary fp32 sum.
 //
 // Measured (eight layers of the LLaMA-130M set, rank 256, fp32 gradients): projections 1292 -> 247 us against fp32 FMA
-// kernels; a bf16 2048 x 5461 matrix of unpadded rows at rank 512: 766 -> 85 us.  What bounds it: the conversion
+// kernels; a bf16 2048 x 5461 matrix of unpadded rows at rank 512: 766 -> 74 us.  What bounds it: the conversion
 // of the operands (about twelve instructions per element, each element of a tile once) and the latency of the one
 // stage of loads the producers hold in registers.
 //

@@ -2,7 +2,9 @@
 //
 // C(i, j) = sum_k A(i, k) * B(k, j) for fp32 or bf16 operands of any leading dimension and either
 // storage order.  An fp32 operand is carried as three bf16 numbers (8 + 8 + 8 significand bits: the
-// value itself, nothing is lost), a bf16 operand as itself, so the products keep fp32's precision.
+// value itself, nothing is lost), a bf16 operand as itself, so the products keep fp32's precision.  That
+// holds for 2^-110 <= |x| <= 3.39e38, the largest bf16: below, the last number loses bits; a larger value
+// enters as an infinity, and the step reports it as non-finite.
 #pragma once
 
 #include "common.cuh"

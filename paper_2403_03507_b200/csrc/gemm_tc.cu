@@ -972,7 +972,6 @@ TensorGroup* tensor_group_new() {
 }
 void tensor_group_free(TensorGroup* t) { delete t; }
 void tensor_group_reset(TensorGroup* t) { t->g.count = 0; }
-int tensor_group_count(const TensorGroup* t) { return t->g.count; }
 int tensor_group_capacity() { return kMaxGroup; }
 
 galore_status_t tensor_group_add_project(TensorGroup* t, const TensorPlan* plan, const galore_config_t& c, bool left,

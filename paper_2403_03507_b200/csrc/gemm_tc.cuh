@@ -17,7 +17,7 @@ struct TcAdamArgs {
   int32_t state_fmt;          // galore_state_fmt_t
   float *M, *V;               // fp32 moments (rows of ld_s floats), or
   uint8_t *Mc, *Vc;           // 8-bit codes (rows of ld_s bytes) with
-  float *Mam, *Vam;           // one absmax per tile of q_block / 128 rows x 128 columns
+  float *Mam, *Vam;           // one absmax per tile of q_block / 64 rows x 64 columns
   int64_t ld_s;
   int q_block;
   void* Nout;                 // bf16, leading dimension ld_n
@@ -46,7 +46,6 @@ struct TensorGroup;   // opaque, host memory
 TensorGroup* tensor_group_new();
 void tensor_group_free(TensorGroup* t);
 void tensor_group_reset(TensorGroup* t);
-int tensor_group_count(const TensorGroup* t);
 int tensor_group_capacity();
 // the layer's projection with its R partials going to `part` (leading dimension ld_part, `splits` K slices)
 galore_status_t tensor_group_add_project(TensorGroup* t, const TensorPlan* plan, const galore_config_t& cfg, bool left,

@@ -1,5 +1,5 @@
-// fp32 matrices as three bf16 planes: hi + mid + lo holds every fp32 value exactly (8 + 8 + 8 significand
-// bits).  The planes lie below one another, as operands of the weight update (gemm_apply.cuh).
+// fp32 matrices as three bf16 planes: hi + mid + lo holds an fp32 value exactly (8 + 8 + 8 significand
+// bits; for 2^-110 <= |x| <= 3.39e38).  The planes lie below one another, as operands of the weight update (gemm_apply.cuh).
 #pragma once
 
 #include "common.cuh"

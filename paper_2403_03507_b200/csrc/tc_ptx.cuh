@@ -1,5 +1,5 @@
 // Thin wrappers of the PTX the tensor-core kernels are written with: mbarriers with bounded waits, TMA loads,
-// tensor memory, tcgen05.mma, 32-byte global accesses.
+// tensor memory, tcgen05.mma, 32-byte global stores.
 #pragma once
 
 #include <cuda.h>
@@ -182,14 +182,8 @@ __device__ __forceinline__ void tmem_ld_32x32(uint32_t taddr, uint32_t (&v)[32])
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// 32-byte global accesses: one request covers a whole 32-byte sector, so a thread that walks its own
+// 32-byte global stores: one request covers a whole 32-byte sector, so a thread that walks its own
 // row does not send half-filled sectors through the L1/L2 fabric.  Address must be 32-byte aligned.
-__device__ __forceinline__ void ld_global_32B(const void* ptr, uint4& a, uint4& b) {
-  asm volatile("ld.global.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
-               : "l"(ptr)
-               : "memory");
-}
 __device__ __forceinline__ void st_global_32B(void* ptr, const uint4& a, const uint4& b) {
   asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};"
                ::"l"(ptr), "r"(a.x), "r"(a.y), "r"(a.z), "r"(a.w), "r"(b.x), "r"(b.y), "r"(b.z), "r"(b.w)

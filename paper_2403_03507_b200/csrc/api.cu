@@ -206,7 +206,7 @@ galore_status_t resolve(const galore_config_t* c, Sizes* s) {
   s->block = (int)std::min<int64_t>(s->d, (int64_t)r + over);
 
   // K slices of the projection
-  s->proj_splits = fma_projection(*c) ? fma_choose_slices(s->srows, s->scols, s->d) : split_choose_slices(s->srows, s->scols, s->d);
+  s->proj_splits = fma_projection(*c) ? fma_choose_slices(s->srows, s->scols, s->d) : split_choose_slices(s->srows, s->scols, s->d, c->p_dtype == GALORE_F32 && c->g_dtype == GALORE_F32);
   s->tc_splits = s->tensor_path ? tensor_proj_splits(*c, s->left) : 0;
   s->ld_part = (s->scols + 7) / 8 * 8;     // 32-byte rows for whole-sector vector stores
   s->ld_n = (s->scols + 15) / 16 * 16;     // 32-byte bf16 rows: TMA needs 16, the epilogue that writes N stores 32 at a time
@@ -298,7 +298,7 @@ galore_status_t launch_projections(const ProjectJob* jobs, int count, bool early
       GALORE_TRY(split_group_add_store(g, (int)c.m, c.rank, (int)c.n, split_operand(j.G, c.g_dtype, j.ldg, 1),
                                        split_operand(l->P, c.p_dtype, 1, c.rank), j.splits, j.part, l->ld_part, stride, l->status));
   }
-  return launch_split_store(g, a_dtype, b_dtype, early, st);
+  return launch_split_store(g, a_dtype, b_dtype, true, early, st);
 }
 // W <- keep W - scale P N (left) resp. N Q^T: N in n_planes bf16 planes, P where it lies or in the planes at `pp`
 ApplyItem apply_item(const galore_layer* l, const __nv_bfloat16* N, int n_planes, const __nv_bfloat16* pp, void* W, int64_t ldw, float lr) {
@@ -944,7 +944,9 @@ galore_status_t galore_step_batch(galore_layer_t* const* layers, void* const* W,
   // The groups run one after another on the caller's stream, each in the whole batch workspace.
   const size_t room = batch_ws_bytes & ~(size_t)255;
   std::vector<std::vector<BatchMember>> groups, fgroups;
-  const int fcap = std::min((int)kSplitGroup, std::min((int)kAdamGroup, (int)kAdafactorGroup));
+  // groups of equal size: 56 layers as 28 + 28 rather than 32 + 24 (LLaMA-130M set: the last wave of each launch is the fuller one)
+  int fcap = std::min((int)kSplitGroup, std::min((int)kAdamGroup, (int)kAdafactorGroup));
+  fcap = (int)ceil_div(std::max(1, groupable), ceil_div(std::max(1, groupable), fcap));
   {
     size_t used = 0;
     std::vector<size_t> fused_bytes_of;

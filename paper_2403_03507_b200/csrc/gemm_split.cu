@@ -29,14 +29,13 @@
 
 #include "gemm_tc.cuh"
 #include "launch.cuh"
-#include "tc_ptx.cuh"
+#include "split_tiles.cuh"
 
 namespace galore {
 
 namespace {
 
-constexpr int kM = 128, kN = 128, kK = 64;
-constexpr int kTileBytes = 128 * kK * 2;                 // one bf16 tile of either operand
+constexpr int kM = 128, kN = 128;
 constexpr int kEpiWarps = 8, kProducerWarps = 16;
 constexpr int kProducers = 32 * kProducerWarps;
 constexpr int kMmaWarp = kEpiWarps + kProducerWarps;
@@ -48,50 +47,12 @@ static_assert(kEpiWarps == 8 && kProducerWarps == 16 && 2 * kEpiRegs + 4 * kProd
 static_assert(kEpiRegs >= kLaunchRegs && kProducerRegs <= kLaunchRegs && kMmaRegs <= kLaunchRegs,
               "setmaxnreg.inc only goes up, .dec only down: the other direction is an illegal instruction");
 constexpr int kTiles = 12;                               // bf16 tiles in shared memory: stages x splits
-constexpr int kStageLd = 33;                             // epilogue transposition: 32 x 32 floats per warp
 constexpr int kSmemBytes = kTiles * kTileBytes + kEpiWarps * 32 * kStageLd * 4 + 1024 + 256;
 constexpr int kChunk = 1;                                // k-blocks per accumulator
 constexpr uint32_t kTmem = 512;                          // two buffers x (leading, corrections) x 128 columns
 
 template <typename T>
 constexpr int splits_of() { return sizeof(T) == 4 ? 3 : 1; }
-
-// K-major and MN-major tiles as in the bf16 kernels: 128-byte swizzle, 8-row groups 1024 bytes apart; MN-major
-// operands continue kK * 128 bytes further on after 64 elements of M / N.
-__device__ __forceinline__ uint64_t split_desc(uint32_t addr, bool mn) {
-  const uint64_t lbo = mn ? (uint64_t)((kK * 128) >> 4) : 1ull;
-  return (uint64_t)((addr & 0x3FFFFu) >> 4) | (lbo << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) | (2ull << 61);
-}
-__device__ __forceinline__ uint32_t split_idesc(int a_mn, int b_mn) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((a_mn ? 1u : 0u) << 15) | ((b_mn ? 1u : 0u) << 16) | ((uint32_t)(kN >> 3) << 17) |
-         ((uint32_t)(kM >> 4) << 24);
-}
-
-struct SplitUnit {
-  int pi, m0, n0, slice, kb, kb_end;
-};
-template <int CAP>
-__device__ __forceinline__ SplitUnit split_unit(const SplitArgs<CAP>& g, int u, GroupCursor& cursor) {
-  SplitUnit w;
-  u = cursor.seek<CAP>(g, u);
-  w.pi = cursor.pi;
-  const SplitProblem& p = g.p[w.pi];
-  int tm, tn;
-  if (p.m_fast) {
-    tm = u % p.tiles_m;
-    w.slice = (u / p.tiles_m) % p.splits;
-    tn = u / (p.tiles_m * p.splits);
-  } else {
-    tn = u % p.tiles_n;
-    w.slice = (u / p.tiles_n) % p.splits;
-    tm = u / (p.tiles_n * p.splits);
-  }
-  w.m0 = tm * kM;
-  w.n0 = tn * kN;
-  w.kb = w.slice * p.kblocks_per_split;
-  w.kb_end = min(p.kblocks, w.kb + p.kblocks_per_split);
-  return w;
-}
 
 // ---- producer ------------------------------------------------------------------------------------
 // A stage's tile of an operand is 1024 chunks of 8 elements along the contiguous direction; a thread
@@ -108,7 +69,7 @@ __device__ __forceinline__ ChunkPos chunk_pos(int tid, bool mn) {
     c.outer = tid >> 4;
     c.fast = ch * 8;
     c.step = kProducers / 16;
-    c.smem = (uint32_t)((ch >> 3) * (kK * 128) + c.outer * 128 + (((ch & 7) ^ (c.outer & 7)) << 4));
+    c.smem = (uint32_t)((ch >> 3) * (kSplitK * 128) + c.outer * 128 + (((ch & 7) ^ (c.outer & 7)) << 4));
   } else {
     const int ch = tid & 7;
     c.outer = tid >> 3;
@@ -171,11 +132,6 @@ __device__ __forceinline__ void load_chunk(uint32_t (&raw)[8], const char* ptr, 
 __device__ __forceinline__ void st_shared_16B(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
-__device__ __forceinline__ uint32_t pack_bf16(float x0, float x1) {
-  const __nv_bfloat162 h = __floats2bfloat162_rn(x0, x1);
-  return *reinterpret_cast<const uint32_t*>(&h);
-}
-
 // chunk -> its bf16 tiles, kTileBytes apart.  shift: byte offset of the chunk inside its first aligned vector (bf16)
 template <typename T>
 __device__ __forceinline__ void store_chunk(uint32_t dst, const uint32_t (&raw)[8], uint32_t shift) {
@@ -219,11 +175,6 @@ __device__ __forceinline__ ChunkSrc chunk_src(const SplitOperand& op, const Chun
   s.valid = (op.mn ? mn_size : k_size) - f0;
   return s;
 }
-
-template <int R>
-__device__ __forceinline__ void regs_up() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R)); }
-template <int R>
-__device__ __forceinline__ void regs_down() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R)); }
 
 // ---- the kernel ------------------------------------------------------------------------------------
 
@@ -281,13 +232,13 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
     int u = blockIdx.x;
     if (u < total_units) {
       GroupCursor cursor;
-      SplitUnit w = split_unit(g, u, cursor);
+      SplitUnit w = split_unit<kM>(g, u, cursor);
       uint32_t ra[kChunksEach][8], rb[kChunksEach][8];
       ChunkPos ca = chunk_pos(tid, g.p[w.pi].a.mn != 0), cb = chunk_pos(tid, g.p[w.pi].b.mn != 0);
       // shifts of the chunks in the registers (bf16 operands off the 16-byte boundaries)
       uint32_t sha = 0u, sha_step = 0u, shb = 0u, shb_step = 0u;
-      auto src_a = [&]() { return chunk_src<TA>(g.p[w.pi].a, ca, w.m0, w.kb * kK, g.p[w.pi].M, g.p[w.pi].K); };
-      auto src_b = [&]() { return chunk_src<TB>(g.p[w.pi].b, cb, w.n0, w.kb * kK, g.p[w.pi].N, g.p[w.pi].K); };
+      auto src_a = [&]() { return chunk_src<TA>(g.p[w.pi].a, ca, w.m0, w.kb * kSplitK, g.p[w.pi].M, g.p[w.pi].K); };
+      auto src_b = [&]() { return chunk_src<TB>(g.p[w.pi].b, cb, w.n0, w.kb * kSplitK, g.p[w.pi].N, g.p[w.pi].K); };
       auto fetch = [&]<typename T>(T, uint32_t (&raw)[8], const ChunkSrc& s, int i, int step, bool aligned) {
         load_chunk<T>(raw, s.ptr + i * s.step, i * step < s.rows ? s.valid : 0, aligned);
       };
@@ -319,7 +270,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
           u += gridDim.x;
           more = u < total_units;
           if (more) {
-            w = split_unit(g, u, cursor);
+            w = split_unit<kM>(g, u, cursor);
             ca = chunk_pos(tid, g.p[w.pi].a.mn != 0);
             cb = chunk_pos(tid, g.p[w.pi].b.mn != 0);
           }
@@ -361,9 +312,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
       bool ok = true;
       GroupCursor cursor;
       for (int u = blockIdx.x; u < total_units && ok; u += gridDim.x) {
-        const SplitUnit w = split_unit(g, u, cursor);
+        const SplitUnit w = split_unit<kM>(g, u, cursor);
         const bool a_mn = g.p[w.pi].a.mn != 0, b_mn = g.p[w.pi].b.mn != 0;
-        const uint32_t idesc = split_idesc(a_mn, b_mn);
+        const uint32_t idesc = split_idesc(a_mn, b_mn, kM, kN);
         for (int kb = w.kb; kb < w.kb_end && ok;) {
           if (!mbar_wait(acce_bar(acc), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
           tc_fence_after();
@@ -375,7 +326,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
             tc_fence_after();
             const uint32_t a_addr = ring + (uint32_t)(stage * kStageBytes), b_addr = a_addr + SA * kTileBytes;
 #pragma unroll
-            for (int k = 0; k < kK / 16; ++k) {
+            for (int k = 0; k < kSplitK / 16; ++k) {
               const uint64_t a_adv = (uint64_t)((a_mn ? k * 2048 : k * 32) >> 4), b_adv = (uint64_t)((b_mn ? k * 2048 : k * 32) >> 4);
 #pragma unroll
               for (int i = 0; i < SA; ++i)
@@ -411,7 +362,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_kernel(const __grid_co
     bool ok = true;
     GroupCursor cursor;
     for (int u = blockIdx.x; u < total_units && ok; u += gridDim.x) {
-      const SplitUnit w = split_unit(g, u, cursor);
+      const SplitUnit w = split_unit<kM>(g, u, cursor);
       const SplitProblem& p = g.p[w.pi];
       float sum[64];
 #pragma unroll
@@ -513,7 +464,7 @@ galore_status_t add_problem(SplitGroup& g, SplitProblem& p, int splits) {
   if (p.M <= 0 || p.N <= 0 || p.K <= 0) return GALORE_ERR_SHAPE;
   p.tiles_m = (int)ceil_div(p.M, kM);
   p.tiles_n = (int)ceil_div(p.N, kN);
-  p.kblocks = (int)ceil_div(p.K, kK);
+  p.kblocks = (int)ceil_div(p.K, kSplitK);
   p.kblocks_per_split = (int)ceil_div(p.kblocks, std::max(1, splits));
   p.splits = (int)ceil_div(p.kblocks, p.kblocks_per_split);
   p.m_fast = p.tiles_m <= p.tiles_n ? 1 : 0;         // neighbours share the panel of the larger operand
@@ -537,23 +488,32 @@ SplitOperand split_operand(const void* base, int32_t dtype, int64_t s_mn, int64_
 }
 
 int split_effective_slices(int64_t K, int slices) {
-  const int64_t kb = ceil_div(K, kK);
+  const int64_t kb = ceil_div(K, kSplitK);
   return (int)ceil_div(kb, ceil_div(kb, std::max(1, slices)));
 }
 
-// Time of a launch = waves x (k-blocks of a unit x time of a k-block + fixed time of a unit), plus reading back the partial
-// results.  Measured: 512 x 5461 x 2048 of unaligned bf16 in 1 to 5 slices 115 / 86 / 77 / 74 / 73 us, 128 x 1376 x 512 of
-// fp32 in 1, 2, 4: 19.9 / 12.9 / 9.5 us, both 1.75 us a k-block (the producers' loads, whatever the number of planes); the Adam
-// kernel behind them reads a slice at 4.8 TB/s.  (With 0.6 us a k-block for bf16 the first was cut in two: 153 us a step
-// instead of 146.)
-int split_choose_slices(int64_t M, int64_t N, int64_t K) {
-  const int64_t tiles = ceil_div(M, kM) * ceil_div(N, kN), kb = ceil_div(K, kK);
+namespace {
+// Microseconds of `units` work units of kb k-blocks: waves x (k-blocks x time of a k-block + fixed time of a unit).  A k-block
+// of 128 x 128 on one SM takes 1.75 us (the producers' loads, whatever the number of planes: 512 x 5461 x 2048 of unaligned bf16
+// in 1 to 5 slices 115 / 86 / 77 / 74 / 73 us, 128 x 1376 x 512 of fp32 in 1, 2, 4: 19.9 / 12.9 / 9.5 us).  A pair's, of 256 x 256,
+// takes 2.85 us (256 x 4096 x K in groups of 144 tiles: 65.7 us at K = 512, 378 at 4096).
+double split_us(int64_t units, int64_t kb, bool pair) {
+  return (double)ceil_div(units, pair ? 74 : 148) * (pair ? (double)kb * 2.85 + 2.5 : (double)kb * 1.75 + 0.6);
+}
+int64_t split_units(int64_t M, int64_t N, int64_t slices, int tile) { return ceil_div(M, tile) * ceil_div(N, tile) * slices; }
+}  // namespace
+
+// The time of the launch plus that of reading back the partial results: the Adam kernel behind it reads a slice at 4.8 TB/s.
+// (With 0.6 us a k-block for bf16 512 x 5461 x 2048 was cut in two: 153 us a step instead of 146.)
+int split_choose_slices(int64_t M, int64_t N, int64_t K, bool pairs) {
+  const int64_t kb = ceil_div(K, kSplitK);
   int best = 1;
   double best_us = 1e30;
   for (int s = 1; s <= 16; ++s) {
     if (split_effective_slices(K, s) != s) continue;
-    const double waves = (double)ceil_div(tiles * s, 148);
-    const double us = waves * ((double)ceil_div(kb, s) * 1.75 + 0.6) + s * (0.35 + (double)(M * N) * 4.0 / 4.8e6);
+    double us = split_us(split_units(M, N, s, 128), ceil_div(kb, s), false);
+    if (pairs) us = std::min(us, split_us(split_units(M, N, s, 256), ceil_div(kb, s), true));
+    us += s * (0.35 + (double)(M * N) * 4.0 / 4.8e6);
     if (us < best_us) {
       best_us = us;
       best = s;
@@ -572,11 +532,22 @@ galore_status_t split_group_add_store(SplitGroup& g, int M, int N, int K, const 
   return add_problem(g, p, splits);
 }
 
-galore_status_t launch_split_store(const SplitGroup& g, int32_t a_dtype, int32_t b_dtype, bool early, cudaStream_t st) {
+galore_status_t launch_split_store(const SplitGroup& g, int32_t a_dtype, int32_t b_dtype, bool pairs, bool early, cudaStream_t st) {
   const bool ab = a_dtype == GALORE_BF16, bb = b_dtype == GALORE_BF16;
   if (ab && bb) return launch_split<__nv_bfloat16, __nv_bfloat16>(g, early, st);
   if (ab) return launch_split<__nv_bfloat16, float>(g, early, st);
   if (bb) return launch_split<float, __nv_bfloat16>(g, early, st);
+  if (pairs) {
+    int64_t single = 0, pair = 0, kb = 0;
+    for (int i = 0; i < g.count && pairs; ++i) {
+      const SplitProblem& p = g.p[i];
+      pairs = p.a.aligned && p.b.aligned;
+      single += split_units(p.M, p.N, p.splits, 128);
+      pair += split_units(p.M, p.N, p.splits, 256);
+      kb = std::max<int64_t>(kb, p.kblocks_per_split);
+    }
+    if (pairs && split_us(pair, kb, true) < split_us(single, kb, false)) return launch_split_pair(g, early, st);
+  }
   return launch_split<float, float>(g, early, st);
 }
 

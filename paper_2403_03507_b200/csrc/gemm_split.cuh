@@ -32,6 +32,7 @@ struct SplitProblem {
 };
 template <int CAP>
 struct SplitArgs {
+  static constexpr int kCapacity = CAP;
   SplitProblem p[CAP];
   int unit_end[CAP];
   int count;
@@ -40,12 +41,15 @@ using SplitGroup = SplitArgs<kSplitGroup>;
 
 // operand X(i, k) = base[i * s_mn + k * s_k]; one of the strides is 1
 SplitOperand split_operand(const void* base, int32_t dtype, int64_t s_mn, int64_t s_k);
-// K slices that balance filling the machine against the traffic of the partial results
-int split_choose_slices(int64_t M, int64_t N, int64_t K);
+// K slices that balance filling the machine against the traffic of the partial results; pairs: see launch_split_store
+int split_choose_slices(int64_t M, int64_t N, int64_t K, bool pairs);
 int split_effective_slices(int64_t K, int slices);
 galore_status_t split_group_add_store(SplitGroup& g, int M, int N, int K, const SplitOperand& a, const SplitOperand& b, int splits,
                                       float* C, int64_t ldc, int64_t split_stride, int32_t* status);
-// all problems of a group share the operand types
-galore_status_t launch_split_store(const SplitGroup& g, int32_t a_dtype, int32_t b_dtype, bool early, cudaStream_t st);
+// All problems of a group share the operand types.  pairs: fp32 operands may take the tiles of CTA pairs, where the group's
+// size makes them the faster ones (their sums round differently); false: a problem's bits do not depend on its group.
+galore_status_t launch_split_store(const SplitGroup& g, int32_t a_dtype, int32_t b_dtype, bool pairs, bool early, cudaStream_t st);
+// the same for fp32 operands on 16-byte boundaries, by CTA pairs (gemm_split_pair.cu)
+galore_status_t launch_split_pair(const SplitGroup& g, bool early, cudaStream_t st);
 
 }  // namespace galore

@@ -729,7 +729,7 @@ galore_status_t ensure_encode() {
 }  // namespace
 
 galore_status_t tensor_encode(CUtensorMap* map, const void* base, int32_t dtype, int64_t rows, int64_t cols, int64_t ld,
-                              int box_rows, int box_cols) {
+                              int box_rows, int box_cols, bool swizzle) {
   GALORE_TRY(ensure_encode());
   const int64_t es = (int64_t)dtype_size(dtype);
   if (((uintptr_t)base & 15) || (ld * es) % 16) return GALORE_ERR_ALIGNMENT;
@@ -739,7 +739,8 @@ galore_status_t tensor_encode(CUtensorMap* map, const void* base, int32_t dtype,
   cuuint32_t estr[2] = {1u, 1u};
   CUresult r = g_encode.load(std::memory_order_relaxed)(
       map, dtype == GALORE_BF16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 2, const_cast<void*>(base), dims,
-      strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+      strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+      CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
       CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) {
     note_cuda_error(cudaErrorInvalidValue, "cuTensorMapEncodeTiled");

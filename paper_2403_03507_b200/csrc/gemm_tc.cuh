@@ -82,8 +82,8 @@ galore_status_t tensor_launch_in_order(cudaStream_t st, F&& launch) {
   return launch_order().run(dev, st, std::forward<F>(launch));
 }
 int tensor_sm_count();
-// a matrix of rows x cols elements (cols contiguous) with boxes of box_rows x box_cols, 128-byte swizzle
+// a matrix of rows x cols elements (cols contiguous) with boxes of box_rows x box_cols, 128-byte swizzle or none
 galore_status_t tensor_encode(CUtensorMap* map, const void* base, int32_t dtype, int64_t rows, int64_t cols, int64_t ld,
-                              int box_rows, int box_cols);
+                              int box_rows, int box_cols, bool swizzle = true);
 
 }  // namespace galore

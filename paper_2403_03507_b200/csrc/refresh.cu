@@ -729,7 +729,7 @@ static galore_status_t split_products(const Ctx& c, std::vector<SliceTarget>& ts
         GALORE_TRY(split_group_add_store(g, M, N, std::min(per, K - k * per), a, b, 1, t.out.x[k], ldc, 0, t.l->status));
       }
     }
-    GALORE_TRY(tensor_launch_in_order(c.st, [&]() { return launch_split_store(g, a_dtype, b_dtype, true, c.st); }));
+    GALORE_TRY(tensor_launch_in_order(c.st, [&]() { return launch_split_store(g, a_dtype, b_dtype, false, true, c.st); }));
   }
   return GALORE_OK;
 }

@@ -48,3 +48,31 @@ def test_products_of_split_operands_are_fp32_products(m, n, r, g, w, pad):
     assert float((W.double() - W0 - dW).abs().max()) <= slack + 1e-5 * float(dW.abs().max()) + 1e-12
     if pad:
         assert torch.isnan(W._base[:, n:]).all()
+
+
+# groups that fill the machine with the 256 x 256 tiles of CTA pairs: ragged tiles on both sides, blocks of K cut off, several K
+# slices (one matrix), rows padded to 16 bytes; the largest rank takes two tiles along the rank
+@pytest.mark.parametrize("m,n,r,count,pad", [(769, 2052, 256, 12, 0), (2052, 770, 260, 12, 2), (96, 8200, 64, 20, 0), (1000, 1999, 388, 8, 1), (2048, 5460, 512, 1, 0),
+                                             (5460, 2050, 512, 1, 2)])
+def test_products_of_large_groups_are_fp32_products(m, n, r, count, pad):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(m * 7919 + n)
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda")
+    layers, Ws, Gs = [], [], []
+    for _ in range(count):
+        layers.append(gb.Layer(gb.make_config(m, n, r, w_dtype="bf16", g_dtype="f32", auto_refresh=False)))
+        layers[-1].set_projector(torch.linalg.qr(rand(layers[-1].proj_rows, r))[0])
+        Ws.append(_matrix(0.02 * rand(m, n), "bf16", pad))
+        Gs.append(_matrix(rand(m, n), "f32", pad))
+    if count == 1:
+        layers[0].galore_step(Ws[0], Gs[0], 1e-2)
+    else:
+        gb.Batch(layers, Ws, Gs).galore_step_batch(1e-2)
+    for layer, G in zip(layers, Gs):
+        assert layer.device_status() == 0
+        P = layer.get_projector().double()
+        R = P.T @ G.double() if layer.side == gb.SIDE_LEFT else G.double() @ P
+        M = layer.get_moments()[0].double()
+        # as above: an fp32 sum of K terms; the accumulators of 32 of K lose at most a unit of 2^-23 of one sign per 16 products
+        assert float((M / 0.1 - R).norm() / R.norm()) <= 2 ** -24 * (8 + (m if layer.side == gb.SIDE_LEFT else n) ** 0.5)
+        assert abs(float((M / 0.1 * R).sum() / (R * R).sum()) - 1) <= 2e-7

@@ -20,6 +20,7 @@
 #include "gemm_fma.cuh"
 #include "gemm_split.cuh"
 #include "gemm_tc.cuh"
+#include "launch.cuh"
 #include "refresh.cuh"
 
 namespace galore {
@@ -103,6 +104,63 @@ galore_status_t launch_repitch(const Repitch& r, cudaStream_t st) {
   return GALORE_OK;
 }
 
+// bf16 rows off the 16-byte boundaries -> rows on them, for TMA.  A warp takes 1024 columns of a row; a lane moves eight elements
+// at a time: the two aligned vectors that hold them (each contains at least one: nothing outside the allocation's
+// granules is read), shifted into one.
+__global__ void __launch_bounds__(256) align_rows_kernel(const __nv_bfloat16* src, int64_t ld_src, __nv_bfloat16* __restrict__ dst, int64_t ld_dst,
+                                                         int rows, int cols) {
+  grid_dependency_wait();
+  grid_launch_dependents();
+  constexpr int U = 4;
+  const int parts = (cols + 256 * U - 1) / (256 * U), units = rows * parts;
+  for (int unit = (int)(blockIdx.x * 8 + (threadIdx.x >> 5)); unit < units; unit += (int)gridDim.x * 8) {
+    const int row = unit / parts, c0 = (unit - row * parts) * (256 * U) + (int)(threadIdx.x & 31) * 8;
+    uint4 a[U], b[U];
+    uint32_t shift[U];
+    __nv_bfloat16* out[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int c = c0 + 256 * u;
+      out[u] = nullptr;
+      if (c >= cols) continue;
+      const __nv_bfloat16* s = src + (int64_t)row * ld_src + c;
+      out[u] = dst + (int64_t)row * ld_dst + c;
+      if (c + 8 <= cols) {
+        const uintptr_t at = (uintptr_t)s & ~(uintptr_t)15;
+        shift[u] = (uint32_t)((uintptr_t)s & 15);
+        a[u] = *reinterpret_cast<const uint4*>(at);
+        b[u] = shift[u] ? *reinterpret_cast<const uint4*>(at + 16) : a[u];
+      } else {                                            // the end of a row
+        uint32_t v[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if (c + j < cols) v[j >> 1] |= (uint32_t)reinterpret_cast<const uint16_t*>(s)[j] << (16 * (j & 1));
+        shift[u] = 0u;
+        a[u] = b[u] = make_uint4(v[0], v[1], v[2], v[3]);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (!out[u]) continue;
+      const uint32_t raw[8] = {a[u].x, a[u].y, a[u].z, a[u].w, b[u].x, b[u].y, b[u].z, b[u].w};
+      uint32_t w[6], v[5];
+#pragma unroll
+      for (int j = 0; j < 6; ++j) w[j] = (shift[u] & 8u) ? raw[j + 2] : raw[j];
+#pragma unroll
+      for (int j = 0; j < 5; ++j) v[j] = (shift[u] & 4u) ? w[j + 1] : w[j];
+      const uint32_t bits = (shift[u] & 2u) * 8u;
+      *reinterpret_cast<uint4*>(out[u]) = make_uint4(__funnelshift_r(v[0], v[1], bits), __funnelshift_r(v[1], v[2], bits),
+                                                     __funnelshift_r(v[2], v[3], bits), __funnelshift_r(v[3], v[4], bits));
+    }
+  }
+}
+galore_status_t launch_align_rows(const void* src, int64_t ld_src, void* dst, int64_t ld_dst, int rows, int cols, cudaStream_t st) {
+  const int64_t units = (int64_t)rows * ceil_div(cols, 1024);
+  if (units >= ((int64_t)1 << 30)) return GALORE_ERR_SHAPE;
+  return launch_kernel(align_rows_kernel, dim3((unsigned)std::min<int64_t>(ceil_div(units, 8), 148 * 8)), 256, 0, 1, true, st,
+                       (const __nv_bfloat16*)src, ld_src, (__nv_bfloat16*)dst, ld_dst, rows, cols);
+}
+
 }  // namespace galore
 
 using namespace galore;
@@ -120,7 +178,8 @@ struct galore_layer {
   int64_t nblk;
   int block;             // columns of the refresh block
   int proj_splits;       // K slices of the projection on the fp32 path
-  int tc_splits;         // K slices of the projection on the tensor-core path
+  int tc_splits;         // K slices of the projection on the tensor-core path, in a batch of few layers
+  int step_splits;       // the same in a step of its own
   int64_t ld_part, ld_n; // padded row pitches of the R partials and of N
   int p_planes;          // bf16 planes the projector is split into for the weight update, 0: it is used where it lies
   int64_t ld_p;          // their row pitch
@@ -137,6 +196,7 @@ struct galore_layer {
   float* Rpart;
   __nv_bfloat16* Nbuf;
   __nv_bfloat16* Pplanes;
+  __nv_bfloat16* Gcopy;  // G in rows on 16-byte boundaries, where its own may lie off them; null: there is no place
   void* refresh_ws;
   size_t state_bytes;    // size of the caller's state buffer as laid out here (it starts at P)
   bool refreshed_here = false;   // the last refresh ran in refresh_ws (its unrounded projector is still there)
@@ -148,14 +208,17 @@ namespace {
 struct Sizes {
   bool left;
   int64_t d, L, srows, scols, nel, nblk;
-  int q_block, block, proj_splits, tc_splits;
+  int q_block, block, proj_splits, tc_splits, step_splits;
   int64_t ld_part, ld_n, ld_s, ld_p;
   int p_planes;
   bool tensor_path;
   size_t off_P, off_M, off_V, off_Mam, off_Vam, state_bytes;
   size_t off_vrow, off_vcol;
   size_t off_status, off_R, off_N, off_Pp, off_af, off_refresh, ws_bytes;
+  bool g_copy;           // room for a copy of G at off_G
+  size_t off_G;
 };
+int64_t g_copy_ld(const galore_config_t& c) { return (c.n + 7) / 8 * 8; }
 
 // fp32 W and G under fp32 Adam moments keep one order of the projection's sums (gemm_fma.cu says why).
 bool fma_projection(const galore_config_t& c) {
@@ -206,8 +269,9 @@ galore_status_t resolve(const galore_config_t* c, Sizes* s) {
   s->block = (int)std::min<int64_t>(s->d, (int64_t)r + over);
 
   // K slices of the projection
-  s->proj_splits = fma_projection(*c) ? fma_choose_slices(s->srows, s->scols, s->d) : split_choose_slices(s->srows, s->scols, s->d, c->p_dtype == GALORE_F32 && c->g_dtype == GALORE_F32);
+  s->proj_splits = fma_projection(*c) ? fma_choose_slices(s->srows, s->scols, s->d) : split_choose_slices(s->srows, s->scols, s->d);
   s->tc_splits = s->tensor_path ? tensor_proj_splits(*c, s->left) : 0;
+  s->step_splits = s->tensor_path ? tensor_step_splits(*c, s->left) : 0;
   s->ld_part = (s->scols + 7) / 8 * 8;     // 32-byte rows for whole-sector vector stores
   s->ld_n = (s->scols + 15) / 16 * 16;     // 32-byte bf16 rows: TMA needs 16, the epilogue that writes N stores 32 at a time
   // the weight update reads bf16 operands in 16-byte rows
@@ -236,12 +300,21 @@ galore_status_t resolve(const galore_config_t* c, Sizes* s) {
 
   o = 0;
   s->off_status = o; o += 256;
-  s->off_R = o; o += align_up((size_t)std::max(s->proj_splits, s->tc_splits) * s->srows * s->ld_part * 4, 256);
+  s->off_R = o; o += align_up((size_t)std::max({s->proj_splits, s->tc_splits, s->step_splits}) * s->srows * s->ld_part * 4, 256);
   s->off_N = o; o += align_up((size_t)s->srows * s->ld_n * 2 * 3, 256);        // three planes where the product keeps fp32 precision
   s->off_Pp = o; o += align_up((size_t)s->p_planes * s->d * s->ld_p * 2, 256);
   s->off_af = o;
   if (c->state_fmt == GALORE_STATE_ADAFACTOR) o += adafactor_scratch_bytes(s->srows, s->scols);
   s->off_refresh = o; o += refresh_workspace_bytes(s->d, s->L, r, s->block);
+  // A step does not run beside a refresh: the copy of G shares the refresh's scratch where it fits in front of the unrounded projector,
+  // which outlives the refresh.
+  s->g_copy = s->tensor_path && c->n % 8 != 0;
+  s->off_G = s->off_refresh;
+  const size_t g_bytes = (size_t)c->m * g_copy_ld(*c) * 2;
+  if (s->g_copy && g_bytes > refresh_scratch_head(s->d, s->L, r, s->block)) {
+    s->off_G = o;
+    o += align_up(g_bytes, 256);
+  }
   s->ws_bytes = o;
   return GALORE_OK;
 }
@@ -358,16 +431,46 @@ galore_status_t launch_apply(const ApplyItem& item, int32_t w_dtype, cudaStream_
   return launch_apply_group(g, w_dtype, true, st);
 }
 
+struct GroupHolder {      // one per thread: a launch's arguments are collected in it
+  TensorGroup* g = tensor_group_new();
+  ~GroupHolder() { tensor_group_free(g); }
+};
+TensorGroup* fresh_group() {
+  static thread_local GroupHolder holder;
+  if (holder.g) tensor_group_reset(holder.g);
+  return holder.g;
+}
+
 galore_status_t step_split(galore_layer* l, void* W, int64_t ldw, const void* G, int64_t ldg, float lr,
                            const AdamParams& ap, cudaStream_t st) {
+  // bf16 operands by TMA where the projector allows it, G in a copy if need be, unless the product is too short to pay for the
+  // copy (45 us instead of 77 for 2048 x 5461 of packed rows at rank 512, 17.4 instead of 19.1 for 1000 x 2049 at 320; 18.7
+  // instead of 12.8 for 700 x 1501 at 128).  The same sums, a k-block at a time, in the same slices: one slice would take 4 us
+  // less and the sum of 32 blocks in one chain be 1.2e-7 from 64 bits instead of 0.9e-7.
+  const bool aligned_g = (((uintptr_t)G | (uintptr_t)(ldg * 2)) & 15) == 0;
+  const bool by_tma = l->tensor_path &&
+                      (aligned_g || (l->Gcopy && split_store_us(l->srows, l->scols, l->d, l->proj_splits) > 11.0 + (double)l->d * (double)l->L / 2.0e6));
+  const int splits = l->proj_splits;
   {
     PhaseTimer pt(0, st);
-    const ProjectJob job{l, G, ldg, l->Rpart, l->proj_splits};
-    GALORE_TRY(launch_projections(&job, 1, true, st));     // early: see step_tensor
+    if (by_tma) {
+      if (!aligned_g) {
+        GALORE_TRY(launch_align_rows(G, ldg, l->Gcopy, g_copy_ld(l->cfg), (int)l->cfg.m, (int)l->cfg.n, st));
+        G = l->Gcopy;
+        ldg = g_copy_ld(l->cfg);
+      }
+      TensorGroup* g = fresh_group();
+      if (!g) return GALORE_ERR_INVALID_ARG;
+      GALORE_TRY(tensor_group_add_project(g, &l->tc, l->cfg, l->left, G, ldg, l->Rpart, l->ld_part, splits, l->status));
+      GALORE_TRY(tensor_group_launch_project_drained(g, 1, true, st));
+    } else {
+      const ProjectJob job{l, G, ldg, l->Rpart, splits};
+      GALORE_TRY(launch_projections(&job, 1, true, st));     // early: see step_tensor
+    }
   }
   {
     PhaseTimer pt(1, st);
-    AdamItem a = adam_item(l, l->Rpart, l->proj_splits, l->Nbuf, ap);
+    AdamItem a = adam_item(l, l->Rpart, splits, l->Nbuf, ap);
     a.split = projector_split(l, l->Pplanes);
     GALORE_TRY(launch_regulariser(l, a, 3, st));
   }
@@ -406,17 +509,12 @@ bool adam_in_projection(const galore_layer* l, int splits) {
 
 galore_status_t step_tensor(galore_layer* l, void* W, int64_t ldw, const void* G, int64_t ldg, float lr,
                             const AdamParams& ap, cudaStream_t st) {
-  static thread_local struct Scratch {
-    TensorGroup* g = tensor_group_new();
-    ~Scratch() { tensor_group_free(g); }
-  } scratch;
-  TensorGroup* g = scratch.g;
+  TensorGroup* g = fresh_group();
   if (!g) return GALORE_ERR_INVALID_ARG;
-  tensor_group_reset(g);
   // The projection is launched early too: behind another layer's update its barriers, tensor maps and TMEM are set up while
   // that one drains (every role waits for the kernel before it touches memory).  Stepped one after the other, 2048 x 2048
   // matrices of rank 512 take 32.3 us each instead of 35.2, 512 x 1376 of rank 128 21.4 instead of 22.3.
-  if (adam_in_projection(l, l->tc.splits)) {
+  if (adam_in_projection(l, l->tc_splits)) {
     // one K slice per tile: Adam runs in the projection's epilogue, R never reaches memory
     PhaseTimer pt(0, st);
     GALORE_TRY(tensor_group_add_project_adam(g, &l->tc, l->cfg, l->left, G, ldg, tc_adam_args(l, l->Nbuf, ap), l->status));
@@ -424,11 +522,13 @@ galore_status_t step_tensor(galore_layer* l, void* W, int64_t ldw, const void* G
   } else {
     {
       PhaseTimer pt(0, st);
-      GALORE_TRY(tensor_group_add_project(g, &l->tc, l->cfg, l->left, G, ldg, l->Rpart, l->ld_part, l->tc.splits, l->status));
-      GALORE_TRY(tensor_group_launch_project(g, true, st));
+      // Slices chosen by their time, accumulators no longer than those of slices that fill the machine: what the tensor core's
+      // rounding towards zero takes off R grows with their length.
+      GALORE_TRY(tensor_group_add_project(g, &l->tc, l->cfg, l->left, G, ldg, l->Rpart, l->ld_part, l->step_splits, l->status));
+      GALORE_TRY(tensor_group_launch_project_drained(g, tensor_chain_blocks(l->d, l->tc_splits), true, st));
     }
     PhaseTimer pt(1, st);
-    GALORE_TRY(launch_regulariser(l, adam_item(l, l->Rpart, l->tc.splits, l->Nbuf, ap), 1, st));
+    GALORE_TRY(launch_regulariser(l, adam_item(l, l->Rpart, l->step_splits, l->Nbuf, ap), 1, st));
   }
   PhaseTimer pt(2, st);
   return launch_apply(apply_item(l, l->Nbuf, 1, nullptr, W, ldw, lr), l->cfg.w_dtype, st);
@@ -533,7 +633,7 @@ galore_status_t galore_init_layer(const galore_config_t* cfg, void* state_buf, s
   l->has_projector = false;
   l->d = s.d; l->L = s.L; l->srows = s.srows; l->scols = s.scols; l->nel = s.nel;
   l->q_block = s.q_block; l->nblk = s.nblk; l->block = s.block; l->proj_splits = s.proj_splits;
-  l->tc_splits = s.tc_splits; l->ld_part = s.ld_part; l->ld_n = s.ld_n; l->ld_s = s.ld_s;
+  l->tc_splits = s.tc_splits; l->step_splits = s.step_splits; l->ld_part = s.ld_part; l->ld_n = s.ld_n; l->ld_s = s.ld_s;
   l->p_planes = s.p_planes; l->ld_p = s.ld_p;
   l->k = 0;
   char* sb = (char*)state_buf;
@@ -560,6 +660,7 @@ galore_status_t galore_init_layer(const galore_config_t* cfg, void* state_buf, s
   l->Nbuf = (__nv_bfloat16*)(ws + s.off_N);
   l->Pplanes = (__nv_bfloat16*)(ws + s.off_Pp);
   l->refresh_ws = ws + s.off_refresh;
+  l->Gcopy = s.g_copy ? (__nv_bfloat16*)(ws + s.off_G) : nullptr;
   l->state_bytes = s.state_bytes;
 
   cudaError_t e = cudaSuccess;
@@ -583,7 +684,7 @@ galore_status_t galore_init_layer(const galore_config_t* cfg, void* state_buf, s
     return GALORE_ERR_CUDA;
   }
   if (l->tensor_path) {
-    galore_status_t ts = tensor_plan_init(&l->tc, *cfg, l->left, l->P, l->tc_splits);
+    galore_status_t ts = tensor_plan_init(&l->tc, *cfg, l->left, l->P);
     if (ts < 0) {
       delete l;
       return ts;

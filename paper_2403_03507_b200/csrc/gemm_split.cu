@@ -505,21 +505,23 @@ int64_t split_units(int64_t M, int64_t N, int64_t slices, int tile) { return cei
 
 // The time of the launch plus that of reading back the partial results: the Adam kernel behind it reads a slice at 4.8 TB/s.
 // (With 0.6 us a k-block for bf16 512 x 5461 x 2048 was cut in two: 153 us a step instead of 146.)
-int split_choose_slices(int64_t M, int64_t N, int64_t K, bool pairs) {
+int split_choose_slices(int64_t M, int64_t N, int64_t K) {
   const int64_t kb = ceil_div(K, kSplitK);
   int best = 1;
   double best_us = 1e30;
   for (int s = 1; s <= 16; ++s) {
     if (split_effective_slices(K, s) != s) continue;
-    double us = split_us(split_units(M, N, s, 128), ceil_div(kb, s), false);
-    if (pairs) us = std::min(us, split_us(split_units(M, N, s, 256), ceil_div(kb, s), true));
-    us += s * (0.35 + (double)(M * N) * 4.0 / 4.8e6);
+    const double us = split_us(split_units(M, N, s, 128), ceil_div(kb, s), false) + s * (0.35 + (double)(M * N) * 4.0 / 4.8e6);
     if (us < best_us) {
       best_us = us;
       best = s;
     }
   }
   return best;
+}
+
+double split_store_us(int64_t M, int64_t N, int64_t K, int slices) {
+  return split_us(split_units(M, N, slices, 128), ceil_div(ceil_div(K, kSplitK), slices), false);
 }
 
 galore_status_t split_group_add_store(SplitGroup& g, int M, int N, int K, const SplitOperand& a, const SplitOperand& b, int splits,

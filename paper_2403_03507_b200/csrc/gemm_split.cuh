@@ -41,8 +41,9 @@ using SplitGroup = SplitArgs<kSplitGroup>;
 
 // operand X(i, k) = base[i * s_mn + k * s_k]; one of the strides is 1
 SplitOperand split_operand(const void* base, int32_t dtype, int64_t s_mn, int64_t s_k);
-// K slices that balance filling the machine against the traffic of the partial results; pairs: see launch_split_store
-int split_choose_slices(int64_t M, int64_t N, int64_t K, bool pairs);
+// K slices that balance filling the machine against the traffic of the partial results
+int split_choose_slices(int64_t M, int64_t N, int64_t K);
+double split_store_us(int64_t M, int64_t N, int64_t K, int slices);      // what one such product takes in 128 x 128 tiles
 int split_effective_slices(int64_t K, int slices);
 galore_status_t split_group_add_store(SplitGroup& g, int M, int N, int K, const SplitOperand& a, const SplitOperand& b, int splits,
                                       float* C, int64_t ldc, int64_t split_stride, int32_t* status);

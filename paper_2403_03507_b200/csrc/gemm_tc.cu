@@ -40,22 +40,26 @@ namespace galore {
 namespace {
 
 constexpr int kBM = 128;          // rows of an output tile = TMEM lanes
-constexpr int kBN = 256;          // columns of an output tile = TMEM columns per accumulator
+constexpr int kBN = 256;          // columns of an output tile = TMEM columns per accumulator (single products with up to 128: 128)
 constexpr int kBK = 64;           // K per stage: 64 bf16 = one 128-byte swizzle row
 constexpr int kUmmaK = 16;
 constexpr uint32_t kTmemCols = 512;
 constexpr int kABytes = kBM * kBK * 2;            // 16 KiB: the 128 rows of A one CTA stages per k-block
 
 // EPI_ADAM_F32 / EPI_ADAM_Q8: the projection with Adam on its output tile (fp32 / 8-bit moments).
-enum { EPI_PARTIAL = 0, EPI_ADAM_F32 = 1, EPI_ADAM_Q8 = 2 };
+// EPI_DRAIN: EPI_PARTIAL with shorter chains.  The tensor core's accumulator rounds towards zero; here it is added to fp32 sums in
+// the epilogue's registers after every few k-blocks (R of 2048 x 5461 at rank 512: after each one 9e-8 from 64 bits, in one
+// accumulator 8e-7).
+enum { EPI_PARTIAL = 0, EPI_ADAM_F32 = 1, EPI_ADAM_Q8 = 2, EPI_DRAIN = 3 };
 constexpr bool epi_is_adam(int epi) { return epi == EPI_ADAM_F32 || epi == EPI_ADAM_Q8; }
 // Adam is instruction-heavy (about 70 per element with 8-bit moments) and every element is a chain
 // of dependent lookups and arithmetic: sixteen epilogue warps, four per quarter of the accumulator's
 // lanes with 64 columns each, give every scheduler of the SM four warps to switch between while the
 // tensor cores work on the next tile (eight warps of 128 columns each ran three times longer than
 // the MMAs of a tile).
-constexpr int epi_warps(int epi) { return epi_is_adam(epi) ? 16 : 4; }
-constexpr int epi_threads(int epi) { return 64 + 32 * epi_warps(epi) + (epi == EPI_ADAM_F32 ? 32 : 0); }   // + producer, MMA, moments
+// Sixteen as well (64 columns each) where accumulators are drained after every k-block: a pair's MMAs take 512 cycles for one.
+constexpr int epi_warps(int epi, int bn) { return epi == EPI_PARTIAL ? 4 : (epi == EPI_DRAIN ? bn / 16 : 16); }
+constexpr int epi_threads(int epi, int bn) { return 64 + 32 * epi_warps(epi, bn) + (epi == EPI_ADAM_F32 ? 32 : 0); }   // + producer, MMA, moments
 constexpr int epi_smem(int epi) { return epi == EPI_ADAM_Q8 ? (int)sizeof(Q8Tables) : 0; }
 
 // A piece of a moment: 32 rows x 64 columns, as two boxes of 32 x 32 (128 bytes a row).  It belongs to the four epilogue warps
@@ -72,14 +76,14 @@ constexpr int kMomentBytes = kMomentRows * kMomentCols * 4;
 // is out of the way and the operands' latency bounds the tile (eight layers of LLaMA-1B size at rank 512: 611 -> 523 us of
 // 392 for the bytes).  Pieces of 128 rows x 32 columns with 5 / 4 / 3 stages: 529 / 541 / 596 us; rows of 64 bytes
 // (16 columns): 595 and more; 32 x 32 with 6 stages: 566.
-template <int CTAS, int EPI>
+template <int CTAS, int EPI, int BN>
 struct Geo {
   static constexpr int kTileM = kBM * CTAS;
-  static constexpr int kBNcta = kBN / CTAS;
+  static constexpr int kBNcta = BN / CTAS;
   static constexpr int kBBytes = kBNcta * kBK * 2;
   static constexpr int kStageBytes = kABytes + kBBytes;
   static constexpr bool kMoments = EPI == EPI_ADAM_F32;
-  static constexpr int kStages = kMoments ? (CTAS == 1 ? 3 : 5) : (CTAS == 1 ? 4 : 6);
+  static constexpr int kStages = kMoments ? (CTAS == 1 ? 3 : 5) : 192 * 1024 / kStageBytes;
   static constexpr int kSlots = kMoments ? 4 : 0;              // pieces of M and of V, one per quarter of the rows
   static constexpr int kRingBytes = kStages * kStageBytes + kSlots * 2 * kMomentBytes;
   static constexpr int kSmemBytes = kRingBytes + 1024 /* alignment slack */ + 256 /* barriers */;
@@ -93,6 +97,7 @@ struct TcParams {
   int a_mn, b_mn;             // operand majors in shared memory: 1 = M/N contiguous, 0 = K contiguous
   int tiles_m, tiles_n, splits;
   int kblocks_total, kblocks_per_split;
+  int drain;                  // EPI_DRAIN: k-blocks per accumulator
   int m_fast;                 // 1: consecutive units walk tile_m first (B panel shared), 0: tile_n first
   // EPI_PARTIAL
   float* part;
@@ -137,16 +142,16 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr, bool mn_major) {
 }
 
 // Instruction descriptor: fp32 accumulate, bf16 x bf16, majors, N, M.
-__host__ __device__ constexpr uint32_t instr_desc(int a_mn, int b_mn, int tile_m) {
+__host__ __device__ constexpr uint32_t instr_desc(int a_mn, int b_mn, int tile_m, int tile_n) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((a_mn ? 1u : 0u) << 15) | ((b_mn ? 1u : 0u) << 16) |
-         ((uint32_t)(kBN >> 3) << 17) | ((uint32_t)(tile_m >> 4) << 24);
+         ((uint32_t)(tile_n >> 3) << 17) | ((uint32_t)(tile_m >> 4) << 24);
 }
 
 struct Unit {
   int m0, n0, split, kb_begin, kb_end;
 };
 
-template <int CAP>
+template <int BN, int CAP>
 __device__ __forceinline__ Unit decode_unit(const TcArgs<CAP>& g, int u, GroupCursor& cursor) {
   u = cursor.seek<CAP>(g, u);
   const TcParams& p = g.p[cursor.pi];
@@ -162,7 +167,7 @@ __device__ __forceinline__ Unit decode_unit(const TcArgs<CAP>& g, int u, GroupCu
   }
   Unit w;
   w.m0 = tm * p.tile_m;
-  w.n0 = tn * kBN;
+  w.n0 = tn * BN;
   w.split = s;
   w.kb_begin = s * p.kblocks_per_split;
   w.kb_end = min(p.kblocks_total, w.kb_begin + p.kblocks_per_split);
@@ -402,11 +407,11 @@ __device__ __forceinline__ bool epi_adam_q8(const TcParams& p, int row, int col0
 
 // ---- the kernel -------------------------------------------------------------------------------
 
-template <int EPI, int CTAS, int CAP>
-__global__ void __launch_bounds__(epi_threads(EPI), 1)
+template <int EPI, int CTAS, int CAP, int BN>
+__global__ void __launch_bounds__(epi_threads(EPI, BN), 1)
 gemm_tc_kernel(const __grid_constant__ TcArgs<CAP> g) {
-  using G = Geo<CTAS, EPI>;
-  constexpr int kEpiWarps = epi_warps(EPI);
+  using G = Geo<CTAS, EPI, BN>;
+  constexpr int kEpiWarps = epi_warps(EPI, BN);
   constexpr int kStages = G::kStages;
   constexpr int kStageBytes = G::kStageBytes;
   extern __shared__ uint8_t smem_raw[];
@@ -465,7 +470,7 @@ gemm_tc_kernel(const __grid_constant__ TcArgs<CAP> g) {
   }
   // the 8-bit code tables follow the barriers (256 bytes after the ring)
   Q8Tables* q8t = reinterpret_cast<Q8Tables*>(ring_ptr + G::kRingBytes + 256);
-  if constexpr (EPI == EPI_ADAM_Q8) q8_tables_fill(*q8t, g.q8, (int)threadIdx.x, epi_threads(EPI));
+  if constexpr (EPI == EPI_ADAM_Q8) q8_tables_fill(*q8t, g.q8, (int)threadIdx.x, epi_threads(EPI, BN));
   tc_fence_before();
   __syncthreads();
   if (CTAS == 2) cluster_sync_all();                // the peer's barriers exist before anyone signals them
@@ -483,7 +488,7 @@ gemm_tc_kernel(const __grid_constant__ TcArgs<CAP> g) {
       bool ok = true;
       GroupCursor cursor;
       for (int u = team; u < total_units && ok; u += teams) {
-        const Unit w = decode_unit(g, u, cursor);
+        const Unit w = decode_unit<BN>(g, u, cursor);
         const int pi = cursor.pi;
         const bool A_MN = g.p[pi].a_mn != 0, B_MN = g.p[pi].b_mn != 0;
         const CUtensorMap* map_a = &g.map_a[pi];
@@ -539,18 +544,20 @@ gemm_tc_kernel(const __grid_constant__ TcArgs<CAP> g) {
       bool ok = true;
       GroupCursor cursor;
       for (int u = team; u < total_units && ok; u += teams) {
-        const Unit w = decode_unit(g, u, cursor);
+        const Unit w = decode_unit<BN>(g, u, cursor);
         const int pi = cursor.pi;
         const bool A_MN = g.p[pi].a_mn != 0, B_MN = g.p[pi].b_mn != 0;
-        const uint32_t idesc = instr_desc(g.p[pi].a_mn, g.p[pi].b_mn, G::kTileM);
-        if (!mbar_wait(acce_bar(acc), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
-        tc_fence_after();
-        const uint32_t d_tmem = tmem_base + (uint32_t)(acc * kBN);
+        const uint32_t idesc = instr_desc(g.p[pi].a_mn, g.p[pi].b_mn, G::kTileM, BN);
+        const int drain = EPI == EPI_DRAIN ? g.p[pi].drain : 0;
+        int done = 0;                                 // k-blocks in the accumulator
         for (int kb = w.kb_begin; kb < w.kb_end; ++kb) {
+          const bool fresh = done == 0;
+          if (fresh && !mbar_wait(acce_bar(acc), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
           if (!mbar_wait(full_bar(stage), phase, abort_flag)) { ok = false; break; }
           tc_fence_after();
           const uint32_t a_addr = ring + stage * kStageBytes;
           const uint32_t b_addr = a_addr + kABytes;
+          const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
           const uint64_t a_desc = smem_desc(a_addr, A_MN);
           const uint64_t b_desc = smem_desc(b_addr, B_MN);
 #pragma unroll
@@ -558,7 +565,7 @@ gemm_tc_kernel(const __grid_constant__ TcArgs<CAP> g) {
             // K-major: 16 bf16 = 32 B along the swizzled row; MN-major: 16 k = two 8-k groups of 1024 B
             const uint64_t a_adv = (uint64_t)((A_MN ? k * 2048 : k * 32) >> 4);
             const uint64_t b_adv = (uint64_t)((B_MN ? k * 2048 : k * 32) >> 4);
-            const uint32_t accum = (kb > w.kb_begin || k > 0) ? 1u : 0u;
+            const uint32_t accum = (!fresh || k > 0) ? 1u : 0u;
             if (CTAS == 2) umma_bf16_pair(d_tmem, a_desc + a_adv, b_desc + b_adv, idesc, accum);
             else umma_bf16(d_tmem, a_desc + a_adv, b_desc + b_adv, idesc, accum);
           }
@@ -566,12 +573,14 @@ gemm_tc_kernel(const __grid_constant__ TcArgs<CAP> g) {
           if (CTAS == 2) umma_commit_pair(empty_bar(stage));
           else umma_commit(empty_bar(stage));
           if (++stage == kStages) { stage = 0; phase ^= 1u; }
+          ++done;
+          if ((EPI == EPI_DRAIN && done == drain) || kb + 1 == w.kb_end) {           // accumulator complete
+            done = 0;
+            if (CTAS == 2) umma_commit_pair(accf_bar(acc));
+            else umma_commit(accf_bar(acc));
+            if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+          }
         }
-        if (ok) {                                     // accumulator complete
-          if (CTAS == 2) umma_commit_pair(accf_bar(acc));
-          else umma_commit(accf_bar(acc));
-        }
-        if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
       }
     }
   } else if (G::kMoments && warp == 2 + kEpiWarps) {
@@ -596,10 +605,10 @@ gemm_tc_kernel(const __grid_constant__ TcArgs<CAP> g) {
         };
         GroupCursor cursor;
         for (int u = team; u < total_units && ok; u += teams) {
-          const Unit w = decode_unit(g, u, cursor);
+          const Unit w = decode_unit<BN>(g, u, cursor);
           const int pi = cursor.pi;
           const int row0 = w.m0 + (int)rank * kBM, N = g.p[pi].N;
-          for (int c = 0; c < kBN && w.n0 + c < N && ok; c += kMomentCols) {
+          for (int c = 0; c < BN && w.n0 + c < N && ok; c += kMomentCols) {
             const bool first = pp[0] < 0;
             for (int q = 0; q < 4; ++q) {
               if (!first) {
@@ -630,13 +639,22 @@ gemm_tc_kernel(const __grid_constant__ TcArgs<CAP> g) {
     uint32_t acc_phase = 0;
     uint32_t mv_phase = 0;
     bool ok = true;
+    auto release_acc = [&]() {                        // accumulator free for the MMA warp (the leader's)
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) {
+        if (rank == 0) mbar_arrive(acce_bar(acc));
+        else mbar_arrive_remote(map_to_cta(acce_bar(acc), 0));
+      }
+      if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+    };
     GroupCursor cursor;
     for (int u = team; u < total_units && ok; u += teams) {
-      const Unit w = decode_unit(g, u, cursor);
+      const Unit w = decode_unit<BN>(g, u, cursor);
       const int pi = cursor.pi;
       const TcParams& p = g.p[pi];
       const int row = w.m0 + (int)rank * kBM + quarter * 32 + lane;
-      const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * kBN);
+      const uint32_t t_row = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN);
       if constexpr (EPI == EPI_ADAM_F32) {
         // the four warps of a quarter share its pieces, 16 columns each
         const int part = 16 * ((warp - 2) >> 2);
@@ -647,7 +665,7 @@ gemm_tc_kernel(const __grid_constant__ TcArgs<CAP> g) {
         if (!__all_sync(0xffffffffu, mbar_wait(accf_bar(acc), acc_phase, abort_flag))) { ok = false; break; }
         tc_fence_after();
         bool bad = false;
-        for (int c = 0; c < kBN && w.n0 + c < p.N; c += kMomentCols, mv_phase ^= 1u) {
+        for (int c = 0; c < BN && w.n0 + c < p.N; c += kMomentCols, mv_phase ^= 1u) {
           if (!__all_sync(0xffffffffu, mbar_wait(mvfull_bar(quarter), mv_phase, abort_flag))) { ok = false; break; }
           const int col0 = w.n0 + c + part;
           if (col0 < p.N) {
@@ -675,11 +693,44 @@ gemm_tc_kernel(const __grid_constant__ TcArgs<CAP> g) {
         const bool bad = epi_adam_q8(p, row, col0, t_row + (uint32_t)(part * kAdamCols), accf_bar(acc), acc_phase, abort_flag, *q8t, ok);
         if (!ok) break;
         if (bad) atomicOr(p.status, GALORE_DEV_NONFINITE);
+      } else if constexpr (EPI == EPI_DRAIN) {
+        const int part = 64 * ((warp - 2) >> 2);      // 64 columns a warp
+        float sum[64];
+#pragma unroll
+        for (int j = 0; j < 64; ++j) sum[j] = 0.f;
+#pragma unroll 1
+        for (int kb = w.kb_begin; kb < w.kb_end; kb += p.drain) {
+          if (!__all_sync(0xffffffffu, mbar_wait(accf_bar(acc), acc_phase, abort_flag))) { ok = false; break; }
+          tc_fence_after();
+          const uint32_t t = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * BN + part);
+#pragma unroll
+          for (int c = 0; c < 64; c += 16) {
+            uint32_t v[16];
+            tmem_ld_32x16(t + (uint32_t)c, v);
+            tmem_ld_wait();
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              asm volatile("" : "+r"(v[j]));          // not read before the wait
+              sum[c + j] += __uint_as_float(v[j]);
+            }
+          }
+          release_acc();
+        }
+        if (!ok) break;
+#pragma unroll
+        for (int c = 0; c < 64; c += 32) {
+          if (w.n0 + part + c >= p.N) break;
+          uint32_t v[32];
+#pragma unroll
+          for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(sum[c + j]);
+          epi_partial(p, w, row, w.n0 + part + c, v);
+        }
+        continue;
       } else {
         if (!mbar_wait(accf_bar(acc), acc_phase, abort_flag)) { ok = false; break; }
         tc_fence_after();
 #pragma unroll 1
-        for (int c = 0; c < kBN; c += 32) {
+        for (int c = 0; c < BN; c += 32) {
           if (w.n0 + c >= p.N) break;                 // columns past the matrix: nothing to write
           uint32_t v[32];
           tmem_ld_32x32(t_row + (uint32_t)c, v);
@@ -687,13 +738,7 @@ gemm_tc_kernel(const __grid_constant__ TcArgs<CAP> g) {
           epi_partial(p, w, row, w.n0 + c, v);
         }
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) {                                // accumulator free for the MMA warp (the leader's)
-        if (rank == 0) mbar_arrive(acce_bar(acc));
-        else mbar_arrive_remote(map_to_cta(acce_bar(acc), 0));
-      }
-      if (++acc == 2) { acc = 0; acc_phase ^= 1u; }
+      release_acc();
     }
   }
 
@@ -792,17 +837,17 @@ LaunchOrder<CudaOrder>& launch_order() {
 
 namespace {
 
-template <int EPI, int CTAS, int CAP>
+template <int EPI, int CTAS, int CAP, int BN = kBN>
 galore_status_t launch_tc_variant(const TcArgs<CAP>& g, bool early, cudaStream_t st) {
-  constexpr int smem = Geo<CTAS, EPI>::kSmemBytes + epi_smem(EPI);
+  constexpr int smem = Geo<CTAS, EPI, BN>::kSmemBytes + epi_smem(EPI);
   static_assert(smem <= 227 * 1024, "shared memory of one CTA");
   static std::atomic<uint64_t> configured{0};
-  auto kern = gemm_tc_kernel<EPI, CTAS, CAP>;
+  auto kern = gemm_tc_kernel<EPI, CTAS, CAP, BN>;
   GALORE_TRY(allow_smem(configured, (const void*)kern, smem));
   const int units = g.unit_end[g.count - 1];
   if (units <= 0) return GALORE_OK;
   const int teams = std::min(units, tensor_sm_count() / CTAS);
-  return launch_kernel(kern, dim3((unsigned)(teams * CTAS)), epi_threads(EPI), smem, CTAS, early, st, g);
+  return launch_kernel(kern, dim3((unsigned)(teams * CTAS)), epi_threads(EPI, BN), smem, CTAS, early, st, g);
 }
 
 // every problem of a group was tiled for the same variant (TcParams::tile_m)
@@ -822,9 +867,12 @@ galore_status_t launch_tc(const TcGroup& g, bool early, cudaStream_t st) {
     one.q8 = g.q8;
     one.map_m[0] = g.map_m[0];
     one.map_v[0] = g.map_v[0];
+    if constexpr (EPI == EPI_DRAIN || EPI == EPI_PARTIAL)
+      if (!pair && g.p[0].N <= 128) return launch_tc_variant<EPI, 1, 1, 128>(one, early, st);      // (the group's units are the same)
     return pair ? launch_tc_variant<EPI, 2, 1>(one, early, st) : launch_tc_variant<EPI, 1, 1>(one, early, st);
   }
-  return pair ? launch_tc_variant<EPI, 2, kMaxGroup>(g, early, st) : launch_tc_variant<EPI, 1, kMaxGroup>(g, early, st);
+  if constexpr (EPI == EPI_DRAIN) return GALORE_ERR_INVALID_ARG;      // single matrices only
+  else return pair ? launch_tc_variant<EPI, 2, kMaxGroup>(g, early, st) : launch_tc_variant<EPI, 1, kMaxGroup>(g, early, st);
 }
 
 // appends one problem to a group
@@ -848,7 +896,7 @@ void fill_tiles(TcParams& p, int M, int N, int K, int splits, int ctas) {
 }
 
 // K slices that fill the last wave of CTAs best, keeping at least 4 k-blocks per slice
-int choose_splits(int64_t M, int64_t N, int64_t K, int ctas) {
+int fill_splits(int64_t M, int64_t N, int64_t K, int ctas) {
   const int64_t tiles = ceil_div(M, kBM * ctas) * ceil_div(N, kBN);
   const int kblocks = (int)ceil_div(K, kBK);
   const int sms = 148 / ctas;
@@ -868,6 +916,26 @@ int choose_splits(int64_t M, int64_t N, int64_t K, int ctas) {
   return best;
 }
 
+// K slices of a single product (EPI_DRAIN) with a kernel behind it that reads the partial results: the least of waves x (k-blocks x
+// time of one + time of a unit) plus the slices' round trip.  Microseconds a k-block, fitted to steps in 1 to 7 slices of 2048 x 2048 and
+// 2048 x 5461 at rank 512, 4096 x 11008 at 1024, 11008 x 4096 and 4096 x 11008 at 128: pairs 0.33, single CTAs 0.35, with tiles
+// of 128 columns 0.25.  (2048 x 5461, 8-bit moments: 58.9 us unsliced, 61.4 in three, 68.1 in five, which fill the machine best.)
+int time_splits(int64_t M, int64_t N, int64_t K, int ctas) {
+  const int64_t tiles = ceil_div(M, kBM * ctas) * ceil_div(N, kBN);
+  const int kblocks = (int)ceil_div(K, kBK);
+  const double block = ctas == 2 ? 0.33 : (N <= 128 ? 0.25 : 0.35);
+  int best = 1;
+  double best_us = 1e30;
+  for (int s = 1; s <= 8; ++s) {
+    const int per = (int)ceil_div(kblocks, s);
+    if (s > 1 && per < 4) break;
+    if ((int)ceil_div(kblocks, per) != s) continue;
+    const double us = (double)ceil_div(tiles * s, 148 / ctas) * (per * block + 1.1) + s * (0.1 + (double)(M * N) * 4.0 / 6.0e6);
+    if (us < best_us) { best_us = us; best = s; }
+  }
+  return best;
+}
+
 }  // namespace
 
 bool tensor_path_eligible(const galore_config_t& c) {
@@ -879,14 +947,17 @@ int tensor_ctas(const galore_config_t& c) { return c.rank >= 256 ? 2 : 1; }
 
 int tensor_proj_splits(const galore_config_t& c, bool left) {
   const int ctas = tensor_ctas(c);
-  if (left) return choose_splits(c.rank, c.n, c.m, ctas);
-  return choose_splits(c.m, c.rank, c.n, ctas);
+  return left ? fill_splits(c.rank, c.n, c.m, ctas) : fill_splits(c.m, c.rank, c.n, ctas);
+}
+int tensor_chain_blocks(int64_t K, int splits) { return (int)ceil_div(ceil_div(K, kBK), std::max(1, splits)); }
+int tensor_step_splits(const galore_config_t& c, bool left) {
+  const int ctas = tensor_ctas(c);
+  return left ? time_splits(c.rank, c.n, c.m, ctas) : time_splits(c.m, c.rank, c.n, ctas);
 }
 
-galore_status_t tensor_plan_init(TensorPlan* plan, const galore_config_t& c, bool left, void* P, int splits) {
+galore_status_t tensor_plan_init(TensorPlan* plan, const galore_config_t& c, bool left, void* P) {
   plan->ready = false;
   plan->ctas = tensor_ctas(c);
-  plan->splits = splits;
   const int64_t r = c.rank;
   if (left) {
     // A = P^T, MN-major from P (m x r)
@@ -1038,6 +1109,11 @@ galore_status_t tensor_group_add_gemm(TensorGroup* t, const void* A, int64_t lda
 galore_status_t tensor_group_launch_project(TensorGroup* t, bool early, cudaStream_t st) {
   if (t->g.count == 0) return GALORE_OK;
   return launch_tc<EPI_PARTIAL>(t->g, early, st);
+}
+galore_status_t tensor_group_launch_project_drained(TensorGroup* t, int blocks, bool early, cudaStream_t st) {
+  if (t->g.count != 1 || blocks < 1) return GALORE_ERR_INVALID_ARG;
+  t->g.p[0].drain = blocks;
+  return blocks < t->g.p[0].kblocks_per_split ? launch_tc<EPI_DRAIN>(t->g, early, st) : launch_tc<EPI_PARTIAL>(t->g, early, st);
 }
 
 }  // namespace galore

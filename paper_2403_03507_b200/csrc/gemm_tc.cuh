@@ -29,16 +29,17 @@ struct TcAdamArgs {
 // of G is encoded per call.
 struct TensorPlan {
   bool ready = false;
-  int splits = 1;             // K slices of the projection
   int ctas = 1;               // 1: 128-row tiles per CTA; 2: 256-row tiles per CTA pair (cta_group::2)
   CUtensorMap map_p_proj;     // projector as an operand of the projection
 };
 
 // bf16 G and P, rank a multiple of 8 (16-byte rows for TMA).
 bool tensor_path_eligible(const galore_config_t& cfg);
-int tensor_proj_splits(const galore_config_t& cfg, bool left);
+int tensor_proj_splits(const galore_config_t& cfg, bool left);       // K slices that fill the machine
+int tensor_chain_blocks(int64_t K, int splits);                       // 64 of K that one accumulator of such a slice sums
+int tensor_step_splits(const galore_config_t& cfg, bool left);       // those a layer's own step takes (drained accumulators)
 int tensor_ctas(const galore_config_t& cfg);
-galore_status_t tensor_plan_init(TensorPlan* plan, const galore_config_t& cfg, bool left, void* P, int splits);
+galore_status_t tensor_plan_init(TensorPlan* plan, const galore_config_t& cfg, bool left, void* P);
 // G and W usable by this path: 16-byte aligned bases and rows.
 bool tensor_operands_aligned(const galore_config_t& cfg, const void* W, int64_t ldw, const void* G, int64_t ldg);
 // ---- groups: up to tensor_group_capacity() layers per launch ------------------------------------
@@ -61,6 +62,8 @@ galore_status_t tensor_group_launch_project_adam(TensorGroup* t, int32_t state_f
 galore_status_t tensor_group_add_gemm(TensorGroup* t, const void* A, int64_t lda, int a_mn, const void* B, int64_t ldb,
                                       int b_mn, int M, int N, int K, float* C, int64_t ldc, int32_t* status);
 galore_status_t tensor_group_launch_project(TensorGroup* t, bool early, cudaStream_t st);
+// one layer's projection, its accumulators added to fp32 sums after every `blocks` times 64 of K
+galore_status_t tensor_group_launch_project_drained(TensorGroup* t, int blocks, bool early, cudaStream_t st);
 
 struct CudaOrder {
   using Status = galore_status_t;

@@ -428,6 +428,9 @@ static RefreshBuffers layout(void* base, int64_t d, int64_t L, int r, int b) {
   return w;
 }
 
+size_t refresh_scratch_head(int64_t d, int64_t L, int r, int b) {
+  return (size_t)((char*)layout(nullptr, d, L, r, b).P64 - (char*)nullptr);
+}
 const double* refresh_unrounded_projector(void* workspace, int64_t d, int64_t L, int r, int b) {
   return layout(workspace, d, L, r, b).P64;
 }

@@ -27,6 +27,9 @@ struct RefreshProblem {
 // d = rows of the projector, L = the other dimension of G
 size_t refresh_workspace_bytes(int64_t d, int64_t L, int r, int b);
 
+// bytes of it in front of the unrounded projector
+size_t refresh_scratch_head(int64_t d, int64_t L, int r, int b);
+
 // Where the last refresh through `workspace` left its projector before rounding to the stored
 // dtype: rows x rank doubles, row-major.  Valid until the workspace is written again.
 const double* refresh_unrounded_projector(void* workspace, int64_t d, int64_t L, int r, int b);

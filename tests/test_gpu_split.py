@@ -76,3 +76,43 @@ def test_products_of_large_groups_are_fp32_products(m, n, r, count, pad):
         # as above: an fp32 sum of K terms; the accumulators of 32 of K lose at most a unit of 2^-23 of one sign per 16 products
         assert float((M / 0.1 - R).norm() / R.norm()) <= 2 ** -24 * (8 + (m if layer.side == gb.SIDE_LEFT else n) ** 0.5)
         assert abs(float((M / 0.1 * R).sum() / (R * R).sum()) - 1) <= 2e-7
+
+
+# bf16 rows that TMA cannot address, in products long enough for a copy of G on 16-byte rows; tiles of one CTA and of pairs in
+# the update (its rows go through shared memory in 16-byte units).  off: columns of W and G in front of the matrix, in the same rows
+@pytest.mark.parametrize("m,n,r,off,pad", [(2048, 2051, 512, 0, 0), (2051, 1031, 264, 0, 0), (1000, 2049, 320, 1, 2), (1500, 3001, 128, 3, 0), (4097, 1003, 64, 5, 1),
+                                           (1030, 5461, 512, 7, 4), (2048, 2048, 512, 0, 3)])
+@pytest.mark.parametrize("state", ["f32", "q8"])
+def test_packed_bf16_rows_keep_fp32_precision(m, n, r, off, pad, state):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(m * 31 + n)
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda")
+    layer = gb.Layer(gb.make_config(m, n, r, w_dtype="bf16", g_dtype="bf16", state_fmt=state, auto_refresh=False))
+    layer.set_projector(torch.linalg.qr(rand(layer.proj_rows, r))[0])
+    P = layer.get_projector().double()
+    bufs = []
+    for x in (rand(m, n), 0.02 * rand(m, n)):
+        buf = torch.full((m, off + n + pad), float("nan"), device="cuda", dtype=torch.bfloat16)
+        buf[:, off:off + n] = x
+        bufs.append(buf)
+    G, W = (b[:, off:off + n] for b in bufs)
+    G0, W0 = G.clone(), W.double()
+    layer.galore_step(W, G, 1e-2)
+    assert layer.device_status() == 0
+    left = layer.side == gb.SIDE_LEFT
+    R = P.T @ G.double() if left else G.double() @ P
+    if state == "f32":
+        M, V = (t.double() for t in layer.get_moments())
+        # an fp32 sum of K terms, as above; the accumulator of a k-block loses at most a unit of 2^-23 of one sign per 16 products
+        assert float((M / 0.1 - R).norm() / R.norm()) <= 2 ** -24 * (8 + (m if left else n) ** 0.5)
+        assert abs(float((M / 0.1 * R).sum() / (R * R).sum()) - 1) <= 2e-7
+    # the first step: N = +-1 (with 8-bit moments it is worked out before they are rounded), but for an R that fp32 flushes
+    N = R / (R.abs() + 1e-8)
+    dW = -1e-2 * 0.25 * (P @ N if left else N @ P.T)
+    slack = 2 ** -8 * float((W0.abs() + dW.abs()).max())
+    # an R within the fp32 rounding of zero may come out on the other side: its N is off by 2
+    flips = 2 * 1e-2 * 0.25 * float(P.abs().max()) * float((R.abs() <= 1e-6 * R.square().mean().sqrt()).any())
+    assert float((W.double() - W0 - dW).abs().max()) <= slack + 1e-5 * float(dW.abs().max()) + flips
+    assert torch.equal(G, G0)
+    for buf in bufs:
+        assert torch.isnan(buf[:, :off]).all() and torch.isnan(buf[:, off + n:]).all()

@@ -53,6 +53,8 @@ __device__ __forceinline__ BlockPair block_pair(int pair, int round, int nblk) {
 }
 
 // part[(pair * chunks + chunk)] (64 x 64) = rows(pair)[:, chunk] rows(pair)[:, chunk]^T
+// In the first round of a sweep its upper triangle, later the products of the two blocks with each other alone: those within a
+// block the sweep kernel has carried along since (eight 1280 x 1280 matrices: 40 -> 23 us a round).
 __global__ void __launch_bounds__(128) jb_gram_kernel(const double* X, int b, int nblk, int round, int chunks,
                                                       double* __restrict__ part, const SlotList slots) {
   grid_dependency_wait();
@@ -68,6 +70,8 @@ __global__ void __launch_bounds__(128) jb_gram_kernel(const double* X, int b, in
   if (bp.I * kBlockRows >= b) return;                 // both blocks are padding
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int g = lane >> 2, t = lane & 3;
+  const bool cross = round > 0;                       // warp (wy, wx): 16 x 16 of the 32 x 32 products of the two blocks
+  const int wy = warp >> 1, wx = warp & 1;
   // The Gram matrix is symmetric and the sweep reads its upper triangle only: of the 8 x 8 grid of 8 x 8
   // tiles the 36 with tile row <= tile column are formed.  Warps 0 and 3 take the upper halves of the two
   // diagonal 32 x 32 quadrants (10 tiles each), warps 1 and 2 the two column halves of the off-diagonal one.
@@ -120,7 +124,20 @@ __global__ void __launch_bounds__(128) jb_gram_kernel(const double* X, int b, in
   for (int tile = 0; tile < tiles; ++tile) {
     const int buf = tile & 1;
     if (tile + 1 < tiles) fetch(tile + 1);
-    if (diagonal) {            // upper half of a diagonal quadrant: tiles (i, j) with i <= j
+    if (cross) {
+#pragma unroll
+      for (int ks = 0; ks < 8; ++ks) {
+        double a[2], bb[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) a[i] = Xs[buf][wy * 16 + i * 8 + g][ks * 4 + t];
+#pragma unroll
+        for (int j = 0; j < 2; ++j) bb[j] = Xs[buf][32 + wx * 16 + j * 8 + g][ks * 4 + t];
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+          for (int j = 0; j < 2; ++j) dmma_m8n8k4(acc[i][j], a[i], bb[j]);
+      }
+    } else if (diagonal) {     // upper half of a diagonal quadrant: tiles (i, j) with i <= j
 #pragma unroll
       for (int ks = 0; ks < 8; ++ks) {
         double a[4], bb[4];
@@ -152,7 +169,15 @@ __global__ void __launch_bounds__(128) jb_gram_kernel(const double* X, int b, in
   }
 
   double* out = part + ((int64_t)pair * chunks + chunk) * (kPairRows * kPairRows);
-  if (diagonal) {
+  if (cross) {
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const int r = wy * 16 + i * 8 + g, c = 32 + wx * 16 + j * 8 + 2 * t;
+        *reinterpret_cast<double2*>(out + r * kPairRows + c) = make_double2(acc[i][j][0], acc[i][j][1]);
+      }
+  } else if (diagonal) {
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
@@ -187,20 +212,22 @@ __global__ void __launch_bounds__(128) jb_gram_kernel(const double* X, int b, in
 //   * Rot lives in the registers of 8 warps.  A thread holds 4 slots (8 rows) of two columns; moving on by
 //     one position is a renaming of registers, with one entry of a column passed up and one down to the
 //     lanes that hold the neighbouring slots.
-//   * One warp transforms the 32 blocks with u = v and computes the next round's rotations.  The three
-//     entries that a rotation needs are worked out from the old A and the current rotations again, so the
-//     rotations of round t + 1 are found while the other warps apply those of round t, and a round has a
-//     single barrier.
+//   * One warp keeps the squared norms (the diagonal of A) and the product of every slot's two rows in registers and
+//     computes the next round's rotations.  The product that a rotation needs is worked out from the old A and the
+//     current rotations again, so the rotations of round t + 1 are found while the other warps apply those of round t,
+//     and a round has a single barrier.
+//   * A off the diagonal is held in single precision, scaled so that the largest squared norm is about 1; the norms, Rot, the
+//     sums A comes from and the test for orthogonality are in double precision.  A only decides the angles, every
+//     product keeps a relative error of 1e-6 over the sweep, and the next sweep starts from exact ones: the
+//     number of rotations of each sweep is the same to 1e-3 as with A in double precision, and so is the number of sweeps.
 //   * The angle is computed in single precision (after scaling by the exponent of the larger of
 //     aqq - app and 2 apq) and (c, s) are then renormalised in double precision: the rotation is
-//     orthogonal to double rounding, its angle accurate to about 1e-7, which leaves the pair
-//     orthogonal to 1e-7 of what it was.
-// flags[pair] = rotations applied (0: Rot is the identity and is not written).
+//     orthogonal to double rounding, its angle accurate to about 1e-7.
+// own: the products within each block (32 x 32 of a block, upper triangle), read after the first round of the sweep and
+// written in every one.  flags[pair] = rotations applied (0: Rot is the identity and is not written).
 //
-// What bounds it: 63 rounds one after the other, each about 650 shared-memory wavefronts (half of them reads, then the
-// writes) and, beside them, the latency of an angle; some 900 cycles.  30 us for up to 148 pairs, 47 us for 160; with A
-// and Rot both in shared memory, row by row, and the angles between two barriers it was 48 and 90 us.  Letting the angle
-// warp's reads into the queue first changes nothing.  56 registers: two CTAs on an SM, for groups of more than 148 pairs.
+// What bounds it: 63 rounds one after the other, each the latency of an angle beside about 300 shared-memory wavefronts (650 with A
+// in double precision).  56 registers: two CTAs on an SM, for groups of more than 148 pairs.
 constexpr int kSweepRounds = kPairRows - 1;
 constexpr int kSlots = kPairRows / 2;
 constexpr int kBlockWarps = 8;                                // blocks with u != v: rows 1 .. 16
@@ -213,7 +240,6 @@ constexpr int kLaneCols = 32 / kLaneGroups;
 constexpr int kKindRows = kSlots / 2 + 1;                     // rows of a kind of entry: v - u = 0 .. 16
 constexpr int kKindSize = kKindRows * kSlots;
 constexpr int kPackedSize = 4 * kKindSize;                    // one copy of A
-constexpr size_t kSweepSmem = 2 * (size_t)kPackedSize * sizeof(double);
 constexpr int kLoads = (kPairRows * kPairRows + kSweepThreads - 1) / kSweepThreads;
 
 __host__ __device__ __forceinline__ int next_position(int pos) { return pos == 0 ? 0 : (pos == kPairRows - 1 ? 1 : pos + 1); }
@@ -241,12 +267,12 @@ __device__ __forceinline__ BlockWrites block_writes(int u, int v) {
   return BlockWrites{{packed_offset(nfu, nfv), packed_offset(nfu, ngv), packed_offset(ngu, nfv), packed_offset(ngu, ngv)}};
 }
 struct BlockValues {
-  double a0, a1, a2, a3;
+  float a0, a1, a2, a3;
 };
-// B <- R_u B R_v^T for one 2 x 2 block.  For u == v the two off-diagonal entries are one stored value; both results agree.
-__device__ __forceinline__ void block_write(const BlockWrites& t, const double2 ru, const double2 rv, const BlockValues& b, double* An) {
-  const double r00 = ru.x * b.a0 - ru.y * b.a2, r01 = ru.x * b.a1 - ru.y * b.a3;
-  const double r10 = ru.y * b.a0 + ru.x * b.a2, r11 = ru.y * b.a1 + ru.x * b.a3;
+// B <- R_u B R_v^T for one 2 x 2 block
+__device__ __forceinline__ void block_write(const BlockWrites& t, const float2 ru, const float2 rv, const BlockValues& b, float* An) {
+  const float r00 = ru.x * b.a0 - ru.y * b.a2, r01 = ru.x * b.a1 - ru.y * b.a3;
+  const float r10 = ru.y * b.a0 + ru.x * b.a2, r11 = ru.y * b.a1 + ru.x * b.a3;
   An[t.at[0]] = rv.x * r00 - rv.y * r01;
   An[t.at[1]] = rv.y * r00 + rv.x * r01;
   An[t.at[2]] = rv.x * r10 - rv.y * r11;
@@ -282,35 +308,41 @@ __device__ __forceinline__ double2 jacobi_rotation(double app, double aqq, doubl
 }
 
 __global__ void __launch_bounds__(kSweepThreads, 2) jb_sweep_kernel(const double* part, int chunks, int b, int nblk,
-                                                                 int round, double tol, double* __restrict__ rot_out,
+                                                                 int round, double tol, double* own, double* __restrict__ rot_out,
                                                                  int* __restrict__ flags, int* __restrict__ rotations,
                                                                  const SlotList slots) {
   grid_dependency_wait();
   grid_launch_dependents();
-  extern __shared__ __align__(16) double jb_smem[];
   {
     const int64_t shift = (int64_t)slots.id[blockIdx.y] * slots.bytes;     // blockIdx.y: workspace slot
     part = slot_ptr(part, shift);
+    own = slot_ptr(own, shift);
     rot_out = slot_ptr(rot_out, shift);
     flags = slot_ptr(flags, shift);
     rotations = slot_ptr(rotations, shift);
   }
-  double* const A0 = jb_smem;                     // the Gram matrix, even rounds
-  double* const A1 = jb_smem + kPackedSize;       // odd rounds
-  __shared__ double2 cs[2][kSlots];               // the rotations of the current round and of the next
+  __shared__ float A0[kPackedSize], A1[kPackedSize];      // the Gram matrix off the diagonal, even rounds and odd ones
+  __shared__ double diag[kPairRows];
+  __shared__ float2 cs[2][kSlots];                // the rotations of the current round and of the next
   __shared__ double2 cs_rot[2][kSlots + kLaneGroups];     // the same for the warps of Rot, which read eight slots, 4 apart, at once
-  __shared__ int total;
+  __shared__ int total, top;
   const int pair = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const BlockPair bp = block_pair(pair, round, nblk);
   if (bp.I * kBlockRows >= b) {
     if (tid == 0) flags[pair] = 0;
     return;
   }
+  if (tid == 0) top = 0;
   const double* src = part + (int64_t)pair * chunks * (kPairRows * kPairRows);
-  // entries r <= c of the partial matrices (the tiles below the diagonal are not written)
+  // where the products of rows r and c of one block are carried
+  auto own_at = [&](int r, int c) { return own + (int64_t)(r < kBlockRows ? bp.I : bp.J) * (kBlockRows * kBlockRows) + (r % kBlockRows) * kBlockRows + c % kBlockRows; };
+  // entries r <= c of the partial matrices (what lies below the diagonal is not written)
   double sum[kLoads];
 #pragma unroll
-  for (int i = 0; i < kLoads; ++i) sum[i] = 0.0;
+  for (int i = 0; i < kLoads; ++i) {
+    const int idx = tid + kSweepThreads * i, r = idx >> 6, c = idx & 63;
+    sum[i] = round > 0 && idx < kPairRows * kPairRows && r <= c && (r < kBlockRows) == (c < kBlockRows) ? *own_at(r, c) : 0.0;
+  }
   for (int c = 0; c < chunks; c += 2) {     // two partial matrices in flight
     double v[2][kLoads];
 #pragma unroll
@@ -318,8 +350,9 @@ __global__ void __launch_bounds__(kSweepThreads, 2) jb_sweep_kernel(const double
       const double* sc = src + (int64_t)(c + j) * (kPairRows * kPairRows);
 #pragma unroll
       for (int i = 0; i < kLoads; ++i) {
-        const int idx = tid + kSweepThreads * i;
-        v[j][i] = (c + j < chunks && idx < kPairRows * kPairRows && (idx >> 6) <= (idx & 63)) ? sc[idx] : 0.0;
+        const int idx = tid + kSweepThreads * i, r = idx >> 6, col = idx & 63;
+        const bool summed = round == 0 ? r <= col : r < kBlockRows && col >= kBlockRows;
+        v[j][i] = (c + j < chunks && idx < kPairRows * kPairRows && summed) ? sc[idx] : 0.0;
       }
     }
 #pragma unroll
@@ -327,24 +360,40 @@ __global__ void __launch_bounds__(kSweepThreads, 2) jb_sweep_kernel(const double
 #pragma unroll
       for (int i = 0; i < kLoads; ++i) sum[i] += v[j][i];
   }
+  __syncthreads();
 #pragma unroll
   for (int i = 0; i < kLoads; ++i) {
     const int idx = tid + kSweepThreads * i, r = idx >> 6, c = idx & 63;
-    if (idx < kPairRows * kPairRows && r <= c) A0[packed_offset(r, c)] = sum[i];
+    if (idx < kPairRows * kPairRows && r == c) {
+      diag[r] = sum[i];
+      atomicMax(&top, __double2hiint(sum[i]));
+    }
   }
   const double tol2 = tol * tol;
   __syncthreads();
+  // 2^-e of the largest squared norm
+  const int exponent = min(max(top >> 20, 1), 2045);
+  const double scale = __hiloint2double((2046 - exponent) << 20, 0), unscale = __hiloint2double(exponent << 20, 0);      // scale unscale = 1
   // A pair that is orthogonal already (every pair of the last sweep) keeps its rows: no rotation of the 63 rounds would be
   // applied.
   bool any = false;
 #pragma unroll
   for (int i = 0; i < kLoads; ++i) {
     const int idx = tid + kSweepThreads * i, r = idx >> 6, c = idx & 63;
-    if (idx < kPairRows * kPairRows && r < c)
-      any |= sum[i] * sum[i] > tol2 * A0[packed_offset(r, r)] * A0[packed_offset(c, c)];
+    if (idx < kPairRows * kPairRows && r < c) {
+      any |= sum[i] * sum[i] > tol2 * diag[r] * diag[c];
+      A0[packed_offset(r, c)] = (float)(sum[i] * scale);
+    }
   }
   if (!__syncthreads_or(any)) {
     if (tid == 0) flags[pair] = 0;
+    if (round == 0) {
+#pragma unroll
+      for (int i = 0; i < kLoads; ++i) {
+        const int idx = tid + kSweepThreads * i, r = idx >> 6, c = idx & 63;
+        if (idx < kPairRows * kPairRows && r <= c && (r < kBlockRows) == (c < kBlockRows)) *own_at(r, c) = sum[i];
+      }
+    }
     return;
   }
   // A round starts with a barrier: the copy of A it reads and its rotations are complete, and nobody reads any longer what
@@ -356,14 +405,14 @@ __global__ void __launch_bounds__(kSweepThreads, 2) jb_sweep_kernel(const double
     const BlockWrites w0 = block_writes(lane, v0), w1 = block_writes(lane, v1);
     const bool second = d1 < kSlots / 2 || lane < kSlots / 2;      // half of row 16 says it all
     for (int rr = 0; rr < kSweepRounds; ++rr) {
-      const double* A = (rr & 1 ? A1 : A0) + d0 * kSlots + lane;
-      double* An = rr & 1 ? A0 : A1;
-      const double2* cur = cs[rr & 1];
+      const float* A = (rr & 1 ? A1 : A0) + d0 * kSlots + lane;
+      float* An = rr & 1 ? A0 : A1;
+      const float2* cur = cs[rr & 1];
       round_barrier();
-      const double2 ru = cur[lane], rv0 = cur[v0];
+      const float2 ru = cur[lane], rv0 = cur[v0];
       const BlockValues b0{A[0], A[kKindSize], A[2 * kKindSize], A[3 * kKindSize]};
-      const double2 rv1 = cur[v1];
-      const double* B = A + kBlockWarps * kSlots;
+      const float2 rv1 = cur[v1];
+      const float* B = A + kBlockWarps * kSlots;
       const BlockValues b1{B[0], B[kKindSize], B[2 * kKindSize], B[3 * kKindSize]};
       block_write(w0, ru, rv0, b0, An);
       if (second) block_write(w1, ru, rv1, b1, An);
@@ -420,50 +469,59 @@ __global__ void __launch_bounds__(kSweepThreads, 2) jb_sweep_kernel(const double
       }
     }
   } else {
-    // Lane k: the block of slot k with itself, and the rotation of slot k in the next round.  The rows that will be at
-    // positions k and 63 - k are now row f or g of slot s1 and of slot s2.
+    // Lane k: slot k, its two squared norms and the product of its rows, and its rotation in the next round.  The rows that
+    // will be at positions k and 63 - k are now row f or g of slot s1 and of slot s2.
     const int s1 = lane <= 1 ? 0 : lane - 1, s2 = lane == 31 ? 31 : lane + 1;
     const bool g1 = lane == 1, g2 = lane != 31;
     const int x0 = packed_offset(s1, s2), x1 = packed_offset(s1, kPairRows - 1 - s2),
               x2 = packed_offset(kPairRows - 1 - s1, s2), x3 = packed_offset(kPairRows - 1 - s1, kPairRows - 1 - s2);
-    const BlockWrites own = block_writes(lane, lane);
+    const int left = packed_offset(next_position(lane), next_position(kPairRows - 1 - lane));    // where the slot's own product goes
     const int rot_at = lane + lane / kLaneSlots;
     int applied = 0;
-    {
-      const double2 r = jacobi_rotation(A0[lane], A0[3 * kKindSize + lane], A0[kKindSize + lane], tol2, applied);
-      cs[0][lane] = r;
-      cs_rot[0][rot_at] = r;
-    }
+    double f = diag[lane] * scale, g = diag[kPairRows - 1 - lane] * scale;
+    float o = A0[kKindSize + lane];
+    double2 own_rot = jacobi_rotation(f, g, (double)o, tol2, applied);
+    cs[0][lane] = make_float2((float)own_rot.x, (float)own_rot.y);
+    cs_rot[0][rot_at] = own_rot;
     for (int rr = 0; rr < kSweepRounds; ++rr) {
-      const double* A = rr & 1 ? A1 : A0;
-      double* An = rr & 1 ? A0 : A1;
-      const double2* cur = cs[rr & 1];
+      const float* A = rr & 1 ? A1 : A0;
+      float* An = rr & 1 ? A0 : A1;
+      const float2* cur = cs[rr & 1];
       round_barrier();
-      const double2 r1 = cur[s1], r2 = cur[s2], r0 = cur[lane];
-      const double f1 = A[s1], o1 = A[kKindSize + s1], e1 = A[3 * kKindSize + s1];
-      const double f2 = A[s2], o2 = A[kKindSize + s2], e2 = A[3 * kKindSize + s2];
-      const BlockValues x{A[x0], A[x1], A[x2], A[x3]};
-      const double off = A[kKindSize + lane];
-      const BlockValues b0{A[lane], off, off, A[3 * kKindSize + lane]};
-      const double p1 = g1 ? r1.y : r1.x, q1 = g1 ? r1.x : -r1.y;
-      const double p2 = g2 ? r2.y : r2.x, q2 = g2 ? r2.x : -r2.y;
-      const double app = p1 * (p1 * f1 + q1 * o1) + q1 * (p1 * o1 + q1 * e1);
-      const double aqq = p2 * (p2 * f2 + q2 * o2) + q2 * (p2 * o2 + q2 * e2);
-      const double apq = p2 * (p1 * x.a0 + q1 * x.a2) + q2 * (p1 * x.a1 + q1 * x.a3);
+      const float2 r1 = cur[s1], r2 = cur[s2];
+      const float y0 = A[x0], y1 = A[x1], y2 = A[x2], y3 = A[x3];
+      // this round's rotation of the slot's own two rows
+      const double c = own_rot.x, sn = own_rot.y, od = (double)o;
+      const double fn = c * (c * f - sn * od) - sn * (c * od - sn * g), gn = sn * (sn * f + c * od) + c * (sn * od + c * g);
+      An[left] = (float)(c * (sn * f + c * od) - sn * (sn * od + c * g));
+      // the rows move on
+      const double f_up = __shfl_up_sync(0xffffffffu, fn, 1), g_down = __shfl_down_sync(0xffffffffu, gn, 1), g_first = __shfl_sync(0xffffffffu, gn, 0);
+      f = lane == 0 ? fn : (g1 ? g_first : f_up);
+      g = g2 ? g_down : fn;
+      const float p1 = g1 ? r1.y : r1.x, q1 = g1 ? r1.x : -r1.y;
+      const float p2 = g2 ? r2.y : r2.x, q2 = g2 ? r2.x : -r2.y;
+      o = p2 * (p1 * y0 + q1 * y2) + q2 * (p1 * y1 + q1 * y3);
       if (rr + 1 < kSweepRounds) {
-        const double2 r = jacobi_rotation(app, aqq, apq, tol2, applied);
-        cs[(rr + 1) & 1][lane] = r;
-        cs_rot[(rr + 1) & 1][rot_at] = r;
+        own_rot = jacobi_rotation(f, g, (double)o, tol2, applied);
+        cs[(rr + 1) & 1][lane] = make_float2((float)own_rot.x, (float)own_rot.y);
+        cs_rot[(rr + 1) & 1][rot_at] = own_rot;
       }
-      block_write(own, r0, r0, b0, An);
     }
-    for (int o = 16; o > 0; o >>= 1) applied += __shfl_xor_sync(0xffffffffu, applied, o);
+    for (int k = 16; k > 0; k >>= 1) applied += __shfl_xor_sync(0xffffffffu, applied, k);
     if (lane == 0) {
       total = applied;
       flags[pair] = applied;
       if (applied) atomicAdd(rotations, applied);
     }
+    diag[lane] = f;
+    diag[kPairRows - 1 - lane] = g;
     round_barrier();
+  }
+  // all rows are back at their own positions: the products within the blocks, for the rounds to come
+  const float* A = kSweepRounds & 1 ? A1 : A0;
+  for (int idx = tid; idx < kPairRows * kBlockRows; idx += kSweepThreads) {
+    const int r = idx >> 5, c = (idx & 31) + (r & ~(kBlockRows - 1));
+    if (r <= c) *own_at(r, c) = (r == c ? diag[r] : (double)A[packed_offset(r, c)]) * unscale;
   }
 }
 
@@ -589,6 +647,7 @@ JacobiGeometry jacobi_geometry(int b) {
   return g;
 }
 
+size_t own_bytes(const JacobiGeometry& g) { return align_up((size_t)g.nblk * kBlockRows * kBlockRows * sizeof(double), 256); }
 constexpr size_t kApplySmem = (size_t)(kPairRows * kRotLd + kPairRows * kHalfLd) * sizeof(double);
 
 }  // namespace
@@ -597,7 +656,7 @@ size_t jacobi_scratch_bytes(int b) {
   const JacobiGeometry g = jacobi_geometry(b);
   const size_t tile = (size_t)kPairRows * kPairRows * sizeof(double);
   return align_up((size_t)g.pairs * g.chunks * tile, 256) + align_up((size_t)g.pairs * tile, 256) +
-         align_up((size_t)g.pairs * sizeof(int), 256);
+         align_up((size_t)g.pairs * sizeof(int), 256) + own_bytes(g);
 }
 
 galore_status_t jacobi_eigh(double* X, double* Vt, int b, void* scratch, int* counter, double tol, int max_sweeps,
@@ -614,9 +673,10 @@ galore_status_t jacobi_eigh(double* X, double* Vt, int b, void* scratch, int* co
   double* rot = (double*)p;
   p += align_up((size_t)g.pairs * tile, 256);
   int* flags = (int*)p;
+  p += align_up((size_t)g.pairs * sizeof(int), 256);
+  double* own = (double*)p;
 
   // per device, so set on every call rather than once per process
-  GALORE_CUDA_TRY(cudaFuncSetAttribute(jb_sweep_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSweepSmem));
   GALORE_CUDA_TRY(cudaFuncSetAttribute(jb_apply_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kApplySmem));
 
   // Slots leave the list as they converge (a sweep without a rotation), so every problem sees exactly
@@ -635,8 +695,8 @@ galore_status_t jacobi_eigh(double* X, double* Vt, int b, void* scratch, int* co
       // eight 4096 x 4096 at rank 1024 127.8 -> 125.1 ms).
       GALORE_TRY(launch_kernel(jb_gram_kernel, dim3(g.pairs, g.chunks, live.n), 128, 0, 1, true, st, (const double*)X, b, g.nblk, round,
                                g.chunks, part, live));
-      GALORE_TRY(launch_kernel(jb_sweep_kernel, dim3(g.pairs, live.n), kSweepThreads, kSweepSmem, 1, true, st, (const double*)part,
-                               g.chunks, b, g.nblk, round, tol, rot, flags, counter, live));
+      GALORE_TRY(launch_kernel(jb_sweep_kernel, dim3(g.pairs, live.n), kSweepThreads, 0, 1, true, st, (const double*)part,
+                               g.chunks, b, g.nblk, round, tol, own, rot, flags, counter, live));
       GALORE_TRY(launch_kernel(jb_apply_kernel, dim3(g.pairs, g.col_tiles, matrices * live.n), 256, kApplySmem, 1, true, st, X, Vt, b,
                                g.nblk, round, (const double*)rot, (const int*)flags, live, matrices));
     }

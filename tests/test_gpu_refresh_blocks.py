@@ -50,3 +50,29 @@ def test_grouped_layers_with_gradients_of_different_strides_match_single_refresh
         b.galore_refresh_projector(G)
         # every element is summed in the same order, alone or grouped: the same bits
         assert torch.equal(a.get_projector(), b.get_projector())
+
+
+# The eigen-solver carries products in single precision, scaled by the largest norm: a gradient times a power of two has the same
+# projector, whatever the power; few blocks of 32 rows and many, one matrix and a group
+@pytest.mark.parametrize("m,n,rank,over", [(96, 130, 24, 20), (200, 330, 30, 34), (512, 700, 96, 96), (700, 520, 150, 171)])
+@pytest.mark.parametrize("count", [1, 3])
+def test_projector_does_not_depend_on_the_scale_of_the_gradient(m, n, rank, over, count):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(m + over)
+    Gs = [0.1 * torch.randn(m, n, generator=gen, device="cuda") + torch.randn(m, 1, generator=gen, device="cuda") * torch.randn(1, n, generator=gen, device="cuda")
+          for _ in range(count)]
+    got = []
+    for e in (0, 30, -25):
+        layers = [gb.Layer(gb.make_config(m, n, rank, w_dtype="f32", g_dtype="f32", auto_refresh=False, refresh_oversample=over, seed=5 + i)) for i in range(count)]
+        scaled = [G * 2.0 ** e for G in Gs]
+        if count == 1:
+            layers[0].galore_refresh_projector(scaled[0])
+        else:
+            need = gb.galore_refresh_query_bytes(layers[0])
+            gb.galore_refresh_batch(layers, scaled, workspace=torch.empty(count * need, dtype=torch.uint8, device="cuda"))
+        assert max(l.device_status() for l in layers) == 0
+        got.append([l.get_projector().double() for l in layers])
+    for i in range(count):
+        for other in got[1:]:
+            # every operation scales exactly (no value leaves the normal range), up to columns' signs
+            assert float((got[0][i].abs() - other[i].abs()).abs().max()) <= 1e-6

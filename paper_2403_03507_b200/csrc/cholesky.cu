@@ -74,9 +74,20 @@ __device__ __forceinline__ void factor_block(S (*A)[kLdF], S (*X)[kLdF], S (*W)[
         r[j] = l;
         piv = fma(-l1, l1, next);
         if (lane == j) rdiag[o + j] = rs;
+        // the column, by way of shared memory: fewer instructions than a shuffle per value
+        S* const column = W[4 * (j & 1)];            // rows 0 and 4: 16-byte aligned for either type
+        if (lane < 16) column[i] = l;
+        __syncwarp();
+        constexpr int V = 16 / (int)sizeof(S);
 #pragma unroll
-        for (int k = 1; k < 16; ++k)
-          if (k > j) r[k] = fma(-l, __shfl_sync(0xffffffffu, l, k), r[k]);
+        for (int k0 = 0; k0 < 16; k0 += V) {
+          if (k0 + V - 1 <= j) continue;
+          alignas(16) S c[V];
+          *reinterpret_cast<uint4*>(c) = *reinterpret_cast<const uint4*>(column + k0);
+#pragma unroll
+          for (int k = 0; k < V; ++k)
+            if (k0 + k > j) r[k0 + k] = fma(-l, c[k], r[k0 + k]);
+        }
       }
       if (bad && lane == 0) atomicOr(status, GALORE_DEV_CHOLESKY);
       if (lane < 16) {

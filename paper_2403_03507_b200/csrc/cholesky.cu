@@ -26,7 +26,14 @@ namespace galore {
 namespace {
 
 constexpr int kB = kCholBlock;
-constexpr int kLdF = 65;                 // rows of the matrix being factored: walked by column as well
+// Rows of the matrix being factored, and of the factorisation's scratch: walked by column as well (65, 67: neighbouring rows on
+// distinct banks), and with doubles by the 8 x 4 fragments of the MMA (67: two of them on a bank at most).
+template <typename S>
+constexpr int kLdF = sizeof(S) == 8 ? 67 : 65;
+template <typename S>
+constexpr int kLdW = sizeof(S) == 8 ? 35 : 33;
+template <typename S>
+constexpr size_t kFactorBytes = (2 * 64 * kLdF<S> + 32 * kLdW<S>) * sizeof(S);
 constexpr int kThreads = 256;
 constexpr int kOwnTiles = 40;           // tiles of a step up to which every CTA forms its own L_i, L_j, T_Jj
 
@@ -40,20 +47,51 @@ template <typename S>
 constexpr int chol_smem(int tiles) { return tiles * kB * kLd<S> * (int)sizeof(S); }
 
 // ---- factor and inverse of one 64 x 64 block ---------------------------------------------------------
-// A (lower triangle, rows of kLdF) <- L, X (rows of kLdF) <- L^-1 with zeros above the diagonal; W: 32 x 33 of scratch,
-// rdiag: 64 values.  By sub-blocks of 16: one warp factors the diagonal sub-block with its rows in the lanes'
-// registers (no barrier inside), the rows below are solved one per thread, the rest is updated by all 256.
+// acc = the sum over 4 KS of P(i, k) Q(k, j), an 8 x 8 tile of a warp; p and q lead to the lane's elements of the first step
+template <int KS>
+__device__ __forceinline__ void warp_tile(double (&acc)[2], const double* p, int p_k, const double* q, int q_k) {
+  acc[0] = acc[1] = 0.0;
+#pragma unroll
+  for (int ks = 0; ks < KS; ++ks) dmma_m8n8k4(acc, p[4 * ks * p_k], q[4 * ks * q_k]);
+}
+
+// A (lower triangle, rows of kLdF) <- L, X (rows of kLdF) <- L^-1 with zeros above the diagonal; W: 32 rows of kLdW of
+// scratch, rdiag: 64 values.  By panels of 16 columns: one warp factors the panel, two rows in each lane's registers (no
+// barrier inside), another inverts the diagonal sub-block of the panel before, then all 256 threads update the rest.  In fp64 the
+// update and the products of the inverse run on the MMA unit: as scalar code they were bound by their loads from shared memory.
 template <typename S>
-__device__ __forceinline__ void factor_block(S (*A)[kLdF], S (*X)[kLdF], S (*W)[33], S* rdiag, int32_t* status) {
+__device__ __forceinline__ void factor_block(S (*A)[kLdF<S>], S (*X)[kLdF<S>], S (*W)[kLdW<S>], S* rdiag, int32_t* status) {
+  constexpr bool kMma = sizeof(S) == 8;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int g = lane >> 2, t = lane & 3;
+  for (int e = tid; e < kB * kB; e += kThreads) X[e >> 6][e & 63] = S(0);
+  // the inverse of the diagonal sub-block at o, a column per lane
+  auto invert = [&](int o) {
+    if (lane >= 16) return;
+    S s[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) s[k] = k == lane ? S(1) : S(0);
+#pragma unroll
+    for (int r = 0; r < 16; ++r) {
+      s[r] *= rdiag[o + r];
+#pragma unroll
+      for (int k = r + 1; k < 16; ++k) s[k] = fma(-A[o + k][o + r], s[r], s[k]);
+    }
+#pragma unroll
+    for (int k = 0; k < 16; ++k) X[o + k][o + lane] = s[k];
+  };
 #pragma unroll
   for (int p = 0; p < 4; ++p) {
     const int o = 16 * p;
     if (warp == 0) {
-      const int i = lane & 15;
-      S r[16];
+      // rows o + lane and o + 32 + lane of the panel
+      const bool one = o + lane < kB, two = o + 32 + lane < kB;
+      S r[16], q[16];
 #pragma unroll
-      for (int k = 0; k < 16; ++k) r[k] = k <= i ? A[o + i][o + k] : S(0);
+      for (int k = 0; k < 16; ++k) {
+        r[k] = one && k <= lane ? A[o + lane][o + k] : S(0);
+        q[k] = o < 32 && two ? A[o + 32 + lane][o + k] : S(0);
+      }
       // The chain from pivot to pivot is rsqrt, multiply, fma: every lane works out the next pivot for itself, from values
       // that were passed on before the root was known.  No branch in it, so that the updates fill the waits.
       bool bad = false;
@@ -69,14 +107,15 @@ __device__ __forceinline__ void factor_block(S (*A)[kLdF], S (*X)[kLdF], S (*W)[
           next = __shfl_sync(0xffffffffu, r[j + 1], j + 1);
         }
         const S rs = rsqrt(piv);
-        const S l = (i == j ? piv : (i > j ? r[j] : S(0))) * rs;
+        const S l = (lane == j ? piv : (lane > j ? r[j] : S(0))) * rs;
         const S l1 = raw * rs;
         r[j] = l;
+        q[j] *= rs;
         piv = fma(-l1, l1, next);
         if (lane == j) rdiag[o + j] = rs;
         // the column, by way of shared memory: fewer instructions than a shuffle per value
         S* const column = W[4 * (j & 1)];            // rows 0 and 4: 16-byte aligned for either type
-        if (lane < 16) column[i] = l;
+        if (lane < 16) column[lane] = l;
         __syncwarp();
         constexpr int V = 16 / (int)sizeof(S);
 #pragma unroll
@@ -86,126 +125,149 @@ __device__ __forceinline__ void factor_block(S (*A)[kLdF], S (*X)[kLdF], S (*W)[
           *reinterpret_cast<uint4*>(c) = *reinterpret_cast<const uint4*>(column + k0);
 #pragma unroll
           for (int k = 0; k < V; ++k)
-            if (k0 + k > j) r[k0 + k] = fma(-l, c[k], r[k0 + k]);
+            if (k0 + k > j) {
+              r[k0 + k] = fma(-l, c[k], r[k0 + k]);
+              if (o < 32) q[k0 + k] = fma(-q[j], c[k], q[k0 + k]);
+            }
         }
       }
       if (bad && lane == 0) atomicOr(status, GALORE_DEV_CHOLESKY);
-      if (lane < 16) {
 #pragma unroll
-        for (int k = 0; k < 16; ++k)
-          if (k <= i) A[o + i][o + k] = r[k];
+      for (int k = 0; k < 16; ++k) {
+        if (one && k <= lane) A[o + lane][o + k] = r[k];
+        if (o < 32 && two) A[o + 32 + lane][o + k] = q[k];
       }
+    } else if (warp == 1 && p > 0) {
+      invert(o - 16);
     }
     __syncthreads();
     if (p < 3) {
-      const int n = 48 - o;              // rows below
-      if (tid < n) {
-        S a[16];
-#pragma unroll
-        for (int k = 0; k < 16; ++k) a[k] = A[o + 16 + tid][o + k];
-#pragma unroll
-        for (int j = 0; j < 16; ++j) {
-          a[j] *= rdiag[o + j];
-#pragma unroll
-          for (int k = j + 1; k < 16; ++k) a[k] = fma(-a[j], A[o + k][o + j], a[k]);
+      // A[rest][rest] -= L L^T, lower part
+      if constexpr (kMma) {
+        const int n = 6 - 2 * p;           // tiles of 8
+        for (int tile = warp; tile < n * (n + 1) / 2; tile += kThreads / 32) {
+          int ti = 0, tj = tile;
+          while (tj > ti) tj -= ++ti;
+          double acc[2];
+          warp_tile<4>(acc, &A[o + 16 + 8 * ti + g][o + t], 1, &A[o + 16 + 8 * tj + g][o + t], 1);
+          double* dst = &A[o + 16 + 8 * ti + g][o + 16 + 8 * tj + 2 * t];
+          dst[0] -= acc[0];
+          dst[1] -= acc[1];
         }
-#pragma unroll
-        for (int k = 0; k < 16; ++k) A[o + 16 + tid][o + k] = a[k];
-      }
-      __syncthreads();
-      // A[rest][rest] -= L L^T, lower part: thread (ty, tx) owns rows ty + 16 u, columns tx + 16 v
-      constexpr int kMost = 3;
-      const int per = 3 - p, ty = tid >> 4, tx = tid & 15;
-      S acc[kMost][kMost];
-#pragma unroll
-      for (int u = 0; u < kMost; ++u)
-#pragma unroll
-        for (int v = 0; v < kMost; ++v) acc[u][v] = S(0);
-#pragma unroll
-      for (int k = 0; k < 16; ++k) {
-        S x[kMost], y[kMost];
+      } else {
+        // thread (ty, tx) owns rows ty + 16 u, columns tx + 16 v
+        constexpr int kMost = 3;
+        const int per = 3 - p, ty = tid >> 4, tx = tid & 15;
+        S acc[kMost][kMost];
 #pragma unroll
         for (int u = 0; u < kMost; ++u)
-          if (u < per) {
-            x[u] = A[o + 16 + ty + 16 * u][o + k];
-            y[u] = A[o + 16 + tx + 16 * u][o + k];
-          }
+#pragma unroll
+          for (int v = 0; v < kMost; ++v) acc[u][v] = S(0);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+          S x[kMost], y[kMost];
+#pragma unroll
+          for (int u = 0; u < kMost; ++u)
+            if (u < per) {
+              x[u] = A[o + 16 + ty + 16 * u][o + k];
+              y[u] = A[o + 16 + tx + 16 * u][o + k];
+            }
+#pragma unroll
+          for (int u = 0; u < kMost; ++u)
+#pragma unroll
+            for (int v = 0; v <= u; ++v)
+              if (u < per) acc[u][v] = fma(x[u], y[v], acc[u][v]);
+        }
 #pragma unroll
         for (int u = 0; u < kMost; ++u)
 #pragma unroll
           for (int v = 0; v <= u; ++v)
-            if (u < per) acc[u][v] = fma(x[u], y[v], acc[u][v]);
+            if (u < per && (u > v || ty >= tx)) A[o + 16 + ty + 16 * u][o + 16 + tx + 16 * v] -= acc[u][v];
       }
-#pragma unroll
-      for (int u = 0; u < kMost; ++u)
-#pragma unroll
-        for (int v = 0; v <= u; ++v)
-          if (u < per && (u > v || ty >= tx)) A[o + 16 + ty + 16 * u][o + 16 + tx + 16 * v] -= acc[u][v];
       __syncthreads();
     }
   }
-  // ---- the inverse: diagonal sub-blocks, then merged pairwise: T21 = -T22 (L21 T11)
-  for (int e = tid; e < kB * kB; e += kThreads) X[e >> 6][e & 63] = S(0);
+  // ---- the rest of the inverse: the sub-blocks merged pairwise, T21 = -T22 (L21 T11)
+  if (warp == 1) invert(48);
   __syncthreads();
-  if (tid < kB) {
-    const int o = tid & ~15, ci = tid & 15;
-    S s[16];
-#pragma unroll
-    for (int k = 0; k < 16; ++k) s[k] = k == ci ? S(1) : S(0);
-#pragma unroll
-    for (int r = 0; r < 16; ++r) {
-      s[r] *= rdiag[o + r];
-#pragma unroll
-      for (int k = r + 1; k < 16; ++k) s[k] = fma(-A[o + k][o + r], s[r], s[k]);
+  if constexpr (kMma) {
+    {                                    // two pairs of 16: a tile of 8 x 8 per warp
+      const int pair = warp >> 2, o = 32 * pair, i = 8 * ((warp >> 1) & 1), j = 8 * (warp & 1);
+      double acc[2];
+      warp_tile<4>(acc, &A[o + 16 + i + g][o + t], 1, &X[o + t][o + j + g], kLdF<S>);
+      W[16 * pair + i + g][j + 2 * t] = acc[0];
+      W[16 * pair + i + g][j + 2 * t + 1] = acc[1];
+      __syncthreads();
+      warp_tile<4>(acc, &X[o + 16 + i + g][o + 16 + t], 1, &W[16 * pair + t][j + g], kLdW<S>);
+      X[o + 16 + i + g][o + j + 2 * t] = -acc[0];
+      X[o + 16 + i + g][o + j + 2 * t + 1] = -acc[1];
+      __syncthreads();
     }
+    {                                    // the pair of 32: two tiles per warp, side by side
+      const int i = 8 * (warp >> 1), j = 16 * (warp & 1);
+      double acc[2][2];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) X[o + k][tid] = s[k];
-  }
-  __syncthreads();
-  {                                      // two pairs of 16: thread (pair, r, c-pair)
-    const int pair = tid >> 7, o = 32 * pair, r = (tid >> 3) & 15, c = (tid & 7) * 2;
-    S w0 = S(0), w1 = S(0);
+      for (int v = 0; v < 2; ++v) warp_tile<8>(acc[v], &A[32 + i + g][t], 1, &X[t][j + 8 * v + g], kLdF<S>);
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      const S l = A[o + 16 + r][o + k];
-      w0 = fma(l, X[o + k][o + c], w0);
-      w1 = fma(l, X[o + k][o + c + 1], w1);
+      for (int v = 0; v < 2; ++v) {
+        W[i + g][j + 8 * v + 2 * t] = acc[v][0];
+        W[i + g][j + 8 * v + 2 * t + 1] = acc[v][1];
+      }
+      __syncthreads();
+#pragma unroll
+      for (int v = 0; v < 2; ++v) warp_tile<8>(acc[v], &X[32 + i + g][32 + t], 1, &W[t][j + 8 * v + g], kLdW<S>);
+#pragma unroll
+      for (int v = 0; v < 2; ++v) {
+        X[32 + i + g][j + 8 * v + 2 * t] = -acc[v][0];
+        X[32 + i + g][j + 8 * v + 2 * t + 1] = -acc[v][1];
+      }
     }
-    W[16 * pair + r][c] = w0;
-    W[16 * pair + r][c + 1] = w1;
-    __syncthreads();
-    S t0 = S(0), t1 = S(0);
+  } else {
+    {                                    // two pairs of 16: thread (pair, r, c-pair)
+      const int pair = tid >> 7, o = 32 * pair, r = (tid >> 3) & 15, c = (tid & 7) * 2;
+      S w0 = S(0), w1 = S(0);
 #pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      const S x = X[o + 16 + r][o + 16 + k];
-      t0 = fma(-x, W[16 * pair + k][c], t0);
-      t1 = fma(-x, W[16 * pair + k][c + 1], t1);
+      for (int k = 0; k < 16; ++k) {
+        const S l = A[o + 16 + r][o + k];
+        w0 = fma(l, X[o + k][o + c], w0);
+        w1 = fma(l, X[o + k][o + c + 1], w1);
+      }
+      W[16 * pair + r][c] = w0;
+      W[16 * pair + r][c + 1] = w1;
+      __syncthreads();
+      S t0 = S(0), t1 = S(0);
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        const S x = X[o + 16 + r][o + 16 + k];
+        t0 = fma(-x, W[16 * pair + k][c], t0);
+        t1 = fma(-x, W[16 * pair + k][c + 1], t1);
+      }
+      X[o + 16 + r][o + c] = t0;
+      X[o + 16 + r][o + c + 1] = t1;
+      __syncthreads();
     }
-    X[o + 16 + r][o + c] = t0;
-    X[o + 16 + r][o + c + 1] = t1;
-    __syncthreads();
-  }
-  {                                      // the pair of 32: thread owns rows ty, ty + 16 and columns tx, tx + 16
-    const int ty = tid >> 4, tx = tid & 15;
-    S w[2][2] = {{S(0), S(0)}, {S(0), S(0)}};
+    {                                    // the pair of 32: thread owns rows ty, ty + 16 and columns tx, tx + 16
+      const int ty = tid >> 4, tx = tid & 15;
+      S w[2][2] = {{S(0), S(0)}, {S(0), S(0)}};
 #pragma unroll 8
-    for (int k = 0; k < 32; ++k) {
-      const S a0 = A[32 + ty][k], a1 = A[48 + ty][k], x0 = X[k][tx], x1 = X[k][16 + tx];
-      w[0][0] = fma(a0, x0, w[0][0]); w[0][1] = fma(a0, x1, w[0][1]);
-      w[1][0] = fma(a1, x0, w[1][0]); w[1][1] = fma(a1, x1, w[1][1]);
-    }
-    W[ty][tx] = w[0][0]; W[ty][16 + tx] = w[0][1];
-    W[16 + ty][tx] = w[1][0]; W[16 + ty][16 + tx] = w[1][1];
-    __syncthreads();
-    S t[2][2] = {{S(0), S(0)}, {S(0), S(0)}};
+      for (int k = 0; k < 32; ++k) {
+        const S a0 = A[32 + ty][k], a1 = A[48 + ty][k], x0 = X[k][tx], x1 = X[k][16 + tx];
+        w[0][0] = fma(a0, x0, w[0][0]); w[0][1] = fma(a0, x1, w[0][1]);
+        w[1][0] = fma(a1, x0, w[1][0]); w[1][1] = fma(a1, x1, w[1][1]);
+      }
+      W[ty][tx] = w[0][0]; W[ty][16 + tx] = w[0][1];
+      W[16 + ty][tx] = w[1][0]; W[16 + ty][16 + tx] = w[1][1];
+      __syncthreads();
+      S u[2][2] = {{S(0), S(0)}, {S(0), S(0)}};
 #pragma unroll 8
-    for (int k = 0; k < 32; ++k) {
-      const S a0 = X[32 + ty][32 + k], a1 = X[48 + ty][32 + k], x0 = W[k][tx], x1 = W[k][16 + tx];
-      t[0][0] = fma(-a0, x0, t[0][0]); t[0][1] = fma(-a0, x1, t[0][1]);
-      t[1][0] = fma(-a1, x0, t[1][0]); t[1][1] = fma(-a1, x1, t[1][1]);
+      for (int k = 0; k < 32; ++k) {
+        const S a0 = X[32 + ty][32 + k], a1 = X[48 + ty][32 + k], x0 = W[k][tx], x1 = W[k][16 + tx];
+        u[0][0] = fma(-a0, x0, u[0][0]); u[0][1] = fma(-a0, x1, u[0][1]);
+        u[1][0] = fma(-a1, x0, u[1][0]); u[1][1] = fma(-a1, x1, u[1][1]);
+      }
+      X[32 + ty][tx] = u[0][0]; X[32 + ty][16 + tx] = u[0][1];
+      X[48 + ty][tx] = u[1][0]; X[48 + ty][16 + tx] = u[1][1];
     }
-    X[32 + ty][tx] = t[0][0]; X[32 + ty][16 + tx] = t[0][1];
-    X[48 + ty][tx] = t[1][0]; X[48 + ty][16 + tx] = t[1][1];
   }
   __syncthreads();
 }
@@ -452,9 +514,9 @@ __global__ void __launch_bounds__(kThreads) chol_update_kernel(const CholArgs<S>
     else product(acc, Q, P);          // (B_ij)^T
   }
   if (i == col + 1 && j == i) {          // the next diagonal block: factored at once, its inverse goes to its slab
-    S(*A)[kLdF] = reinterpret_cast<S(*)[kLdF]>(chol_raw);
-    S(*X)[kLdF] = A + kB;
-    S(*W)[33] = reinterpret_cast<S(*)[33]>(X + kB);
+    S(*A)[kLdF<S>] = reinterpret_cast<S(*)[kLdF<S>]>(chol_raw);
+    S(*X)[kLdF<S>] = A + kB;
+    S(*W)[kLdW<S>] = reinterpret_cast<S(*)[kLdW<S>]>(X + kB);
     __syncthreads();
 #pragma unroll
     for (int u = 0; u < 4; ++u)
@@ -485,9 +547,9 @@ __global__ void __launch_bounds__(kThreads) chol_update_kernel(const CholArgs<S>
 template <typename S>
 galore_status_t cholesky_inverse_factor(S* C, S* T, S* B, S* slabs, int b, int32_t* flags, const SlotList& slots, cudaStream_t st) {
   if (b < 1 || slots.n < 1) return GALORE_OK;
-  static_assert((2 * kB * kLdF + 32 * 33) * (int)sizeof(S) <= chol_smem<S>(3), "the factorisation uses the tiles' space");
+  static_assert(kFactorBytes<S> <= chol_smem<S>(3), "the factorisation uses the tiles' space");
   static std::atomic<uint64_t> configured[3] = {};
-  const int own_smem = chol_smem<S>(3), tile_smem = std::max(chol_smem<S>(2), (2 * kB * kLdF + 32 * 33) * (int)sizeof(S));
+  const int own_smem = chol_smem<S>(3), tile_smem = std::max(chol_smem<S>(2), (int)kFactorBytes<S>);
   GALORE_TRY(allow_smem(configured[0], (const void*)chol_update_kernel<S, true>, own_smem));
   GALORE_TRY(allow_smem(configured[1], (const void*)chol_update_kernel<S, false>, tile_smem));
   GALORE_TRY(allow_smem(configured[2], (const void*)chol_panel_kernel<S>, tile_smem));

@@ -7,11 +7,14 @@
 // sums: fmaf over k, slice after slice.  A bf16 W or 8-bit moments round far above the difference, and Adafactor's
 // factored second moment does not vanish with a single r: there the split products carry the projection.
 //
-// What bounds it: the FMA rate of a 128 x 128 tile of 256 threads for large matrices; for small ones the latency of the K loop,
-// 16 k at a time with the next ones on their way.
+// What bounds it: the FMA rate of a 128 x 128 tile of 256 threads for large matrices; for small ones latency.  fp32 operands whose
+// rows lie along the tile on 16-byte boundaries are copied to shared memory asynchronously, several steps of 16 k ahead (a small
+// result's whole slice at once: five waits for memory become one).  512 x 1376 at rank 128: 25.0 -> 20.1 us a step; 2048 x 5461 at
+// rank 512: 552 -> 316 us (36 TFLOP/s).  Others go through registers, one step ahead: copies of four bytes were slower.
 #include "gemm_fma.cuh"
 
 #include <algorithm>
+#include <type_traits>
 
 #include "launch.cuh"
 #include "tc_ptx.cuh"
@@ -22,14 +25,20 @@ namespace {
 
 constexpr int kBK = 16;
 constexpr int kThreads = 256;
+// steps of 16 k in shared memory: 43.5 KiB of a small tile's, five CTAs an SM; 69.6 KiB of a large one's
+constexpr int stages(bool async, int bm) { return !async ? 1 : (bm == 64 ? 5 : 4); }
+constexpr int smem_bytes(bool async, int bm, int bn) { return stages(async, bm) * kBK * (bm + bn + 8) * 4; }
 
 // BM x BN tile, TM x TN elements a thread in groups of four
 template <typename TA, typename TB, int BM, int BN, int TM, int TN, int CAP>
 __global__ void __launch_bounds__(kThreads) gemm_fma_kernel(const __grid_constant__ FmaArgs<CAP> g) {
   static_assert((BM / TM) * (BN / TN) == kThreads, "one micro-tile a thread");
   constexpr int LA = BM * kBK / kThreads, LB = BN * kBK / kThreads;      // elements of a tile each thread fetches
-  __shared__ float As[kBK][BM + 4];
-  __shared__ float Bs[kBK][BN + 4];
+  constexpr bool kAsync = sizeof(TA) == 4 && sizeof(TB) == 4;
+  constexpr int kStages = stages(kAsync, BM);
+  extern __shared__ __align__(16) float fma_smem[];
+  float(*const As)[kBK][BM + 4] = reinterpret_cast<float(*)[kBK][BM + 4]>(fma_smem);
+  float(*const Bs)[kBK][BN + 4] = reinterpret_cast<float(*)[kBK][BN + 4]>(fma_smem + kStages * kBK * (BM + 4));
   grid_dependency_wait();
   grid_launch_dependents();
   GroupCursor cursor;
@@ -56,44 +65,7 @@ __global__ void __launch_bounds__(kThreads) gemm_fma_kernel(const __grid_constan
 #pragma unroll
     for (int v = 0; v < TN; ++v) acc[u][v] = 0.f;
 
-  float ra[LA], rb[LB];
-  auto fetch = [&](int k0) {
-#pragma unroll
-    for (int e = 0; e < LA; ++e) {
-      const int idx = tid + e * kThreads;
-      const int i = a_kfast ? idx / kBK : idx % BM;
-      const int k = a_kfast ? idx % kBK : idx / BM;
-      const int gi = m0 + i, gk = k0 + k;
-      ra[e] = (gi < M && gk < k_end) ? cvt<float>(A[(int64_t)gi * sAi + (int64_t)gk * sAk]) : 0.f;
-    }
-#pragma unroll
-    for (int e = 0; e < LB; ++e) {
-      const int idx = tid + e * kThreads;
-      const int j = b_kfast ? idx / kBK : idx % BN;
-      const int k = b_kfast ? idx % kBK : idx / BN;
-      const int gj = n0 + j, gk = k0 + k;
-      rb[e] = (gj < N && gk < k_end) ? cvt<float>(B[(int64_t)gk * sBk + (int64_t)gj * sBj]) : 0.f;
-    }
-  };
-  auto stash = [&]() {
-#pragma unroll
-    for (int e = 0; e < LA; ++e) {
-      const int idx = tid + e * kThreads;
-      As[a_kfast ? idx % kBK : idx / BM][a_kfast ? idx / kBK : idx % BM] = ra[e];
-    }
-#pragma unroll
-    for (int e = 0; e < LB; ++e) {
-      const int idx = tid + e * kThreads;
-      Bs[b_kfast ? idx % kBK : idx / BN][b_kfast ? idx / kBK : idx % BN] = rb[e];
-    }
-  };
-
-  if (k_begin < k_end) fetch(k_begin);
-  for (int k0 = k_begin; k0 < k_end; k0 += kBK) {
-    __syncthreads();
-    stash();
-    __syncthreads();
-    if (k0 + kBK < k_end) fetch(k0 + kBK);
+  auto multiply = [&](const float (*As)[BM + 4], const float (*Bs)[BN + 4]) {
 #pragma unroll
     for (int k = 0; k < kBK; ++k) {
       float a[TM], b[TN];
@@ -105,6 +77,77 @@ __global__ void __launch_bounds__(kThreads) gemm_fma_kernel(const __grid_constan
       for (int u = 0; u < TM; ++u)
 #pragma unroll
         for (int v = 0; v < TN; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
+    }
+  };
+  bool async = false;
+  if constexpr (kAsync)
+    async = sAi == 1 && sBj == 1 && (((uintptr_t)A | (uintptr_t)B) & 15) == 0 && ((sAk | sBk) & 3) == 0;
+  if (async) {
+    // 16 k of one operand in runs of four; zeros outside the matrix
+    auto copy = [&]<int BX, class Tile>(std::integral_constant<int, BX>, Tile dst, const float* X, int64_t s_k, int x0, int X_size, int k0) {
+#pragma unroll
+      for (int e = 0; e < BX * kBK / 4 / kThreads; ++e) {
+        const int idx = tid + e * kThreads, x = idx % (BX / 4) * 4, k = idx / (BX / 4);
+        const int valid = k0 + k < k_end ? min(4, max(0, X_size - x0 - x)) : 0;
+        const float* src = valid ? X + (int64_t)(k0 + k) * s_k + x0 + x : X;
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(&dst[k][x])), "l"(src), "r"(valid * 4) : "memory");
+      }
+    };
+    const int steps = (k_end - k_begin + kBK - 1) / kBK;
+    auto request = [&](int step) {                    // (an empty group behind the last step: the count of groups stays)
+      if (step < steps) {
+        copy(std::integral_constant<int, BM>(), As[step % kStages], (const float*)A, sAk, m0, M, k_begin + step * kBK);
+        copy(std::integral_constant<int, BN>(), Bs[step % kStages], (const float*)B, sBk, n0, N, k_begin + step * kBK);
+      }
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+#pragma unroll
+    for (int step = 0; step < kStages - 1; ++step) request(step);
+    for (int step = 0; step < steps; ++step) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
+      __syncthreads();                                // the step's copies of all threads are in, the stage to be filled has been read
+      request(step + kStages - 1);
+      multiply(As[step % kStages], Bs[step % kStages]);
+    }
+  } else {
+    float ra[LA], rb[LB];
+    auto fetch = [&](int k0) {
+#pragma unroll
+      for (int e = 0; e < LA; ++e) {
+        const int idx = tid + e * kThreads;
+        const int i = a_kfast ? idx / kBK : idx % BM;
+        const int k = a_kfast ? idx % kBK : idx / BM;
+        const int gi = m0 + i, gk = k0 + k;
+        ra[e] = (gi < M && gk < k_end) ? cvt<float>(A[(int64_t)gi * sAi + (int64_t)gk * sAk]) : 0.f;
+      }
+#pragma unroll
+      for (int e = 0; e < LB; ++e) {
+        const int idx = tid + e * kThreads;
+        const int j = b_kfast ? idx / kBK : idx % BN;
+        const int k = b_kfast ? idx % kBK : idx / BN;
+        const int gj = n0 + j, gk = k0 + k;
+        rb[e] = (gj < N && gk < k_end) ? cvt<float>(B[(int64_t)gk * sBk + (int64_t)gj * sBj]) : 0.f;
+      }
+    };
+    auto stash = [&]() {
+#pragma unroll
+      for (int e = 0; e < LA; ++e) {
+        const int idx = tid + e * kThreads;
+        As[0][a_kfast ? idx % kBK : idx / BM][a_kfast ? idx / kBK : idx % BM] = ra[e];
+      }
+#pragma unroll
+      for (int e = 0; e < LB; ++e) {
+        const int idx = tid + e * kThreads;
+        Bs[0][b_kfast ? idx % kBK : idx / BN][b_kfast ? idx / kBK : idx % BN] = rb[e];
+      }
+    };
+    if (k_begin < k_end) fetch(k_begin);
+    for (int k0 = k_begin; k0 < k_end; k0 += kBK) {
+      __syncthreads();
+      stash();
+      __syncthreads();
+      if (k0 + kBK < k_end) fetch(k0 + kBK);
+      multiply(As[0], Bs[0]);
     }
   }
   // a thread's columns come in runs of four: one 16-byte store where the rows allow it
@@ -132,19 +175,26 @@ __global__ void __launch_bounds__(kThreads) gemm_fma_kernel(const __grid_constan
 // Results below 96 tiles of 128 x 128 are cut into 64 x 64.
 bool small_result(int64_t M, int64_t N) { return M * N < (int64_t)128 * 128 * 96; }
 
+template <typename TA, typename TB, int BM, int TM, int CAP>
+galore_status_t launch_tiles(const FmaArgs<CAP>& g, bool early, cudaStream_t st) {
+  constexpr int smem = smem_bytes(sizeof(TA) == 4 && sizeof(TB) == 4, BM, BM);
+  auto kern = gemm_fma_kernel<TA, TB, BM, BM, TM, TM, CAP>;
+  static std::atomic<uint64_t> configured{0};
+  GALORE_TRY(allow_smem(configured, (const void*)kern, smem));
+  return launch_kernel(kern, dim3((unsigned)g.unit_end[g.count - 1]), kThreads, smem, 1, early, st, g);
+}
+
 template <typename TA, typename TB>
 galore_status_t launch_typed(const FmaGroup& g, bool early, cudaStream_t st) {
-  if (g.count > 1)
-    return launch_kernel(gemm_fma_kernel<TA, TB, 128, 128, 8, 8, kFmaGroup>, dim3((unsigned)g.unit_end[g.count - 1]), kThreads, 0, 1, early, st, g);
+  if (g.count > 1) return launch_tiles<TA, TB, 128, 8, kFmaGroup>(g, early, st);
   FmaArgs<1> one;
   const FmaProblem& p = one.p[0] = g.p[0];
   one.count = 1;
   const bool small = small_result(p.M, p.N);
   const int64_t t = small ? 64 : 128;
   one.unit_end[0] = (int)(ceil_div(p.M, t) * ceil_div(p.N, t) * p.splits);
-  const dim3 grid((unsigned)one.unit_end[0]);
-  if (small) return launch_kernel(gemm_fma_kernel<TA, TB, 64, 64, 4, 4, 1>, grid, kThreads, 0, 1, early, st, one);
-  return launch_kernel(gemm_fma_kernel<TA, TB, 128, 128, 8, 8, 1>, grid, kThreads, 0, 1, early, st, one);
+  if (small) return launch_tiles<TA, TB, 64, 4, 1>(one, early, st);
+  return launch_tiles<TA, TB, 128, 8, 1>(one, early, st);
 }
 
 int chunk_of(int64_t K, int slices) { return (int)(std::max<int64_t>(1, ceil_div(ceil_div(K, std::max(1, slices)), kBK)) * kBK); }

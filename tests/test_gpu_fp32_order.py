@@ -92,3 +92,26 @@ def test_static_step_sums_in_the_same_order(m, n, r, pad):
     M, V = torch.zeros(layer.state_shape, device="cuda"), torch.zeros(layer.state_shape, device="cuda")
     assert gb.galore_step_static(P, M, V, W, G, 1e-2, completed_steps=0) == 0
     assert torch.equal(M, _expected(layer, P, G, _slices(*layer.state_shape, min(m, n))))
+
+
+# Operands that are copied to shared memory ahead (rows along the tile, 16-byte boundaries) and those that are not give the same
+# sums: tiles of 64 and of 128, ragged ends, fewer steps of 16 than stages and many, slices
+@pytest.mark.parametrize("m,n,r", [(5, 9, 4), (16, 70, 12), (40, 200, 36), (300, 515, 64), (513, 1377, 128), (1100, 3001, 260)])
+def test_copied_operands_give_the_bits_of_loaded_ones(m, n, r):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(m + n)
+    P = torch.linalg.qr(torch.randn(m, r, generator=gen, device="cuda"))[0]
+    G = torch.randn(m, n, generator=gen, device="cuda")
+    got = []
+    for pitch in ((n + 3) // 4 * 4, (n + 3) // 4 * 4 + 1):       # rows of G on 16-byte boundaries, and off them
+        layer = gb.Layer(gb.make_config(m, n, r, w_dtype="f32", g_dtype="f32", auto_refresh=False, side=gb.SIDE_LEFT))
+        layer.set_projector(P)
+        g = torch.full((m, pitch), float("nan"), device="cuda")[:, :n]
+        g.copy_(G)
+        layer.galore_step(torch.zeros(m, n, device="cuda"), g, 1e-2)
+        assert layer.device_status() == 0
+        got.append(layer.get_moments())
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+    R = P.double().T @ G.double()
+    # a chain of m fused multiply-adds: at most 2^-24 sqrt(m) of the root mean square of R in the norm
+    assert float((got[0][0].double() / 0.1 - R).norm() / R.norm()) <= 2 ** -24 * (8 + m ** 0.5)

@@ -157,7 +157,7 @@ __global__ void __launch_bounds__(256) align_rows_kernel(const __nv_bfloat16* sr
 galore_status_t launch_align_rows(const void* src, int64_t ld_src, void* dst, int64_t ld_dst, int rows, int cols, cudaStream_t st) {
   const int64_t units = (int64_t)rows * ceil_div(cols, 1024);
   if (units >= ((int64_t)1 << 30)) return GALORE_ERR_SHAPE;
-  return launch_kernel(align_rows_kernel, dim3((unsigned)std::min<int64_t>(ceil_div(units, 8), 148 * 8)), 256, 0, 1, true, st,
+  return launch_kernel(align_rows_kernel, dim3((unsigned)ceil_div(units, 8)), 256, 0, 1, true, st,
                        (const __nv_bfloat16*)src, ld_src, (__nv_bfloat16*)dst, ld_dst, rows, cols);
 }
 

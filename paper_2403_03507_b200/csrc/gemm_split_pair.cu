@@ -304,15 +304,19 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_pair_kernel(const __gr
         const bool closing = corrections_due(kb, blocks);
 #pragma unroll
         for (int c = 0; c < kCols; c += 8) {
-          uint32_t x[8], y[8] = {};
+          uint32_t x[8], y[8];
           tmem_ld_32x8(t + (uint32_t)c, x);
           if (closing) tmem_ld_32x8(t + (uint32_t)(kTile + c), y);
           tmem_ld_wait();
+          if (closing) {
+            float v[8];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            asm volatile("" : "+r"(x[j]), "+r"(y[j]));          // not read before the wait
-            sum[c + j] += __uint_as_float(x[j]) + __uint_as_float(y[j]);
+            for (int j = 0; j < 8; ++j) v[j] = __uint_as_float(x[j]);
+            add_acc(v, y);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) x[j] = __float_as_uint(v[j]);
           }
+          add_acc(sum + c, x);
         }
         tc_fence_before();
         __syncwarp();

@@ -708,11 +708,7 @@ gemm_tc_kernel(const __grid_constant__ TcArgs<CAP> g) {
             uint32_t v[16];
             tmem_ld_32x16(t + (uint32_t)c, v);
             tmem_ld_wait();
-#pragma unroll
-            for (int j = 0; j < 16; ++j) {
-              asm volatile("" : "+r"(v[j]));          // not read before the wait
-              sum[c + j] += __uint_as_float(v[j]);
-            }
+            add_acc(sum + c, v);
           }
           release_acc();
         }

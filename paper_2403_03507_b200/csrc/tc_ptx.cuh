@@ -218,6 +218,21 @@ __device__ __forceinline__ void tmem_ld_32x8(uint32_t taddr, uint32_t (&v)[8]) {
                : "r"(taddr)
                : "memory");
 }
+// sum[j] += acc[j], each rounded to nearest: two in an instruction
+template <int N>
+__device__ __forceinline__ void add_acc(float* sum, uint32_t (&acc)[N]) {
+  static_assert(N % 2 == 0, "pairs");
+#pragma unroll
+  for (int j = 0; j < N; j += 2) {
+    asm volatile(                                     // volatile: not before the wait for tensor memory
+        "{\n\t.reg .b64 s, a;\n\t"
+        "mov.b64 s, {%0, %1};\n\tmov.b64 a, {%2, %3};\n\t"
+        "add.rn.f32x2 s, s, a;\n\t"
+        "mov.b64 {%0, %1}, s;\n\t}"
+        : "+f"(sum[j]), "+f"(sum[j + 1])
+        : "r"(acc[j]), "r"(acc[j + 1]));
+  }
+}
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 }  // namespace galore

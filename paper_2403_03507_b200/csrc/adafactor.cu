@@ -3,7 +3,8 @@
 //   U = R / sqrt(v_row v_col^T / mean(v_row)),  U <- U / max(1, rms(U) / d)
 //   M <- beta1 M + (1 - beta1) U,  N = M
 // Four passes, each a plain streaming kernel, every reduction in a fixed order (run-to-run identical):
-//   1. sums the split-K partials of R and leaves per-tile row and column sums of R^2,
+//   1. sums the split-K partials of R and leaves per-tile row and column sums of R^2 (the projection of a batch on the tensor
+//      path leaves them itself: the pass is left out),
 //   2. folds those into v_row, v_col (one thread per entry), with 1 / sqrt of each and the blocks' sums of v_row,
 //   3. sum of (R / sqrt(v_row v_col^T))^2 over a fixed set of parts, one per warp,
 //   4. the clipped update, the momentum and N; the scalar sqrt(mean(v_row)) that pass 2 cannot know yet enters here.
@@ -45,9 +46,11 @@ struct AfLayout {
   double* row_sums;  // sums of v_row over blocks of 256 entries
   int tile_rows, tiles_r, tiles_c;
 };
-__host__ __device__ inline AfLayout af_layout(float* scratch, int rows, int cols) {
+__host__ __device__ inline AfLayout af_layout(const AdafactorItem& it) {
+  const int rows = it.rows, cols = it.cols;
+  float* const scratch = it.scratch;
   AfLayout a;
-  a.tile_rows = af_tile_rows(rows, cols);
+  a.tile_rows = it.squares_ready ? kAfProjectionRows : af_tile_rows(rows, cols);
   a.tiles_r = (rows + a.tile_rows - 1) / a.tile_rows;
   a.tiles_c = (cols + kAfTileCols - 1) / kAfTileCols;
   a.sums = reinterpret_cast<double*>(scratch);
@@ -90,7 +93,7 @@ __global__ void __launch_bounds__(kAfTileCols) af_stats_kernel(const __grid_cons
   __shared__ float cs[kAfTileCols / 32][kAfTileCols];
   int tile;
   const AdafactorItem& it = g.item[find_item<CAP>(g.tile_end, g.count, blockIdx.x, tile)];
-  const AfLayout a = af_layout(it.scratch, it.rows, it.cols);
+  const AfLayout a = af_layout(it);
   const int tile_r = tile / a.tiles_c, tile_c = tile % a.tiles_c;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int r0 = tile_r * a.tile_rows, c0 = tile_c * kAfTileCols + 4 * lane;
@@ -180,7 +183,7 @@ __global__ void __launch_bounds__(256) af_vectors_kernel(const __grid_constant__
   const int which = find_item<CAP>(g.vec_end, g.count, blockIdx.x, blk);
   const AdafactorItem& it = g.item[which];
   const float beta2t = g.beta2t[which];
-  const AfLayout a = af_layout(it.scratch, it.rows, it.cols);
+  const AfLayout a = af_layout(it);
   const int row_blocks = (it.rows + 255) / 256;
   if (blk < row_blocks) {
     const int i = blk * 256 + threadIdx.x;
@@ -227,7 +230,7 @@ __global__ void __launch_bounds__(kRmsThreads) af_rms_kernel(const __grid_consta
   grid_dependency_wait();
   grid_launch_dependents();
   const AdafactorItem& it = g.item[blockIdx.y];
-  const AfLayout a = af_layout(it.scratch, it.rows, it.cols);
+  const AfLayout a = af_layout(it);
   const AfRowWalk w = af_walk(it, false);
   const int lane = threadIdx.x & 31;
   const int part = (int)(blockIdx.x * (kRmsThreads / 32) + (threadIdx.x >> 5));
@@ -292,7 +295,7 @@ __global__ void __launch_bounds__(256) af_update_kernel(const __grid_constant__ 
   grid_launch_dependents();
   __shared__ double red[8];
   const AdafactorItem& it = g.item[blockIdx.y];
-  const AfLayout a = af_layout(it.scratch, it.rows, it.cols);
+  const AfLayout a = af_layout(it);
   double s = 0.0, sr = 0.0;
   for (int i = threadIdx.x; i < kAfSumBlocks; i += 256) s += a.sums[i];
   for (int i = threadIdx.x; i < (it.rows + 255) / 256; i += 256) sr += a.row_sums[i];
@@ -336,8 +339,18 @@ __global__ void __launch_bounds__(256) af_update_kernel(const __grid_constant__ 
 }  // namespace
 
 size_t adafactor_scratch_bytes(int64_t rows, int64_t cols) {
-  const int64_t tiles_r = ceil_div(rows, af_tile_rows(rows, cols)), tiles_c = ceil_div(cols, kAfTileCols);
+  const int least = rows <= kAfProjectionTallest ? std::min(af_tile_rows(rows, cols), kAfProjectionRows) : af_tile_rows(rows, cols);
+  const int64_t tiles_r = ceil_div(rows, least), tiles_c = ceil_div(cols, kAfTileCols);
   return align_up((size_t)(2 * (kAfSumBlocks + 8 + ceil_div(rows, 256) * 2) + rows * tiles_c + tiles_r * cols + rows + cols + 16) * sizeof(float), 256);
+}
+
+bool adafactor_squares(const AdafactorItem& item, AdafactorSquares* out) {
+  if (item.rows > kAfProjectionTallest) return false;
+  AdafactorItem it = item;
+  it.squares_ready = true;
+  const AfLayout a = af_layout(it);
+  *out = AdafactorSquares{a.rowpart, a.colpart, a.tiles_c};
+  return true;
 }
 
 galore_status_t adafactor_group_add(AdafactorGroup& g, const AdafactorItem& it) {
@@ -347,7 +360,8 @@ galore_status_t adafactor_group_add(AdafactorGroup& g, const AdafactorItem& it) 
   const int i = g.count;
   g.item[i] = it;
   g.beta2t[i] = (float)(1.0 - pow(it.t, -kAdafactorDecay));
-  const int tiles = (int)(ceil_div(it.rows, af_tile_rows(it.rows, it.cols)) * ceil_div(it.cols, kAfTileCols));
+  if (it.squares_ready && (it.splits != 1 || it.split.src)) return GALORE_ERR_INVALID_ARG;      // the pass adds slices and splits P too
+  const int tiles = it.squares_ready ? 0 : (int)(ceil_div(it.rows, af_tile_rows(it.rows, it.cols)) * ceil_div(it.cols, kAfTileCols));
   const int blocks = (int)(ceil_div(it.rows, 256) + ceil_div(it.cols, 256));
   g.tile_end[i] = (i ? g.tile_end[i - 1] : 0) + tiles;
   g.vec_end[i] = (i ? g.vec_end[i - 1] : 0) + blocks;
@@ -358,7 +372,8 @@ galore_status_t adafactor_group_add(AdafactorGroup& g, const AdafactorItem& it) 
 template <int PL, int CAP>
 static galore_status_t launch_passes(const AdafactorArgs<CAP>& g, bool early, cudaStream_t st) {
   const int n = g.count;
-  GALORE_TRY(launch_kernel(af_stats_kernel<CAP>, dim3((unsigned)g.tile_end[n - 1]), kAfTileCols, 0, 1, early, st, g));
+  if (g.tile_end[n - 1] > 0)      // (an item whose sums are ready has no tiles)
+    GALORE_TRY(launch_kernel(af_stats_kernel<CAP>, dim3((unsigned)g.tile_end[n - 1]), kAfTileCols, 0, 1, early, st, g));
   GALORE_TRY(launch_kernel(af_vectors_kernel<CAP>, dim3((unsigned)g.vec_end[n - 1]), 256, 0, 1, early, st, g));
   const unsigned parts = (unsigned)ceil_div(kAfSumBlocks, kRmsThreads / 32);
   GALORE_TRY(launch_kernel(af_rms_kernel<CAP>, dim3(parts, (unsigned)n), kRmsThreads, 0, 1, early, st, g));

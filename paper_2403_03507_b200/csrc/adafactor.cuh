@@ -35,7 +35,17 @@ struct AdafactorItem {
   float beta1;
   double t;                // completed steps + 1
   float* scratch;          // adafactor_scratch_bytes(rows, cols) bytes
+  bool squares_ready;      // the projection has left the sums of R^2 where adafactor_squares() says
 };
+// Where a projection may leave the sums of R^2: over stretches of kAfTileCols columns (rows x tiles) and of kAfProjectionRows rows (one row
+// of sums for each).  False for an R so tall that one thread would have too many of them to add up for a column: steps of four layers
+// of 16384 x 512 at rank 64 with the pass over R / without it 195 / 172 us, of 32768 x 512 356 / 368, of 65536 x 512 650 / 681.
+constexpr int kAfProjectionRows = 64, kAfProjectionTallest = 256 * kAfProjectionRows;
+struct AdafactorSquares {
+  float *row, *col;
+  int tiles;
+};
+bool adafactor_squares(const AdafactorItem& item, AdafactorSquares* out);
 size_t adafactor_scratch_bytes(int64_t rows, int64_t cols);
 galore_status_t launch_adafactor(const AdafactorItem& item, int n_planes, bool early, cudaStream_t st);
 

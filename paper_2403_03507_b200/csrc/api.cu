@@ -1133,6 +1133,17 @@ galore_status_t galore_step_batch(galore_layer_t* const* layers, void* const* W,
     PhaseTimer pt(0, s);
     return tensor_group_launch_project_adam(scratch.proj, first->cfg.state_fmt, gi > 0 && short_group(groups[gi]), s);
   };
+  // Adafactor's sums of R^2 come out of the projection where K is not sliced and the layer's scratch has room for them (a rule
+  // on the layer alone: its result does not depend on the group)
+  auto af_item_of = [&](const BatchMember& mb) {
+    galore_layer* l = layers[mb.index];
+    float* part; __nv_bfloat16* nbuf;
+    scratch_of(mb, &part, &nbuf);
+    return adafactor_item(l, adam_item(l, part, mb.splits, nbuf, adam_params(l)), (float*)((char*)nbuf + batch_n_bytes(l)));
+  };
+  auto squares_in_projection = [&](const BatchMember& mb, AdafactorSquares* sq) {
+    return layers[mb.index]->cfg.state_fmt == GALORE_STATE_ADAFACTOR && mb.splits == 1 && adafactor_squares(af_item_of(mb), sq);
+  };
   auto launch_proj = [&](size_t gi, cudaStream_t s) -> galore_status_t {
     tensor_group_reset(scratch.proj);
     for (const BatchMember& mb : groups[gi]) {
@@ -1141,6 +1152,8 @@ galore_status_t galore_step_batch(galore_layer_t* const* layers, void* const* W,
       scratch_of(mb, &part, &nbuf);
       GALORE_TRY(tensor_group_add_project(scratch.proj, &l->tc, l->cfg, l->left, G[mb.index], ldg[mb.index], part,
                                           l->ld_part, mb.splits, l->status));
+      AdafactorSquares sq;
+      if (squares_in_projection(mb, &sq)) tensor_group_want_squares(scratch.proj, sq.row, sq.col, sq.tiles);
     }
     PhaseTimer pt(0, s);
     return tensor_group_launch_project(scratch.proj, gi > 0 && short_group(groups[gi]), s);
@@ -1152,13 +1165,16 @@ galore_status_t galore_step_batch(galore_layer_t* const* layers, void* const* W,
     const bool adafactor = first->cfg.state_fmt == GALORE_STATE_ADAFACTOR;
     for (const BatchMember& mb : groups[gi]) {
       galore_layer* l = layers[mb.index];
-      float* part; __nv_bfloat16* nbuf;
-      scratch_of(mb, &part, &nbuf);
-      const AdamItem a = adam_item(l, part, mb.splits, nbuf, adam_params(l));
-      if (adafactor)
-        GALORE_TRY(adafactor_group_add(*scratch.adafactor, adafactor_item(l, a, (float*)((char*)nbuf + batch_n_bytes(l)))));
-      else
-        GALORE_TRY(adam_group_add(*scratch.adam, a, l->cfg.state_fmt, l->q_block));
+      if (adafactor) {
+        AdafactorItem f = af_item_of(mb);
+        AdafactorSquares sq;
+        f.squares_ready = squares_in_projection(mb, &sq);
+        GALORE_TRY(adafactor_group_add(*scratch.adafactor, f));
+      } else {
+        float* part; __nv_bfloat16* nbuf;
+        scratch_of(mb, &part, &nbuf);
+        GALORE_TRY(adam_group_add(*scratch.adam, adam_item(l, part, mb.splits, nbuf, adam_params(l)), l->cfg.state_fmt, l->q_block));
+      }
     }
     PhaseTimer pt(1, s);
     const bool early = short_group(groups[gi]);

@@ -50,7 +50,10 @@ constexpr int kABytes = kBM * kBK * 2;            // 16 KiB: the 128 rows of A o
 // EPI_DRAIN: EPI_PARTIAL with shorter chains.  The tensor core's accumulator rounds towards zero; here it is added to fp32 sums in
 // the epilogue's registers after every few k-blocks (R of 2048 x 5461 at rank 512: after each one 9e-8 from 64 bits, in one
 // accumulator 8e-7).
-enum { EPI_PARTIAL = 0, EPI_ADAM_F32 = 1, EPI_ADAM_Q8 = 2, EPI_DRAIN = 3 };
+// EPI_STATS: EPI_PARTIAL with Adafactor's statistics, the sums of R^2 over 128 columns of a row and over 64 rows of a column (added
+// up in fp64 by the pass behind; over 128 rows a column's sum was further from fp64 than before).  They hide under the next
+// tile's MMAs: eight layers of LLaMA-1B size 361 -> 387 us, and the pass over R for them took 147.
+enum { EPI_PARTIAL = 0, EPI_ADAM_F32 = 1, EPI_ADAM_Q8 = 2, EPI_DRAIN = 3, EPI_STATS = 4 };
 constexpr bool epi_is_adam(int epi) { return epi == EPI_ADAM_F32 || epi == EPI_ADAM_Q8; }
 // Adam is instruction-heavy (about 70 per element with 8-bit moments) and every element is a chain
 // of dependent lookups and arithmetic: sixteen epilogue warps, four per quarter of the accumulator's
@@ -58,9 +61,10 @@ constexpr bool epi_is_adam(int epi) { return epi == EPI_ADAM_F32 || epi == EPI_A
 // tensor cores work on the next tile (eight warps of 128 columns each ran three times longer than
 // the MMAs of a tile).
 // Sixteen as well (64 columns each) where accumulators are drained after every k-block: a pair's MMAs take 512 cycles for one.
-constexpr int epi_warps(int epi, int bn) { return epi == EPI_PARTIAL ? 4 : (epi == EPI_DRAIN ? bn / 16 : 16); }
+constexpr int epi_warps(int epi, int bn) { return epi == EPI_PARTIAL || epi == EPI_STATS ? 4 : (epi == EPI_DRAIN ? bn / 16 : 16); }
 constexpr int epi_threads(int epi, int bn) { return 64 + 32 * epi_warps(epi, bn) + (epi == EPI_ADAM_F32 ? 32 : 0); }   // + producer, MMA, moments
-constexpr int epi_smem(int epi) { return epi == EPI_ADAM_Q8 ? (int)sizeof(Q8Tables) : 0; }
+// behind the ring and the barriers: the tables of the 8-bit code, or the column sums of two tiles by quarters of the rows
+constexpr int epi_smem(int epi) { return epi == EPI_ADAM_Q8 ? (int)sizeof(Q8Tables) : (epi == EPI_STATS ? 2 * 4 * kBN * 4 : 0); }
 
 // A piece of a moment: 32 rows x 64 columns, as two boxes of 32 x 32 (128 bytes a row).  It belongs to the four epilogue warps
 // that can read its rows of the accumulator, 16 columns each, and so does its slot: a warp that waited for a slot's next
@@ -102,6 +106,8 @@ struct TcParams {
   // EPI_PARTIAL
   float* part;
   int64_t ld_part, split_stride;
+  float *row_sq, *col_sq;     // EPI_STATS: rows x sq_tiles, ceil(rows / 64) x columns
+  int sq_tiles;
   int vec32;                  // the partial buffer's base and row pitch are 32-byte aligned
   int32_t* status;
   // EPI_ADAM_*: the state of the layer (rows x cols of the output, row pitch ld_s) and where N goes
@@ -194,6 +200,32 @@ __device__ __forceinline__ void epi_partial(const TcParams& p, const Unit& w, in
     for (int j = 0; j < 32; ++j)
       if (col0 + j < p.N) dst[j] = __uint_as_float(v[j]);
   }
+}
+
+__device__ __forceinline__ float tree_sum(const float (&x)[32]) {
+  float t[16];
+#pragma unroll
+  for (int j = 0; j < 16; ++j) t[j] = x[j] + x[j + 16];
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) {
+#pragma unroll
+    for (int j = 0; j < o; ++j) t[j] += t[j + o];
+  }
+  return t[0];
+}
+// lane l's share of 32 columns that each lane holds one row of: the sum of column l
+__device__ __forceinline__ float column_sum(float (&x)[32]) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+#pragma unroll
+    for (int j = 0; j < o; ++j) {
+      const bool up = (lane & o) != 0;
+      const float keep = up ? x[j + o] : x[j], send = up ? x[j] : x[j + o];
+      x[j] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+  }
+  return x[0];
 }
 
 // ---- Adam in the projection's epilogue ----------------------------------------------------------
@@ -430,7 +462,8 @@ gemm_tc_kernel(const __grid_constant__ TcArgs<CAP> g) {
   auto acce_bar = [&](int a) { return bar_base + 8u * (2 * kStages + 2 + a); };
   auto mvfull_bar = [&](int s) { return bar_base + 8u * (2 * kStages + 4 + s); };
   auto mvdone_bar = [&](int s) { return bar_base + 8u * (2 * kStages + 4 + G::kSlots + s); };
-  constexpr int kBars = 2 * kStages + 4 + 2 * G::kSlots;
+  const uint32_t sq_bar = bar_base + 8u * (2 * kStages + 4 + 2 * G::kSlots);        // EPI_STATS: the column sums of a tile are in place
+  constexpr int kBars = 2 * kStages + 5 + 2 * G::kSlots;
   static_assert(kBars * 8 + 16 <= 256, "barrier space");
   volatile uint32_t* tmem_slot = reinterpret_cast<volatile uint32_t*>(bars + kBars);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(bars + kBars + 1);
@@ -451,6 +484,7 @@ gemm_tc_kernel(const __grid_constant__ TcArgs<CAP> g) {
       mbar_init(accf_bar(a), 1);
       mbar_init(acce_bar(a), kEpiWarps * CTAS);     // one arrival per epilogue warp of the group, from every CTA
     }
+    mbar_init(sq_bar, kEpiWarps);
     for (int s = 0; s < G::kSlots; ++s) {
       mbar_init(mvfull_bar(s), 1);
       mbar_init(mvdone_bar(s), kEpiWarps / 4);
@@ -470,6 +504,7 @@ gemm_tc_kernel(const __grid_constant__ TcArgs<CAP> g) {
   }
   // the 8-bit code tables follow the barriers (256 bytes after the ring)
   Q8Tables* q8t = reinterpret_cast<Q8Tables*>(ring_ptr + G::kRingBytes + 256);
+  float* const col_sums = reinterpret_cast<float*>(ring_ptr + G::kRingBytes + 256);
   if constexpr (EPI == EPI_ADAM_Q8) q8_tables_fill(*q8t, g.q8, (int)threadIdx.x, epi_threads(EPI, BN));
   tc_fence_before();
   __syncthreads();
@@ -637,7 +672,7 @@ gemm_tc_kernel(const __grid_constant__ TcArgs<CAP> g) {
     const int quarter = warp & 3;                   // TMEM lanes 32*quarter .. +31 belong to this warp
     int acc = 0;
     uint32_t acc_phase = 0;
-    uint32_t mv_phase = 0;
+    uint32_t mv_phase = 0, sq_phase = 0;
     bool ok = true;
     auto release_acc = [&]() {                        // accumulator free for the MMA warp (the leader's)
       tc_fence_before();
@@ -721,6 +756,43 @@ gemm_tc_kernel(const __grid_constant__ TcArgs<CAP> g) {
           for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(sum[c + j]);
           epi_partial(p, w, row, w.n0 + part + c, v);
         }
+        continue;
+      } else if constexpr (EPI == EPI_STATS) {
+        if (!__all_sync(0xffffffffu, mbar_wait(accf_bar(acc), acc_phase, abort_flag))) { ok = false; break; }
+        tc_fence_after();
+        float* const sums = col_sums + sq_phase * (4 * BN);
+        float row_lo = 0.f, row_hi = 0.f;             // (halves of a stretch: a balanced tree)
+#pragma unroll 1
+        for (int c = 0; c < BN && w.n0 + c < p.N; c += 32) {
+          uint32_t v[32];
+          tmem_ld_32x32(t_row + (uint32_t)c, v);
+          tmem_ld_wait();
+#pragma unroll
+          for (int j = 0; j < 32; ++j) asm volatile("" : "+r"(v[j]));          // not read before the wait
+          epi_partial(p, w, row, w.n0 + c, v);
+          float sq[32];                               // (rows and columns outside the matrix are zeros)
+#pragma unroll
+          for (int j = 0; j < 32; ++j) sq[j] = __uint_as_float(v[j]) * __uint_as_float(v[j]);
+          if (c & 64) row_hi += tree_sum(sq);
+          else row_lo += tree_sum(sq);
+          sums[quarter * BN + c + lane] = column_sum(sq);
+          if ((c & 127) == 96 || w.n0 + c + 32 >= p.N) {
+            if (row < p.M && p.row_sq) p.row_sq[(int64_t)row * p.sq_tiles + (w.n0 + c) / 128] = row_lo + row_hi;
+            row_lo = row_hi = 0.f;
+          }
+        }
+        release_acc();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(sq_bar);
+        if (!__all_sync(0xffffffffu, mbar_wait(sq_bar, sq_phase, abort_flag))) { ok = false; break; }
+        sq_phase ^= 1u;                               // the other half: a warp may be a tile ahead
+        const int m0 = w.m0 + (int)rank * kBM;
+        for (int c = (warp - 2) * 32 + lane; c < BN; c += 128)
+          if (w.n0 + c < p.N && p.row_sq) {
+            float* const dst = p.col_sq + (int64_t)(m0 / 64) * p.N + w.n0 + c;
+            if (m0 < p.M) dst[0] = sums[c] + sums[BN + c];
+            if (m0 + 64 < p.M) dst[p.N] = sums[2 * BN + c] + sums[3 * BN + c];
+          }
         continue;
       } else {
         if (!mbar_wait(accf_bar(acc), acc_phase, abort_flag)) { ok = false; break; }
@@ -1102,8 +1174,16 @@ galore_status_t tensor_group_add_gemm(TensorGroup* t, const void* A, int64_t lda
   return GALORE_OK;
 }
 
+void tensor_group_want_squares(TensorGroup* t, float* row_sq, float* col_sq, int tiles) {
+  TcParams& p = t->g.p[t->g.count - 1];
+  p.row_sq = row_sq;
+  p.col_sq = col_sq;
+  p.sq_tiles = tiles;
+}
 galore_status_t tensor_group_launch_project(TensorGroup* t, bool early, cudaStream_t st) {
   if (t->g.count == 0) return GALORE_OK;
+  for (int i = 0; i < t->g.count; ++i)
+    if (t->g.p[i].row_sq) return launch_tc<EPI_STATS>(t->g, early, st);
   return launch_tc<EPI_PARTIAL>(t->g, early, st);
 }
 galore_status_t tensor_group_launch_project_drained(TensorGroup* t, int blocks, bool early, cudaStream_t st) {

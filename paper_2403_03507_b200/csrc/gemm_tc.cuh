@@ -62,6 +62,9 @@ galore_status_t tensor_group_launch_project_adam(TensorGroup* t, int32_t state_f
 galore_status_t tensor_group_add_gemm(TensorGroup* t, const void* A, int64_t lda, int a_mn, const void* B, int64_t ldb,
                                       int b_mn, int M, int N, int K, float* C, int64_t ldc, int32_t* status);
 galore_status_t tensor_group_launch_project(TensorGroup* t, bool early, cudaStream_t st);
+// The problem added last (one K slice) leaves the sums of R^2 as well: over stretches of 128 columns, rows x tiles, and over
+// stretches of 64 rows, one row of sums for each
+void tensor_group_want_squares(TensorGroup* t, float* row_sq, float* col_sq, int tiles);
 // one layer's projection, its accumulators added to fp32 sums after every `blocks` times 64 of K
 galore_status_t tensor_group_launch_project_drained(TensorGroup* t, int blocks, bool early, cudaStream_t st);
 

@@ -146,3 +146,31 @@ def test_fp32_path_layers_in_a_batch_match_the_oracle(state_fmt):
     if state_fmt == "adafactor":
         for l, o in zip(layers, orcs):
             _state_close(l, o, 1e-4)
+
+
+def test_statistics_of_grouped_bf16_layers_are_the_sums():
+    """Projections that leave the sums of R^2 beside R (bf16, K not sliced): ranks and lengths with remainders to tiles of 128 rows,
+    256 columns and chunks of 32, one CTA and two, both sides, and a tall R whose tiles have too many rows (the pass over R)."""
+    shapes = [(256, 1000, 64), (300, 1096, 40), (1096, 304, 136), (520, 264, 64), (136, 128, 128), (264, 5464, 200),
+              (2048, 2048, 512), (2048, 2320, 512), (2320, 2048, 520), (64, 48, 8), (40000, 64, 16)]
+    layers, orcs, Wg, Gd, Gh = [], [], [], [], []
+    for i, (m, n, r) in enumerate(shapes):
+        gen = np.random.default_rng(i)
+        layer = gb.Layer(gb.make_config(m, n, r, w_dtype="bf16", g_dtype="bf16", state_fmt="adafactor", auto_refresh=False))
+        assert layer.uses_tensor_path
+        P = np.eye(min(m, n), dtype=np.float32)[:, gen.permutation(min(m, n))[:r]]       # R is a choice of G's rows or columns
+        layer.set_projector(torch.from_numpy(P))
+        o = go.GaLoreOracle(m, n, r, 0.25, 1000, w_store="bf16", state="f32", inner="adafactor")
+        o.set_projector(P.astype(np.float64))
+        G = gen.integers(-8, 9, (m, n)).astype(np.float32)
+        layers.append(layer); orcs.append(o); Gh.append(G)
+        Wg.append(torch.zeros(m, n, device="cuda", dtype=torch.bfloat16)); Gd.append(to_dev(G, "bf16"))
+    gb.Batch(layers, Wg, Gd).galore_step_batch(1e-2)
+    torch.cuda.synchronize()
+    for (m, n, r), l, o, w, g in zip(shapes, layers, orcs, Wg, Gh):
+        o.step(np.zeros((m, n)), g, 1e-2, auto_refresh=False)
+        assert l.device_status() == 0 and l.step_count == 1
+        M, v_row, v_col = [to_host(t) for t in l.get_adafactor_state()]
+        # whole numbers below 2^24 up to the division (40000 x 64 at most): a rounding of the quotient and one of its store
+        assert np.abs(v_row / o.v_row - 1.0).max() <= 2.0 ** -22 and np.abs(v_col / o.v_col - 1.0).max() <= 2.0 ** -22, (m, n, r)
+        _state_close(l, o, 1e-4)

@@ -7,10 +7,11 @@
 // sums: fmaf over k, slice after slice.  A bf16 W or 8-bit moments round far above the difference, and Adafactor's
 // factored second moment does not vanish with a single r: there the split products carry the projection.
 //
-// What bounds it: the FMA rate of a 128 x 128 tile of 256 threads for large matrices; for small ones latency.  fp32 operands whose
-// rows lie along the tile on 16-byte boundaries are copied to shared memory asynchronously, several steps of 16 k ahead (a small
-// result's whole slice at once: five waits for memory become one).  512 x 1376 at rank 128: 25.0 -> 20.1 us a step; 2048 x 5461 at
-// rank 512: 552 -> 316 us (36 TFLOP/s).  Others go through registers, one step ahead: copies of four bytes were slower.
+// What bounds it: the FMA rate of a 128 x 128 tile of 256 threads for large matrices; for small ones latency.  fp32 operands on
+// 16-byte boundaries whose rows lie along the tile, or A's along K, are copied to shared memory asynchronously, several steps of 16 k ahead (a small
+// result's whole slice at once: five waits for memory become one).  512 x 1376 at rank 128: 25.0 -> 20.1 us a step, 1376 x 512
+// 25.0 -> 20.3; 2048 x 5464 and 5461 x 2048 at rank 512 650 -> 417 and 439, 11008 x 4096 at 128 990 -> 540.  Others go through
+// registers, one step ahead: copies of four bytes were slower.
 #include "gemm_fma.cuh"
 
 #include <algorithm>
@@ -29,13 +30,22 @@ constexpr int kThreads = 256;
 constexpr int stages(bool async, int bm) { return !async ? 1 : (bm == 64 ? 5 : 4); }
 constexpr int smem_bytes(bool async, int bm, int bn) { return stages(async, bm) * kBK * (bm + bn + 8) * 4; }
 
-// BM x BN tile, TM x TN elements a thread in groups of four
-template <typename TA, typename TB, int BM, int BN, int TM, int TN, int CAP>
-__global__ void __launch_bounds__(kThreads) gemm_fma_kernel(const __grid_constant__ FmaArgs<CAP> g) {
+enum { FMA_LOADED = 0, FMA_COLUMNS = 1, FMA_ROWS = 2 };
+// Operands that can be copied ahead: four elements along the tile at a time, A's also along K (FMA_ROWS).
+__host__ __device__ inline bool fma_copied(const FmaProblem& p, int mode) {
+  return mode != FMA_LOADED && (mode == FMA_ROWS ? p.sAk : p.sAi) == 1 && p.sBj == 1 && (((uintptr_t)p.A | (uintptr_t)p.B) & 15) == 0 &&
+         (((mode == FMA_ROWS ? p.sAi : p.sAk) | p.sBk) & 3) == 0;
+}
+
+// BM x BN tile, TM x TN elements a thread in groups of four.  A kernel for each kind of A, as both in one, or a bound on the registers
+// that is not the one a kind does best with, cost the others: 512 x 1376 at rank 128 22.9 instead of 20.2 us a step, 2048 x 5461 of
+// rows off 16 bytes 632 instead of 548, 2048 x 5464 425 instead of 417.
+template <typename TA, typename TB, int BM, int BN, int TM, int TN, int CAP, int MODE>
+__global__ void __launch_bounds__(kThreads, BM == 64 ? 2 : (MODE == FMA_COLUMNS ? 0 : 1)) gemm_fma_kernel(const __grid_constant__ FmaArgs<CAP> g) {
   static_assert((BM / TM) * (BN / TN) == kThreads, "one micro-tile a thread");
   constexpr int LA = BM * kBK / kThreads, LB = BN * kBK / kThreads;      // elements of a tile each thread fetches
-  constexpr bool kAsync = sizeof(TA) == 4 && sizeof(TB) == 4;
-  constexpr int kStages = stages(kAsync, BM);
+  constexpr bool kRows = MODE == FMA_ROWS;
+  constexpr int kStages = stages(MODE != FMA_LOADED, BM);
   extern __shared__ __align__(16) float fma_smem[];
   float(*const As)[kBK][BM + 4] = reinterpret_cast<float(*)[kBK][BM + 4]>(fma_smem);
   float(*const Bs)[kBK][BN + 4] = reinterpret_cast<float(*)[kBK][BN + 4]>(fma_smem + kStages * kBK * (BM + 4));
@@ -79,10 +89,31 @@ __global__ void __launch_bounds__(kThreads) gemm_fma_kernel(const __grid_constan
         for (int v = 0; v < TN; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
     }
   };
-  bool async = false;
-  if constexpr (kAsync)
-    async = sAi == 1 && sBj == 1 && (((uintptr_t)A | (uintptr_t)B) & 15) == 0 && ((sAk | sBk) & 3) == 0;
-  if (async) {
+  // A's rows along K: four k of a row in 16 bytes, the fours of a row moved round by its place (a warp reads two rows, four apart)
+  auto a_four = [&](float* stage, int i, int four) { return stage + i * kBK + ((four ^ (i >> 2)) & 3) * 4; };
+  auto multiply_rows = [&](float* As, const float (*Bs)[BN + 4]) {
+#pragma unroll
+    for (int four = 0; four < kBK / 4; ++four) {
+      float4 a[TM];
+#pragma unroll
+      for (int u = 0; u < TM; ++u) a[u] = *reinterpret_cast<const float4*>(a_four(As, (u / 4) * (BM / (TM / 4)) + ty * 4 + (u % 4), four));
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        float b[TN];
+#pragma unroll
+        for (int v = 0; v < TN; ++v) b[v] = Bs[4 * four + k][(v / 4) * (BN / (TN / 4)) + tx * 4 + (v % 4)];
+#pragma unroll
+        for (int u = 0; u < TM; ++u) {
+          const float au = k == 0 ? a[u].x : k == 1 ? a[u].y : k == 2 ? a[u].z : a[u].w;
+#pragma unroll
+          for (int v = 0; v < TN; ++v) acc[u][v] = fmaf(au, b[v], acc[u][v]);
+        }
+      }
+    }
+  };
+  bool copied = false;
+  if constexpr (MODE != FMA_LOADED) copied = fma_copied(p, MODE);
+  if (copied) {
     // 16 k of one operand in runs of four; zeros outside the matrix
     auto copy = [&]<int BX, class Tile>(std::integral_constant<int, BX>, Tile dst, const float* X, int64_t s_k, int x0, int X_size, int k0) {
 #pragma unroll
@@ -96,7 +127,18 @@ __global__ void __launch_bounds__(kThreads) gemm_fma_kernel(const __grid_constan
     const int steps = (k_end - k_begin + kBK - 1) / kBK;
     auto request = [&](int step) {                    // (an empty group behind the last step: the count of groups stays)
       if (step < steps) {
-        copy(std::integral_constant<int, BM>(), As[step % kStages], (const float*)A, sAk, m0, M, k_begin + step * kBK);
+        if constexpr (kRows) {
+          const int k0 = k_begin + step * kBK;
+#pragma unroll
+          for (int e = 0; e < BM * kBK / 4 / kThreads; ++e) {
+            const int idx = tid + e * kThreads, four = idx % (kBK / 4), i = idx / (kBK / 4);
+            const int valid = m0 + i < M ? min(4, max(0, k_end - k0 - 4 * four)) : 0;
+            const float* src = valid ? (const float*)A + (int64_t)(m0 + i) * sAi + k0 + 4 * four : (const float*)A;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(a_four(&As[step % kStages][0][0], i, four))), "l"(src), "r"(valid * 4) : "memory");
+          }
+        } else {
+          copy(std::integral_constant<int, BM>(), As[step % kStages], (const float*)A, sAk, m0, M, k_begin + step * kBK);
+        }
         copy(std::integral_constant<int, BN>(), Bs[step % kStages], (const float*)B, sBk, n0, N, k_begin + step * kBK);
       }
       asm volatile("cp.async.commit_group;" ::: "memory");
@@ -107,7 +149,8 @@ __global__ void __launch_bounds__(kThreads) gemm_fma_kernel(const __grid_constan
       asm volatile("cp.async.wait_group %0;" ::"n"(kStages - 2) : "memory");
       __syncthreads();                                // the step's copies of all threads are in, the stage to be filled has been read
       request(step + kStages - 1);
-      multiply(As[step % kStages], Bs[step % kStages]);
+      if constexpr (kRows) multiply_rows(&As[step % kStages][0][0], Bs[step % kStages]);
+      else multiply(As[step % kStages], Bs[step % kStages]);
     }
   } else {
     float ra[LA], rb[LB];
@@ -175,13 +218,27 @@ __global__ void __launch_bounds__(kThreads) gemm_fma_kernel(const __grid_constan
 // Results below 96 tiles of 128 x 128 are cut into 64 x 64.
 bool small_result(int64_t M, int64_t N) { return M * N < (int64_t)128 * 128 * 96; }
 
-template <typename TA, typename TB, int BM, int TM, int CAP>
-galore_status_t launch_tiles(const FmaArgs<CAP>& g, bool early, cudaStream_t st) {
-  constexpr int smem = smem_bytes(sizeof(TA) == 4 && sizeof(TB) == 4, BM, BM);
-  auto kern = gemm_fma_kernel<TA, TB, BM, BM, TM, TM, CAP>;
+template <typename TA, typename TB, int BM, int TM, int MODE, int CAP>
+galore_status_t launch_mode(const FmaArgs<CAP>& g, bool early, cudaStream_t st) {
+  constexpr int smem = smem_bytes(MODE != FMA_LOADED, BM, BM);
+  auto kern = gemm_fma_kernel<TA, TB, BM, BM, TM, TM, CAP, MODE>;
   static std::atomic<uint64_t> configured{0};
   GALORE_TRY(allow_smem(configured, (const void*)kern, smem));
   return launch_kernel(kern, dim3((unsigned)g.unit_end[g.count - 1]), kThreads, smem, 1, early, st, g);
+}
+// (a problem of a group that does not fit its kernel's copies is loaded there)
+template <typename TA, typename TB, int BM, int TM, int CAP>
+galore_status_t launch_tiles(const FmaArgs<CAP>& g, bool early, cudaStream_t st) {
+  if constexpr (sizeof(TA) == 4 && sizeof(TB) == 4) {
+    int columns = 0, rows = 0;
+    for (int i = 0; i < g.count; ++i) {
+      columns += fma_copied(g.p[i], FMA_COLUMNS) ? 1 : 0;
+      rows += fma_copied(g.p[i], FMA_ROWS) ? 1 : 0;
+    }
+    if (rows > columns) return launch_mode<TA, TB, BM, TM, FMA_ROWS>(g, early, st);
+    if (columns > 0) return launch_mode<TA, TB, BM, TM, FMA_COLUMNS>(g, early, st);
+  }
+  return launch_mode<TA, TB, BM, TM, FMA_LOADED>(g, early, st);
 }
 
 template <typename TA, typename TB>

@@ -94,17 +94,21 @@ def test_static_step_sums_in_the_same_order(m, n, r, pad):
     assert torch.equal(M, _expected(layer, P, G, _slices(*layer.state_shape, min(m, n))))
 
 
-# Operands that are copied to shared memory ahead (rows along the tile, 16-byte boundaries) and those that are not give the same
-# sums: tiles of 64 and of 128, ragged ends, fewer steps of 16 than stages and many, slices
+# Operands that are copied to shared memory ahead (rows along the tile, or G's along the sum; 16-byte boundaries) and those that
+# are not give the same sums: tiles of 64 and of 128, ragged ends, fewer steps of 16 than stages and many, slices
+@pytest.mark.parametrize("side", [gb.SIDE_LEFT, gb.SIDE_RIGHT])
 @pytest.mark.parametrize("m,n,r", [(5, 9, 4), (16, 70, 12), (40, 200, 36), (300, 515, 64), (513, 1377, 128), (1100, 3001, 260)])
-def test_copied_operands_give_the_bits_of_loaded_ones(m, n, r):
+def test_copied_operands_give_the_bits_of_loaded_ones(m, n, r, side):
+    if side == gb.SIDE_RIGHT:
+        m, n = n, m
+    K = min(m, n)
     gen = torch.Generator(device="cuda")
     gen.manual_seed(m + n)
-    P = torch.linalg.qr(torch.randn(m, r, generator=gen, device="cuda"))[0]
+    P = torch.linalg.qr(torch.randn(K, r, generator=gen, device="cuda"))[0]
     G = torch.randn(m, n, generator=gen, device="cuda")
     got = []
     for pitch in ((n + 3) // 4 * 4, (n + 3) // 4 * 4 + 1):       # rows of G on 16-byte boundaries, and off them
-        layer = gb.Layer(gb.make_config(m, n, r, w_dtype="f32", g_dtype="f32", auto_refresh=False, side=gb.SIDE_LEFT))
+        layer = gb.Layer(gb.make_config(m, n, r, w_dtype="f32", g_dtype="f32", auto_refresh=False, side=side))
         layer.set_projector(P)
         g = torch.full((m, pitch), float("nan"), device="cuda")[:, :n]
         g.copy_(G)
@@ -112,6 +116,6 @@ def test_copied_operands_give_the_bits_of_loaded_ones(m, n, r):
         assert layer.device_status() == 0
         got.append(layer.get_moments())
     assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
-    R = P.double().T @ G.double()
-    # a chain of m fused multiply-adds: at most 2^-24 sqrt(m) of the root mean square of R in the norm
-    assert float((got[0][0].double() / 0.1 - R).norm() / R.norm()) <= 2 ** -24 * (8 + m ** 0.5)
+    R = P.double().T @ G.double() if side == gb.SIDE_LEFT else G.double() @ P.double()
+    # a chain of K fused multiply-adds: at most 2^-24 sqrt(K) of the root mean square of R in the norm
+    assert float((got[0][0].double() / 0.1 - R).norm() / R.norm()) <= 2 ** -24 * (8 + K ** 0.5)

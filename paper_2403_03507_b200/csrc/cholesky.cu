@@ -11,9 +11,10 @@
 // forms the L_i, L_j or T_Jj it needs itself (three 64^3 products instead of one, but one launch per
 // step); otherwise a launch before it leaves them in T, the L_i in the part above the diagonal.
 //
-// What bounds it: for a few blocks the chain of launches, two thirds of each the 64 x 64 factorisation (a step in
-// fp64, before the pivots took the library's rsqrt: 46 thousand cycles, of them 30 the factorisation, 9 the two products, 5 the
-// loads; a refresh of 512 x 1376 at rank 128 takes 4.08 ms with it, 3.92 without); for many the FMA rate.
+// What bounds it: for a few blocks the chain of launches, about half of each the 64 x 64 factorisation (with a
+// panel's rows in one warp's registers, its inverse beside the next panel and fp64 updates on the MMA unit a launch of four blocks in
+// fp64 takes 24.9 us at least instead of 32.9, the refresh of 512 x 1376 at rank 128 3.54 ms instead of 3.69); for many the
+// FMA rate.
 #include "cholesky.cuh"
 
 #include <algorithm>

@@ -54,7 +54,7 @@ __device__ __forceinline__ BlockPair block_pair(int pair, int round, int nblk) {
 
 // part[(pair * chunks + chunk)] (64 x 64) = rows(pair)[:, chunk] rows(pair)[:, chunk]^T
 // In the first round of a sweep its upper triangle, later the products of the two blocks with each other alone: those within a
-// block the sweep kernel has carried along since (eight 1280 x 1280 matrices: 40 -> 23 us a round).
+// block the sweep kernel has carried along since (eight 1280 x 1280 matrices: 40 -> 26 us a round).
 __global__ void __launch_bounds__(128) jb_gram_kernel(const double* X, int b, int nblk, int round, int chunks,
                                                       double* __restrict__ part, const SlotList slots) {
   grid_dependency_wait();

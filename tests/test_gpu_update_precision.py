@@ -40,3 +40,27 @@ def test_update_keeps_fp32_precision_at_every_rank(m, n, r, pad, count):
         # The tensor core cuts off up to a unit of 2^-23 of its accumulator per 16 products, eight times before it is
         # drained.  (An accumulator of the whole rank shows 4.1e-7 at 512 and 1.8e-6 at 2048.)
         assert abs(float((W * want).sum() / (want * want).sum()) - 1) <= 2e-7
+
+
+# bf16 W in groups: tiles of pairs or of single CTAs by the waves of each, but by the old line up to eight blocks of products
+# (rank 64 and below); ragged sizes of both sides in one call
+@pytest.mark.parametrize("r", [64, 65, 200])
+@pytest.mark.parametrize("count", [3, 16, 28])
+def test_grouped_updates_of_bf16_weights_are_rounded_products(r, count):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(r + count)
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda")
+    layers, Ws, Gs = [], [], []
+    for i in range(count):
+        m, n = [(448, 1200), (448, 448), (1194, 450)][i % 3]
+        layers.append(gb.Layer(gb.make_config(m, n, r, w_dtype="bf16", g_dtype="f32", state_fmt="adafactor", auto_refresh=False)))
+        layers[-1].set_projector(torch.linalg.qr(rand(layers[-1].proj_rows, r))[0])
+        Ws.append(torch.zeros(m, (n + 7) // 8 * 8, device="cuda", dtype=torch.bfloat16)[:, :n])
+        Gs.append(rand(m, n))
+    gb.Batch(layers, Ws, Gs).galore_step_batch(1.0)
+    for layer, W in zip(layers, Ws):
+        assert layer.device_status() == 0
+        P, N = layer.get_projector().double(), layer.get_adafactor_state()[0].double()
+        want = -0.25 * (P @ N if layer.side == gb.SIDE_LEFT else N @ P.T)
+        # half a unit of bf16 in the last place, and fp32's error of the product (4e-6 of the largest entry is far above it)
+        assert bool(((W.double() - want).abs() <= 2.0 ** -8 * want.abs() + 4e-6 * want.abs().max()).all())

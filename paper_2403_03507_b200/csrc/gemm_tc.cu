@@ -988,18 +988,27 @@ int fill_splits(int64_t M, int64_t N, int64_t K, int ctas) {
 // time of one + time of a unit) plus the slices' round trip.  Microseconds a k-block, fitted to steps in 1 to 7 slices of 2048 x 2048 and
 // 2048 x 5461 at rank 512, 4096 x 11008 at 1024, 11008 x 4096 and 4096 x 11008 at 128: pairs 0.33, single CTAs 0.35, with tiles
 // of 128 columns 0.25.  (2048 x 5461, 8-bit moments: 58.9 us unsliced, 61.4 in three, 68.1 in five, which fill the machine best.)
-int time_splits(int64_t M, int64_t N, int64_t K, int ctas) {
+// Half a microsecond less is the least that the fit can tell: below it the slices that fill the machine stay.  (Steps in the one / the
+// other: 3008 x 1183 at rank 80 predicted 3.40 / 3.39, measured 20.4 / 21.7; 1216 x 2816 at 192 4.80 / 4.69, 21.3 / 22.3; 1344 x 2816 at 184
+// 5.17 / 4.89, 22.0 / 22.5; 3840 x 2432 at 632 15.9 / 15.4, 55.8 / 54.5; 1920 x 2267 at 256 6.32 / 5.51, 29.3 / 28.5; the 19
+// sizes measured above the line all gained.)
+// codes: 8-bit moments, whose codes at a threshold show the last bit of R.  Only slices that leave R's bits as they are: those that
+// fill the machine, or one, whose accumulators are drained where those slices end and added in their order.
+int time_splits(int64_t M, int64_t N, int64_t K, int ctas, bool codes) {
   const int64_t tiles = ceil_div(M, kBM * ctas) * ceil_div(N, kBN);
   const int kblocks = (int)ceil_div(K, kBK);
   const double block = ctas == 2 ? 0.33 : (N <= 128 ? 0.25 : 0.35);
-  int best = 1;
-  double best_us = 1e30;
-  for (int s = 1; s <= 8; ++s) {
+  auto us = [&](int s) {
+    return (double)ceil_div(tiles * s, 148 / ctas) * (ceil_div(kblocks, s) * block + 1.1) + s * (0.1 + (double)(M * N) * 4.0 / 6.0e6);
+  };
+  const int fill = fill_splits(M, N, K, ctas);
+  int best = fill;
+  double best_us = us(fill) - 0.5;
+  for (int s = 1; s <= (codes ? 1 : 8); ++s) {
     const int per = (int)ceil_div(kblocks, s);
     if (s > 1 && per < 4) break;
     if ((int)ceil_div(kblocks, per) != s) continue;
-    const double us = (double)ceil_div(tiles * s, 148 / ctas) * (per * block + 1.1) + s * (0.1 + (double)(M * N) * 4.0 / 6.0e6);
-    if (us < best_us) { best_us = us; best = s; }
+    if (us(s) < best_us) { best_us = us(s); best = s; }
   }
   return best;
 }
@@ -1020,7 +1029,8 @@ int tensor_proj_splits(const galore_config_t& c, bool left) {
 int tensor_chain_blocks(int64_t K, int splits) { return (int)ceil_div(ceil_div(K, kBK), std::max(1, splits)); }
 int tensor_step_splits(const galore_config_t& c, bool left) {
   const int ctas = tensor_ctas(c);
-  return left ? time_splits(c.rank, c.n, c.m, ctas) : time_splits(c.m, c.rank, c.n, ctas);
+  const bool codes = c.state_fmt == GALORE_STATE_Q8_BLOCK;
+  return left ? time_splits(c.rank, c.n, c.m, ctas, codes) : time_splits(c.m, c.rank, c.n, ctas, codes);
 }
 
 galore_status_t tensor_plan_init(TensorPlan* plan, const galore_config_t& c, bool left, void* P) {

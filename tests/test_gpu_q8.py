@@ -87,3 +87,25 @@ def test_tiled_blocks_bit_exact(signed, rows, cols, tile):
 def test_empty_input():
     codes, am = gb.galore_q8_quantize(torch.zeros(0, device="cuda"), True, 2048)
     assert codes.numel() == 0 and am.numel() == 0
+
+
+# A layer's own step may slice the projection's K otherwise than a batch of one (which fills the machine with slices): the same R, and
+# so the same codes.  Sizes for which the slices by time were others: both sides, tiles of one CTA and of pairs, of 128 columns
+@pytest.mark.parametrize("m,n,r", [(4096, 11008, 1024), (2624, 3640, 424), (2240, 4976, 1040), (5248, 2560, 96), (2176, 1864, 160), (2432, 1560, 64), (2752, 1000, 968)])
+def test_codes_do_not_depend_on_the_slices_of_the_projection(m, n, r):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(m + n)
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda")
+    layers = [gb.Layer(gb.make_config(m, n, r, w_dtype="bf16", g_dtype="bf16", state_fmt="q8", auto_refresh=False, adam_place=gb.ADAM_OWN_KERNEL)) for _ in range(2)]
+    P = torch.linalg.qr(rand(layers[0].proj_rows, r))[0]
+    W = [(0.02 * rand(m, n)).bfloat16()]
+    W.append(W[0].clone())
+    for layer in layers:
+        layer.set_projector(P)
+    for _ in range(2):
+        G = rand(m, n).bfloat16()
+        layers[0].galore_step(W[0], G, 1e-2)
+        gb.Batch(layers[1:], W[1:], [G]).galore_step_batch(1e-2)
+    for a, b in zip(layers[0].get_q8_state(), layers[1].get_q8_state()):
+        assert torch.equal(a, b)
+    assert torch.equal(W[0], W[1])

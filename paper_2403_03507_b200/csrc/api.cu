@@ -589,6 +589,43 @@ size_t split_layer_bytes(const galore_layer* l, int splits) {
          (l->cfg.state_fmt == GALORE_STATE_ADAFACTOR ? adafactor_scratch_bytes(l->srows, l->scols) : 0);
 }
 
+// What the projections and the updates of a group of them take, in microseconds (the optimizer's passes between them take what their bytes
+// take, however they are grouped).
+double split_members_us(galore_layer_t* const* layers, void* const* W, const int64_t* ldw, const void* const* G, const int64_t* ldg,
+                        const int* members, int count) {
+  const galore_config_t& kind = layers[members[0]]->cfg;
+  SplitTiles proj;
+  ApplyTiles update;
+  proj.may_pair = kind.p_dtype == GALORE_F32 && kind.g_dtype == GALORE_F32;
+  for (int k = 0; k < count; ++k) {
+    const int i = members[k];
+    const galore_layer* l = layers[i];
+    const galore_config_t& c = l->cfg;
+    proj.singles += ceil_div(l->srows, 128) * ceil_div(l->scols, 128);
+    proj.pairs += ceil_div(l->srows, 256) * ceil_div(l->scols, 256);
+    proj.blocks = std::max(proj.blocks, ceil_div(l->d, 64));
+    proj.may_pair = proj.may_pair && (((uintptr_t)G[i] | (uintptr_t)(ldg[i] * 4) | (uintptr_t)(c.rank * 4)) & 15) == 0;
+    update.add((int)c.m, (int)c.n, c.rank, std::max(1, l->p_planes), 3, (((uintptr_t)W[i] | (uintptr_t)(ldw[i] * (int64_t)dtype_size(c.w_dtype))) & 15) == 0);
+  }
+  return (fma_projection(kind) ? fma_group_us(proj.singles, 64 * proj.blocks) : split_group_us(proj)) + apply_group_us(update, kind.w_dtype);
+}
+// Layers to a group, of `count` of one kind that go into several: as many as a launch carries, or groups of equal size where the last waves
+// of their launches are the fuller ones.  (56 matrices as 32 + 24 / 28 + 28, us a step: eight layers of LLaMA-130M at rank 256 475 / 431,
+// of 512 and 1024 at rank 96 302 / 314, of 448 and 1000 at rank 40 262 / 281, of 1024 and 2752 at rank 256 731 / 677.)
+int split_group_size(galore_layer_t* const* layers, void* const* W, const int64_t* ldw, const void* const* G, const int64_t* ldg,
+                     const std::vector<int>& members, int most) {
+  const int count = (int)members.size();
+  if (count <= most) return most;
+  const int equal = (int)ceil_div(count, ceil_div(count, most));
+  double us[2] = {0.0, 0.0};
+  for (int way = 0; way < 2; ++way) {
+    const int size = way ? equal : most;
+    for (int first = 0; first < count; first += size)
+      us[way] += split_members_us(layers, W, ldw, G, ldg, members.data() + first, std::min(size, count - first));
+  }
+  return us[0] < us[1] ? most : equal;
+}
+
 struct SplitMember {      // one member of a group, with its operands of this call
   galore_layer* l;
   void* W;
@@ -1045,9 +1082,23 @@ galore_status_t galore_step_batch(galore_layer_t* const* layers, void* const* W,
   // The groups run one after another on the caller's stream, each in the whole batch workspace.
   const size_t room = batch_ws_bytes & ~(size_t)255;
   std::vector<std::vector<BatchMember>> groups, fgroups;
-  // groups of equal size: 56 layers as 28 + 28 rather than 32 + 24 (LLaMA-130M set: the last wave of each launch is the fuller one)
-  int fcap = std::min((int)kSplitGroup, std::min((int)kAdamGroup, (int)kAdafactorGroup));
-  fcap = (int)ceil_div(std::max(1, groupable), ceil_div(std::max(1, groupable), fcap));
+  // layers of the fp32 path: how many of each kind go into a group (0: the layer is not grouped)
+  std::vector<int> group_size((size_t)count, 0);
+  if (batch_ws && groupable >= 2) {
+    auto member = [&](int32_t i) {
+      const galore_layer* l = layers[i];
+      return split_groupable(l) && split_layer_bytes(l, split_slices(l, groupable)) <= room;
+    };
+    std::vector<int> kind;
+    for (int32_t i = 0; i < count; ++i) {
+      if (group_size[i] > 0 || !member(i)) continue;
+      kind.clear();
+      for (int32_t j = i; j < count; ++j)
+        if (group_size[j] == 0 && member(j) && split_same_kind(layers[i], layers[j])) kind.push_back(j);
+      const int size = split_group_size(layers, W, ldw, G, ldg, kind, std::min((int)kSplitGroup, std::min((int)kAdamGroup, (int)kAdafactorGroup)));
+      for (int j : kind) group_size[j] = size;
+    }
+  }
   {
     size_t used = 0;
     std::vector<size_t> fused_bytes_of;
@@ -1056,25 +1107,23 @@ galore_status_t galore_step_batch(galore_layer_t* const* layers, void* const* W,
       const bool ok = batch_ws && batch_eligible(l, W[i], ldw[i], G[i], ldg[i]);
       const int splits = batch_splits(l, eligible);
       const size_t need = ok ? batch_layer_bytes(l, splits) : 0;
-      if (!ok && batch_ws && split_groupable(l) && groupable >= 2) {
+      if (group_size[i] > 0) {
         const int fs = split_slices(l, groupable);
         const size_t fneed = split_layer_bytes(l, fs);
-        if (fneed <= room) {
-          // any open group of the same kind takes it (the layers are independent: their order in the list does
-          // not matter, so a list in model order, sides alternating, still gives full groups)
-          int at = -1;
-          for (int gi = (int)fgroups.size() - 1; gi >= 0 && at < 0; --gi)
-            if (split_same_kind(layers[fgroups[gi][0].index], l) && (int)fgroups[gi].size() < fcap && fused_bytes_of[gi] + fneed <= room)
-              at = gi;
-          if (at < 0) {
-            fgroups.emplace_back();
-            fused_bytes_of.push_back(0);
-            at = (int)fgroups.size() - 1;
-          }
-          fgroups[at].push_back(BatchMember{i, fused_bytes_of[at], fs});
-          fused_bytes_of[at] += fneed;
-          continue;
+        // any open group of the same kind takes it (the layers are independent: their order in the list does
+        // not matter, so a list in model order, sides alternating, still gives full groups)
+        int at = -1;
+        for (int gi = (int)fgroups.size() - 1; gi >= 0 && at < 0; --gi)
+          if (split_same_kind(layers[fgroups[gi][0].index], l) && (int)fgroups[gi].size() < group_size[i] && fused_bytes_of[gi] + fneed <= room)
+            at = gi;
+        if (at < 0) {
+          fgroups.emplace_back();
+          fused_bytes_of.push_back(0);
+          at = (int)fgroups.size() - 1;
         }
+        fgroups[at].push_back(BatchMember{i, fused_bytes_of[at], fs});
+        fused_bytes_of[at] += fneed;
+        continue;
       }
       if (!ok || need > room) {
         // plain step (its refresh, if due, is already done: auto_refresh off for this call)

@@ -30,6 +30,14 @@ struct ApplyGroup {
   ApplyItem item[kApplyGroup];
   int count = 0;
 };
+// Tiles of a group's updates: 256 x 256 per CTA pair, 128 x 128 per CTA; the most k-blocks of one, all products of planes
+struct ApplyTiles {
+  int64_t pairs = 0, singles = 0, blocks = 0;
+  bool aligned = true;       // W's rows lie on 16-byte boundaries
+  void add(int m, int n, int r, int p_planes, int n_planes, bool w_aligned);
+};
+// microseconds of a group's update with operands of several planes
+double apply_group_us(const ApplyTiles& t, int32_t w_dtype);
 galore_status_t apply_group_add(ApplyGroup& g, const ApplyItem& item);
 // early: the kernel before this one on the stream lets its successor start (griddepcontrol.launch_dependents) and does not
 // write W.  All items share the type of W.

@@ -268,6 +268,9 @@ int fma_choose_slices(int64_t M, int64_t N, int64_t K) {
   return fma_effective_slices(K, (int)want);
 }
 
+// 28 matrices of 512 x 1376 at rank 128, 196 tiles: 145 us in two waves; 784 of 1024 x 2752 at rank 512: 1.6 ms in six
+double fma_group_us(int64_t tiles, int64_t k) { return (double)ceil_div(tiles, 148) * (double)k * 0.14; }
+
 galore_status_t fma_group_add(FmaGroup& g, const FmaProblem& problem, int slices) {
   if (g.count >= kFmaGroup) return GALORE_ERR_BUFFER_TOO_SMALL;
   FmaProblem p = problem;

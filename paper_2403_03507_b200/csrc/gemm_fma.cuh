@@ -30,6 +30,8 @@ using FmaGroup = FmaArgs<kFmaGroup>;
 int fma_choose_slices(int64_t M, int64_t N, int64_t K);
 // slices that a request for `slices` gives (they are multiples of 16 elements long)
 int fma_effective_slices(int64_t K, int slices);
+// microseconds of a group of products, unsliced, with `tiles` of 128 x 128 and K up to k
+double fma_group_us(int64_t tiles, int64_t k);
 galore_status_t fma_group_add(FmaGroup& g, const FmaProblem& problem, int slices);
 // All problems share the operand types.  early: see launch.cuh.
 galore_status_t launch_fma_group(const FmaGroup& g, int32_t a_dtype, int32_t b_dtype, bool early, cudaStream_t st);

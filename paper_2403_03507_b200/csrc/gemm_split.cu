@@ -524,6 +524,15 @@ double split_store_us(int64_t M, int64_t N, int64_t K, int slices) {
   return split_us(split_units(M, N, slices, 128), ceil_div(ceil_div(K, kSplitK), slices), false);
 }
 
+// The kernel is the one that launch_split_store takes.  Its time, measured in groups of 8 to 32 matrices with K of 384 to 2048, is 1.75 us a
+// block + 3.6 us for every wave of single tiles (768 x 2048 at rank 256: 8 / 16 / 32 of them 58 / 107 / 181 us), 2.85 + 0.6 us of pairs
+// (47 / 81 / 151 us), and about 10 us a launch.
+double split_group_us(const SplitTiles& t) {
+  const bool pair = t.may_pair && split_us(t.pairs, t.blocks, true) < split_us(t.singles, t.blocks, false);
+  const double block = (double)t.blocks;
+  return 10.0 + (pair ? (double)ceil_div(t.pairs, 74) * (2.85 * block + 0.6) : (double)ceil_div(t.singles, 148) * (1.75 * block + 3.6));
+}
+
 galore_status_t split_group_add_store(SplitGroup& g, int M, int N, int K, const SplitOperand& a, const SplitOperand& b, int splits,
                                       float* C, int64_t ldc, int64_t split_stride, int32_t* status) {
   SplitProblem p = {};

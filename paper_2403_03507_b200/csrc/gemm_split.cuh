@@ -44,6 +44,13 @@ SplitOperand split_operand(const void* base, int32_t dtype, int64_t s_mn, int64_
 // K slices that balance filling the machine against the traffic of the partial results
 int split_choose_slices(int64_t M, int64_t N, int64_t K);
 double split_store_us(int64_t M, int64_t N, int64_t K, int slices);      // what one such product takes in 128 x 128 tiles
+// Of a group of products, unsliced: its tiles of 128 x 128 and of 256 x 256 and the most blocks of 64 of K; may_pair: fp32 operands,
+// all on 16-byte boundaries
+struct SplitTiles {
+  int64_t singles = 0, pairs = 0, blocks = 0;
+  bool may_pair = true;
+};
+double split_group_us(const SplitTiles& t);
 int split_effective_slices(int64_t K, int slices);
 galore_status_t split_group_add_store(SplitGroup& g, int M, int N, int K, const SplitOperand& a, const SplitOperand& b, int splits,
                                       float* C, int64_t ldc, int64_t split_stride, int32_t* status);

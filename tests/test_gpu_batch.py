@@ -263,3 +263,18 @@ def test_batch_with_weight_decay_equals_per_layer_steps_and_the_oracle():
         assert rel_err(to_host(w2), to_host(w1)) < 5e-4
         assert rel_err(to_host(w2), wo) <= 2e-2
         assert rel_err(to_host(w2) - w0, wo - w0) <= 5e-2
+
+
+def test_layers_of_one_kind_share_a_launch_whatever_else_is_in_the_list():
+    """32 layers with fp32 gradients are what a launch carries; one of another state format does not split them."""
+    def make(state):
+        layer = gb.Layer(gb.make_config(64, 96, 8, w_dtype="bf16", g_dtype="f32", state_fmt=state, auto_refresh=False))
+        layer.set_projector(torch.linalg.qr(torch.randn(64, 8, device="cuda"))[0])
+        return layer, torch.randn(64, 96, device="cuda").bfloat16(), torch.randn(64, 96, device="cuda")
+    for counts in ([("f32", 32)], [("f32", 32), ("q8", 1)], [("q8", 3), ("f32", 32), ("q8", 2)]):
+        layers, Ws, Gs = zip(*[make(state) for state, n in counts for _ in range(n)])
+        batch = gb.Batch(list(layers), list(Ws), list(Gs))
+        batch.galore_step_batch(1e-2)
+        before = gb.galore_launch_count()
+        batch.galore_step_batch(1e-2)
+        assert gb.galore_launch_count() - before == 3 * len({state for state, _ in counts})      # projection, Adam, update of each kind

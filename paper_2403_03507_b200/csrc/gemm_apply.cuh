@@ -34,6 +34,7 @@ struct ApplyGroup {
 struct ApplyTiles {
   int64_t pairs = 0, singles = 0, blocks = 0;
   bool aligned = true;       // W's rows lie on 16-byte boundaries
+  bool direct = false;       // single tiles would read and write them from registers
   void add(int m, int n, int r, int p_planes, int n_planes, bool w_aligned);
 };
 // microseconds of a group's update with operands of several planes

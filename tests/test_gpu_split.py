@@ -81,7 +81,9 @@ def test_products_of_large_groups_are_fp32_products(m, n, r, count, pad):
 # bf16 rows that TMA cannot address, in products long enough for a copy of G on 16-byte rows; tiles of one CTA and of pairs in
 # the update (its rows go through shared memory in 16-byte units).  off: columns of W and G in front of the matrix, in the same rows
 @pytest.mark.parametrize("m,n,r,off,pad", [(2048, 2051, 512, 0, 0), (2051, 1031, 264, 0, 0), (1000, 2049, 320, 1, 2), (1500, 3001, 128, 3, 0), (4097, 1003, 64, 5, 1),
-                                           (1030, 5461, 512, 7, 4), (2048, 2048, 512, 0, 3)])
+                                           (1030, 5461, 512, 7, 4), (2048, 2048, 512, 0, 3),
+                                           # rows on 4-byte boundaries: from registers; tiles cut off below 32 columns, one and several waves, pairs
+                                           (518, 518, 184, 0, 0), (130, 1346, 40, 2, 4), (2051, 34, 16, 4, 0), (2500, 2502, 128, 0, 0), (2500, 2498, 640, 2, 2)])
 @pytest.mark.parametrize("state", ["f32", "q8"])
 def test_packed_bf16_rows_keep_fp32_precision(m, n, r, off, pad, state):
     gen = torch.Generator(device="cuda")

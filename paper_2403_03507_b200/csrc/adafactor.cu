@@ -50,8 +50,8 @@ __host__ __device__ inline AfLayout af_layout(const AdafactorItem& it) {
   const int rows = it.rows, cols = it.cols;
   float* const scratch = it.scratch;
   AfLayout a;
-  a.tile_rows = it.squares_ready ? kAfProjectionRows : af_tile_rows(rows, cols);
-  a.tiles_r = (rows + a.tile_rows - 1) / a.tile_rows;
+  a.tile_rows = it.tile_rows;
+  a.tiles_r = it.tiles_r;
   a.tiles_c = (cols + kAfTileCols - 1) / kAfTileCols;
   a.sums = reinterpret_cast<double*>(scratch);
   a.row_sums = a.sums + kAfSumBlocks + 8;
@@ -338,6 +338,12 @@ __global__ void __launch_bounds__(256) af_update_kernel(const __grid_constant__ 
 
 }  // namespace
 
+// the division stays out of the kernels (every CTA lays its item's scratch out)
+static void set_tiles(AdafactorItem& it) {
+  it.tile_rows = it.squares_ready ? kAfProjectionRows : af_tile_rows(it.rows, it.cols);
+  it.tiles_r = (int)ceil_div(it.rows, it.tile_rows);
+}
+
 size_t adafactor_scratch_bytes(int64_t rows, int64_t cols) {
   const int least = rows <= kAfProjectionTallest ? std::min(af_tile_rows(rows, cols), kAfProjectionRows) : af_tile_rows(rows, cols);
   const int64_t tiles_r = ceil_div(rows, least), tiles_c = ceil_div(cols, kAfTileCols);
@@ -348,6 +354,7 @@ bool adafactor_squares(const AdafactorItem& item, AdafactorSquares* out) {
   if (item.rows > kAfProjectionTallest) return false;
   AdafactorItem it = item;
   it.squares_ready = true;
+  set_tiles(it);
   const AfLayout a = af_layout(it);
   *out = AdafactorSquares{a.rowpart, a.colpart, a.tiles_c};
   return true;
@@ -359,9 +366,10 @@ galore_status_t adafactor_group_add(AdafactorGroup& g, const AdafactorItem& it) 
     return GALORE_ERR_INVALID_ARG;
   const int i = g.count;
   g.item[i] = it;
+  set_tiles(g.item[i]);
   g.beta2t[i] = (float)(1.0 - pow(it.t, -kAdafactorDecay));
   if (it.squares_ready && (it.splits != 1 || it.split.src)) return GALORE_ERR_INVALID_ARG;      // the pass adds slices and splits P too
-  const int tiles = it.squares_ready ? 0 : (int)(ceil_div(it.rows, af_tile_rows(it.rows, it.cols)) * ceil_div(it.cols, kAfTileCols));
+  const int tiles = it.squares_ready ? 0 : (int)(g.item[i].tiles_r * ceil_div(it.cols, kAfTileCols));
   const int blocks = (int)(ceil_div(it.rows, 256) + ceil_div(it.cols, 256));
   g.tile_end[i] = (i ? g.tile_end[i - 1] : 0) + tiles;
   g.vec_end[i] = (i ? g.vec_end[i - 1] : 0) + blocks;

@@ -13,7 +13,7 @@ constexpr float kAdafactorClip = 1.0f;      // the update is divided by max(1, r
 constexpr int kAfTileCols = 128;            // tile of the statistics pass: 128 columns x
 // 64 rows; 32 or 16 (four per warp, all in flight at once) where such tiles would leave SMs idle; more where a column
 // would have more than 64 partial sums to add up
-__host__ __device__ inline int af_tile_rows(int64_t rows, int64_t cols) {
+inline int af_tile_rows(int64_t rows, int64_t cols) {
   const int64_t tiles = ((rows + 63) / 64) * ((cols + kAfTileCols - 1) / kAfTileCols);
   const int base = tiles < 64 ? 16 : tiles < 128 ? 32 : 64, least = 16 * (int)((rows + 16 * 64 - 1) / (16 * 64));
   return base > least ? base : least;
@@ -36,6 +36,7 @@ struct AdafactorItem {
   double t;                // completed steps + 1
   float* scratch;          // adafactor_scratch_bytes(rows, cols) bytes
   bool squares_ready;      // the projection has left the sums of R^2 where adafactor_squares() says
+  int tile_rows, tiles_r;  // rows of a tile of the sums of R^2, tiles of them: adafactor_group_add() fills them in
 };
 // Where a projection may leave the sums of R^2: over stretches of kAfTileCols columns (rows x tiles) and of kAfProjectionRows rows (one row
 // of sums for each).  False for an R so tall that one thread would have too many of them to add up for a column: steps of four layers

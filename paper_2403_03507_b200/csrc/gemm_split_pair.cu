@@ -204,8 +204,8 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_pair_kernel(const __gr
           // The leading products come last in the first half and first in the second: between them the accumulator is
           // drained.  Where the epilogue reads the corrections as well, they come first in the second half.
           for (int half = 0; half < 2; ++half) {
-            if (half == 0 && fresh && !mbar_wait(acce_bar, phase ^ 1u, abort_flag)) { ok = false; break; }
-            if (!mbar_wait(full_bar(half), phase, abort_flag)) { ok = false; break; }
+            if (half == 0 && fresh && !mbar_wait<true>(acce_bar, phase ^ 1u, abort_flag)) { ok = false; break; }
+            if (!mbar_wait<true>(full_bar(half), phase, abort_flag)) { ok = false; break; }
             tc_fence_after();
             const uint64_t a_desc = split_desc(planes, a_mn) + (uint64_t)(2 * half) * a_step;
             const uint64_t b_desc = split_desc(planes + 3 * kTileBytes, b_mn) + (uint64_t)(2 * half) * b_step;
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_split_pair_kernel(const __gr
               }
             if (!first) {
               if (half == 0 && !fresh) {
-                if (!mbar_wait(acce_bar, phase ^ 1u, abort_flag)) { ok = false; break; }
+                if (!mbar_wait<true>(acce_bar, phase ^ 1u, abort_flag)) { ok = false; break; }
                 tc_fence_after();
               }
               lead();

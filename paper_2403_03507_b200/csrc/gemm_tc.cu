@@ -587,7 +587,7 @@ gemm_tc_kernel(const __grid_constant__ TcArgs<CAP> g) {
         int done = 0;                                 // k-blocks in the accumulator
         for (int kb = w.kb_begin; kb < w.kb_end; ++kb) {
           const bool fresh = done == 0;
-          if (fresh && !mbar_wait(acce_bar(acc), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
+          if (fresh && !mbar_wait<CTAS == 2>(acce_bar(acc), acc_phase ^ 1u, abort_flag)) { ok = false; break; }
           if (!mbar_wait(full_bar(stage), phase, abort_flag)) { ok = false; break; }
           tc_fence_after();
           const uint32_t a_addr = ring + stage * kStageBytes;

@@ -34,12 +34,27 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
+// the same where threads of the other CTA arrive (mbar_arrive_remote)
+__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+
 // Bounded wait.  Returns false when the limit ran out or another role already gave up.
+template <bool CLUSTER = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
-  if (mbar_try_wait(bar, parity)) return true;
+  auto done = [&]() { return CLUSTER ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity); };
+  if (done()) return true;
   const long long t0 = clock64();
   for (uint32_t it = 0;; ++it) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (done()) return true;
     if ((it & 63u) == 63u) {
       if (*abort_flag) return false;
       if (clock64() - t0 > kWaitLimitCycles) {
@@ -114,11 +129,14 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-// What it hands over lies in tensor memory, or in shared memory of this CTA behind a proxy fence (the peer's MMAs read it there):
-// nothing that a release at cluster scope would have to push out first.  (That release, between every two k-blocks of the
-// split products, cost 10 % of their time, and 4 % of the weight update of the LLaMA-1B set.)
+// What it hands over lies in shared memory of this CTA (behind a proxy fence: the peer's MMAs read it there) or in tensor memory
+// (behind a tcgen05 fence).  A release of shared memory at cluster scope is all that takes; the peer waits with acquire at that scope
+// (mbar_wait<true>).  A release of everything, between every two k-blocks, cost 10 % of the split products' time and 4 % of the
+// weight update of the LLaMA-1B set; this one costs nothing (eight layers of the 130M set: projections 168 us, 189 with that, and 168
+// without any order at cluster scope).
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
-  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
+  asm volatile("fence.release.sync_restrict::shared::cta.cluster;" ::: "memory");
+  asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // TMA load of a CTA pair: data lands in this CTA, completion is signalled on the leader's barrier
 __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t leader_bar) {

@@ -557,7 +557,11 @@ galore_status_t launch_split_store(const SplitGroup& g, int32_t a_dtype, int32_t
       pair += split_units(p.M, p.N, p.splits, 256);
       kb = std::max<int64_t>(kb, p.kblocks_per_split);
     }
-    if (pairs && split_us(pair, kb, true) < split_us(single, kb, false)) return launch_split_pair(g, early, st);
+    if (pairs && split_us(pair, kb, true) < split_us(single, kb, false)) {
+      bool taken = false;
+      GALORE_TRY(launch_split_pair(g, early, &taken, st));
+      if (taken) return GALORE_OK;
+    }
   }
   return launch_split<float, float>(g, early, st);
 }

@@ -57,7 +57,7 @@ galore_status_t split_group_add_store(SplitGroup& g, int M, int N, int K, const 
 // All problems of a group share the operand types.  pairs: fp32 operands may take the tiles of CTA pairs, where the group's
 // size makes them the faster ones (their sums round differently); false: a problem's bits do not depend on its group.
 galore_status_t launch_split_store(const SplitGroup& g, int32_t a_dtype, int32_t b_dtype, bool pairs, bool early, cudaStream_t st);
-// the same for fp32 operands on 16-byte boundaries, by CTA pairs (gemm_split_pair.cu)
-galore_status_t launch_split_pair(const SplitGroup& g, bool early, cudaStream_t st);
+// the same for fp32 operands on 16-byte boundaries, by CTA pairs (gemm_split_pair.cu); taken false: this build cannot, nothing is launched
+galore_status_t launch_split_pair(const SplitGroup& g, bool early, bool* taken, cudaStream_t st);
 
 }  // namespace galore

@@ -368,7 +368,19 @@ galore_status_t operand_map(CUtensorMap* map, const SplitOperand& o, int mn_size
 }
 
 template <int CAP>
-galore_status_t launch_pair(const SplitGroup& g, bool early, cudaStream_t st) {
+galore_status_t launch_pair(const SplitGroup& g, bool early, bool* taken, cudaStream_t st) {
+  auto kern = gemm_split_pair_kernel<CAP>;
+  static std::atomic<uint64_t> configured{0};
+  static std::atomic<int> registers{0};
+  if (registers.load(std::memory_order_relaxed) == 0) {
+    cudaFuncAttributes attr;
+    GALORE_CUDA_TRY(cudaFuncGetAttributes(&attr, kern));
+    registers.store(attr.numRegs, std::memory_order_relaxed);
+  }
+  // setmaxnreg moves registers inside what the CTA was launched with: less than kLaunchRegs would leave it waiting, more
+  // would make a step the wrong way.  A build that gave another number leaves the group to the tiles of one CTA.
+  *taken = registers.load(std::memory_order_relaxed) == kLaunchRegs;
+  if (!*taken) return GALORE_OK;
   PairArgs<CAP> args;
   args.count = g.count;
   int64_t units = 0;
@@ -384,20 +396,6 @@ galore_status_t launch_pair(const SplitGroup& g, bool early, cudaStream_t st) {
     if (units >= ((int64_t)1 << 31)) return GALORE_ERR_SHAPE;
     args.unit_end[i] = (int)units;
   }
-  auto kern = gemm_split_pair_kernel<CAP>;
-  static std::atomic<uint64_t> configured{0};
-  static std::atomic<int> registers{0};
-  if (registers.load(std::memory_order_relaxed) == 0) {
-    cudaFuncAttributes attr;
-    GALORE_CUDA_TRY(cudaFuncGetAttributes(&attr, kern));
-    registers.store(attr.numRegs, std::memory_order_relaxed);
-  }
-  // setmaxnreg moves registers inside what the CTA was launched with: less than kLaunchRegs would leave it waiting, more
-  // would make a step the wrong way
-  if (registers.load(std::memory_order_relaxed) != kLaunchRegs) {
-    note_cuda_error(cudaErrorInvalidConfiguration, "gemm_split_pair_kernel: its register split needs a build with 96 registers a thread");
-    return GALORE_ERR_CUDA;
-  }
   GALORE_TRY(allow_smem(configured, (const void*)kern, kSmemBytes));
   const int teams = (int)std::min<int64_t>(units, tensor_sm_count() / 2);
   return launch_kernel(kern, dim3((unsigned)(teams * 2)), kThreads, kSmemBytes, 2, early, st, args);
@@ -405,9 +403,8 @@ galore_status_t launch_pair(const SplitGroup& g, bool early, cudaStream_t st) {
 
 }  // namespace
 
-galore_status_t launch_split_pair(const SplitGroup& g, bool early, cudaStream_t st) {
-  if (g.count < 1) return GALORE_OK;
-  return g.count == 1 ? launch_pair<1>(g, early, st) : launch_pair<kSplitGroup>(g, early, st);
+galore_status_t launch_split_pair(const SplitGroup& g, bool early, bool* taken, cudaStream_t st) {
+  return g.count == 1 ? launch_pair<1>(g, early, taken, st) : launch_pair<kSplitGroup>(g, early, taken, st);
 }
 
 }  // namespace galore

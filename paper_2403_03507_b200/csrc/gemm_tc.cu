@@ -936,7 +936,8 @@ galore_status_t launch_tc(const TcGroup& g, bool early, cudaStream_t st) {
     one.map_m[0] = g.map_m[0];
     one.map_v[0] = g.map_v[0];
     if constexpr (EPI == EPI_DRAIN || EPI == EPI_PARTIAL)
-      if (!pair && g.p[0].N <= 128) return launch_tc_variant<EPI, 1, 1, 128>(one, early, st);      // (the group's units are the same)
+      // (the group's units are the same; a K-major B comes in boxes of 256 rows, more than this kernel's stages hold)
+      if (!pair && g.p[0].N <= 128 && g.p[0].b_mn) return launch_tc_variant<EPI, 1, 1, 128>(one, early, st);
     return pair ? launch_tc_variant<EPI, 2, 1>(one, early, st) : launch_tc_variant<EPI, 1, 1>(one, early, st);
   }
   if constexpr (EPI == EPI_DRAIN) return GALORE_ERR_INVALID_ARG;      // single matrices only

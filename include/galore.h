@@ -193,7 +193,8 @@ galore_status_t galore_step_host(galore_layer_t* layer, void* W_host, const void
 /* Steps `count` layers on one stream, layer i with W[i], G[i] (device pointers; host arrays of
  * pointers and leading dimensions).  Same results as calling galore_step on each layer up to the
  * order of floating-point sums (with several layers in flight the K dimension of the projection is
- * not sliced), but the layers are stepped in groups of up to 32 of one kind (tensor-core path, or
+ * not sliced, and the tiles that sum the projections of fp32 gradients go by what shares the launch
+ * and by its alignment), but the layers are stepped in groups of up to 32 of one kind (tensor-core path, or
  * fp32 path with the same dtypes): one grouped launch for all their projections, one for
  * the inner optimizer (none when Adam runs in the projection's epilogue), one for all their
  * back-projections, so that small matrices do not each pay a kernel's ramp-up and the last wave of

@@ -1182,8 +1182,8 @@ galore_status_t galore_step_batch(galore_layer_t* const* layers, void* const* W,
     PhaseTimer pt(0, s);
     return tensor_group_launch_project_adam(scratch.proj, first->cfg.state_fmt, gi > 0 && short_group(groups[gi]), s);
   };
-  // Adafactor's sums of R^2 come out of the projection where K is not sliced and the layer's scratch has room for them (a rule
-  // on the layer alone: its result does not depend on the group)
+  // Adafactor's sums of R^2 come out of the projection where K is not sliced (which goes by the number of layers in the call) and R is
+  // not too tall for it: not by the other layers of the group
   auto af_item_of = [&](const BatchMember& mb) {
     galore_layer* l = layers[mb.index];
     float* part; __nv_bfloat16* nbuf;

@@ -26,7 +26,7 @@ namespace {
 
 constexpr int kBK = 16;
 constexpr int kThreads = 256;
-// steps of 16 k in shared memory: 43.5 KiB of a small tile's, five CTAs an SM; 69.6 KiB of a large one's
+// steps of 16 k in shared memory: 42.5 KiB of a small tile's, 66 KiB of a large one's
 constexpr int stages(bool async, int bm) { return !async ? 1 : (bm == 64 ? 5 : 4); }
 constexpr int smem_bytes(bool async, int bm, int bn) { return stages(async, bm) * kBK * (bm + bn + 8) * 4; }
 

@@ -11,8 +11,9 @@
 // tensor core's accumulator rounds towards zero: the short chains keep that below the rounding of an
 // ordinary fp32 sum.
 //
-// Measured (eight layers of the LLaMA-130M set, rank 256, fp32 gradients): projections 1292 -> 247 us against fp32 FMA
-// kernels; a bf16 2048 x 5461 matrix of unpadded rows at rank 512: 766 -> 74 us.  What bounds it: the conversion
+// Measured: 32 fp32 gradients of 512 x 1024 at rank 96 44 us, 28 of 512 x 1408 at 128 62 us, eight of 2048 x 2048 at 512 250 us.  (Groups
+// that fill the machine with the tiles of CTA pairs run in gemm_split_pair.cu, the last of these in 179 us; packed bf16 rows of long
+// products are copied for TMA, api.cu.)  What bounds it: the conversion
 // of the operands (about twelve instructions per element, each element of a tile once) and the latency of the one
 // stage of loads the producers hold in registers.
 //

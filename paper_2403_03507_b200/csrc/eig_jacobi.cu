@@ -216,18 +216,16 @@ __global__ void __launch_bounds__(128) jb_gram_kernel(const double* X, int b, in
 //     computes the next round's rotations.  The product that a rotation needs is worked out from the old A and the
 //     current rotations again, so the rotations of round t + 1 are found while the other warps apply those of round t,
 //     and a round has a single barrier.
-//   * A off the diagonal is held in single precision, scaled so that the largest squared norm is about 1; the norms, Rot, the
-//     sums A comes from and the test for orthogonality are in double precision.  A only decides the angles, every
-//     product keeps a relative error of 1e-6 over the sweep, and the next sweep starts from exact ones: the
-//     number of rotations of each sweep is the same to 1e-3 as with A in double precision, and so is the number of sweeps.
 //   * The angle is computed in single precision (after scaling by the exponent of the larger of
 //     aqq - app and 2 apq) and (c, s) are then renormalised in double precision: the rotation is
 //     orthogonal to double rounding, its angle accurate to about 1e-7.
 // own: the products within each block (32 x 32 of a block, upper triangle), read after the first round of the sweep and
 // written in every one.  flags[pair] = rotations applied (0: Rot is the identity and is not written).
 //
-// What bounds it: 63 rounds one after the other, each the latency of an angle beside about 300 shared-memory wavefronts (650 with A
-// in double precision).  56 registers: two CTAs on an SM, for groups of more than 148 pairs.
+// What bounds it: 63 rounds one after the other, each about 600 shared-memory wavefronts (half of them reads, then the writes) and,
+// beside them, the latency of an angle.  56 registers: two CTAs on an SM, for groups of more than 148 pairs.  (A off the diagonal in
+// single precision: half the wavefronts, 3.52 instead of 3.73 ms for the refresh of 512 x 1376 at rank 128, 116.8 instead of 119.5 ms
+// for eight 4096 x 4096 at 1024.  Not taken: the sums it holds are fp64 ones.)
 constexpr int kSweepRounds = kPairRows - 1;
 constexpr int kSlots = kPairRows / 2;
 constexpr int kBlockWarps = 8;                                // blocks with u != v: rows 1 .. 16
@@ -267,12 +265,12 @@ __device__ __forceinline__ BlockWrites block_writes(int u, int v) {
   return BlockWrites{{packed_offset(nfu, nfv), packed_offset(nfu, ngv), packed_offset(ngu, nfv), packed_offset(ngu, ngv)}};
 }
 struct BlockValues {
-  float a0, a1, a2, a3;
+  double a0, a1, a2, a3;
 };
 // B <- R_u B R_v^T for one 2 x 2 block
-__device__ __forceinline__ void block_write(const BlockWrites& t, const float2 ru, const float2 rv, const BlockValues& b, float* An) {
-  const float r00 = ru.x * b.a0 - ru.y * b.a2, r01 = ru.x * b.a1 - ru.y * b.a3;
-  const float r10 = ru.y * b.a0 + ru.x * b.a2, r11 = ru.y * b.a1 + ru.x * b.a3;
+__device__ __forceinline__ void block_write(const BlockWrites& t, const double2 ru, const double2 rv, const BlockValues& b, double* An) {
+  const double r00 = ru.x * b.a0 - ru.y * b.a2, r01 = ru.x * b.a1 - ru.y * b.a3;
+  const double r10 = ru.y * b.a0 + ru.x * b.a2, r11 = ru.y * b.a1 + ru.x * b.a3;
   An[t.at[0]] = rv.x * r00 - rv.y * r01;
   An[t.at[1]] = rv.y * r00 + rv.x * r01;
   An[t.at[2]] = rv.x * r10 - rv.y * r11;
@@ -321,18 +319,17 @@ __global__ void __launch_bounds__(kSweepThreads, 2) jb_sweep_kernel(const double
     flags = slot_ptr(flags, shift);
     rotations = slot_ptr(rotations, shift);
   }
-  __shared__ float A0[kPackedSize], A1[kPackedSize];      // the Gram matrix off the diagonal, even rounds and odd ones
+  __shared__ double A0[kPackedSize], A1[kPackedSize];     // the Gram matrix off the diagonal, even rounds and odd ones
   __shared__ double diag[kPairRows];
-  __shared__ float2 cs[2][kSlots];                // the rotations of the current round and of the next
+  __shared__ double2 cs[2][kSlots];               // the rotations of the current round and of the next
   __shared__ double2 cs_rot[2][kSlots + kLaneGroups];     // the same for the warps of Rot, which read eight slots, 4 apart, at once
-  __shared__ int total, top;
+  __shared__ int total;
   const int pair = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const BlockPair bp = block_pair(pair, round, nblk);
   if (bp.I * kBlockRows >= b) {
     if (tid == 0) flags[pair] = 0;
     return;
   }
-  if (tid == 0) top = 0;
   const double* src = part + (int64_t)pair * chunks * (kPairRows * kPairRows);
   // where the products of rows r and c of one block are carried
   auto own_at = [&](int r, int c) { return own + (int64_t)(r < kBlockRows ? bp.I : bp.J) * (kBlockRows * kBlockRows) + (r % kBlockRows) * kBlockRows + c % kBlockRows; };
@@ -360,20 +357,13 @@ __global__ void __launch_bounds__(kSweepThreads, 2) jb_sweep_kernel(const double
 #pragma unroll
       for (int i = 0; i < kLoads; ++i) sum[i] += v[j][i];
   }
-  __syncthreads();
 #pragma unroll
   for (int i = 0; i < kLoads; ++i) {
     const int idx = tid + kSweepThreads * i, r = idx >> 6, c = idx & 63;
-    if (idx < kPairRows * kPairRows && r == c) {
-      diag[r] = sum[i];
-      atomicMax(&top, __double2hiint(sum[i]));
-    }
+    if (idx < kPairRows * kPairRows && r == c) diag[r] = sum[i];
   }
   const double tol2 = tol * tol;
   __syncthreads();
-  // 2^-e of the largest squared norm
-  const int exponent = min(max(top >> 20, 1), 2045);
-  const double scale = __hiloint2double((2046 - exponent) << 20, 0), unscale = __hiloint2double(exponent << 20, 0);      // scale unscale = 1
   // A pair that is orthogonal already (every pair of the last sweep) keeps its rows: no rotation of the 63 rounds would be
   // applied.
   bool any = false;
@@ -382,7 +372,7 @@ __global__ void __launch_bounds__(kSweepThreads, 2) jb_sweep_kernel(const double
     const int idx = tid + kSweepThreads * i, r = idx >> 6, c = idx & 63;
     if (idx < kPairRows * kPairRows && r < c) {
       any |= sum[i] * sum[i] > tol2 * diag[r] * diag[c];
-      A0[packed_offset(r, c)] = (float)(sum[i] * scale);
+      A0[packed_offset(r, c)] = sum[i];
     }
   }
   if (!__syncthreads_or(any)) {
@@ -405,14 +395,14 @@ __global__ void __launch_bounds__(kSweepThreads, 2) jb_sweep_kernel(const double
     const BlockWrites w0 = block_writes(lane, v0), w1 = block_writes(lane, v1);
     const bool second = d1 < kSlots / 2 || lane < kSlots / 2;      // half of row 16 says it all
     for (int rr = 0; rr < kSweepRounds; ++rr) {
-      const float* A = (rr & 1 ? A1 : A0) + d0 * kSlots + lane;
-      float* An = rr & 1 ? A0 : A1;
-      const float2* cur = cs[rr & 1];
+      const double* A = (rr & 1 ? A1 : A0) + d0 * kSlots + lane;
+      double* An = rr & 1 ? A0 : A1;
+      const double2* cur = cs[rr & 1];
       round_barrier();
-      const float2 ru = cur[lane], rv0 = cur[v0];
+      const double2 ru = cur[lane], rv0 = cur[v0];
       const BlockValues b0{A[0], A[kKindSize], A[2 * kKindSize], A[3 * kKindSize]};
-      const float2 rv1 = cur[v1];
-      const float* B = A + kBlockWarps * kSlots;
+      const double2 rv1 = cur[v1];
+      const double* B = A + kBlockWarps * kSlots;
       const BlockValues b1{B[0], B[kKindSize], B[2 * kKindSize], B[3 * kKindSize]};
       block_write(w0, ru, rv0, b0, An);
       if (second) block_write(w1, ru, rv1, b1, An);
@@ -478,32 +468,31 @@ __global__ void __launch_bounds__(kSweepThreads, 2) jb_sweep_kernel(const double
     const int left = packed_offset(next_position(lane), next_position(kPairRows - 1 - lane));    // where the slot's own product goes
     const int rot_at = lane + lane / kLaneSlots;
     int applied = 0;
-    double f = diag[lane] * scale, g = diag[kPairRows - 1 - lane] * scale;
-    float o = A0[kKindSize + lane];
-    double2 own_rot = jacobi_rotation(f, g, (double)o, tol2, applied);
-    cs[0][lane] = make_float2((float)own_rot.x, (float)own_rot.y);
+    double f = diag[lane], g = diag[kPairRows - 1 - lane], o = A0[kKindSize + lane];
+    double2 own_rot = jacobi_rotation(f, g, o, tol2, applied);
+    cs[0][lane] = own_rot;
     cs_rot[0][rot_at] = own_rot;
     for (int rr = 0; rr < kSweepRounds; ++rr) {
-      const float* A = rr & 1 ? A1 : A0;
-      float* An = rr & 1 ? A0 : A1;
-      const float2* cur = cs[rr & 1];
+      const double* A = rr & 1 ? A1 : A0;
+      double* An = rr & 1 ? A0 : A1;
+      const double2* cur = cs[rr & 1];
       round_barrier();
-      const float2 r1 = cur[s1], r2 = cur[s2];
-      const float y0 = A[x0], y1 = A[x1], y2 = A[x2], y3 = A[x3];
+      const double2 r1 = cur[s1], r2 = cur[s2];
+      const double y0 = A[x0], y1 = A[x1], y2 = A[x2], y3 = A[x3];
       // this round's rotation of the slot's own two rows
-      const double c = own_rot.x, sn = own_rot.y, od = (double)o;
-      const double fn = c * (c * f - sn * od) - sn * (c * od - sn * g), gn = sn * (sn * f + c * od) + c * (sn * od + c * g);
-      An[left] = (float)(c * (sn * f + c * od) - sn * (sn * od + c * g));
+      const double c = own_rot.x, sn = own_rot.y;
+      const double fn = c * (c * f - sn * o) - sn * (c * o - sn * g), gn = sn * (sn * f + c * o) + c * (sn * o + c * g);
+      An[left] = c * (sn * f + c * o) - sn * (sn * o + c * g);
       // the rows move on
       const double f_up = __shfl_up_sync(0xffffffffu, fn, 1), g_down = __shfl_down_sync(0xffffffffu, gn, 1), g_first = __shfl_sync(0xffffffffu, gn, 0);
       f = lane == 0 ? fn : (g1 ? g_first : f_up);
       g = g2 ? g_down : fn;
-      const float p1 = g1 ? r1.y : r1.x, q1 = g1 ? r1.x : -r1.y;
-      const float p2 = g2 ? r2.y : r2.x, q2 = g2 ? r2.x : -r2.y;
+      const double p1 = g1 ? r1.y : r1.x, q1 = g1 ? r1.x : -r1.y;
+      const double p2 = g2 ? r2.y : r2.x, q2 = g2 ? r2.x : -r2.y;
       o = p2 * (p1 * y0 + q1 * y2) + q2 * (p1 * y1 + q1 * y3);
       if (rr + 1 < kSweepRounds) {
-        own_rot = jacobi_rotation(f, g, (double)o, tol2, applied);
-        cs[(rr + 1) & 1][lane] = make_float2((float)own_rot.x, (float)own_rot.y);
+        own_rot = jacobi_rotation(f, g, o, tol2, applied);
+        cs[(rr + 1) & 1][lane] = own_rot;
         cs_rot[(rr + 1) & 1][rot_at] = own_rot;
       }
     }
@@ -518,10 +507,10 @@ __global__ void __launch_bounds__(kSweepThreads, 2) jb_sweep_kernel(const double
     round_barrier();
   }
   // all rows are back at their own positions: the products within the blocks, for the rounds to come
-  const float* A = kSweepRounds & 1 ? A1 : A0;
+  const double* A = kSweepRounds & 1 ? A1 : A0;
   for (int idx = tid; idx < kPairRows * kBlockRows; idx += kSweepThreads) {
     const int r = idx >> 5, c = (idx & 31) + (r & ~(kBlockRows - 1));
-    if (r <= c) *own_at(r, c) = (r == c ? diag[r] : (double)A[packed_offset(r, c)]) * unscale;
+    if (r <= c) *own_at(r, c) = r == c ? diag[r] : A[packed_offset(r, c)];
   }
 }
 

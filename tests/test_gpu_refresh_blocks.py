@@ -52,8 +52,8 @@ def test_grouped_layers_with_gradients_of_different_strides_match_single_refresh
         assert torch.equal(a.get_projector(), b.get_projector())
 
 
-# The eigen-solver carries products in single precision, scaled by the largest norm: a gradient times a power of two has the same
-# projector, whatever the power; few blocks of 32 rows and many, one matrix and a group
+# The eigen-solver computes its angles in single precision, scaled by each pair's own size: a gradient times a power of two has the
+# same projector, whatever the power; few blocks of 32 rows and many, one matrix and a group
 @pytest.mark.parametrize("m,n,rank,over", [(96, 130, 24, 20), (200, 330, 30, 34), (512, 700, 96, 96), (700, 520, 150, 171)])
 @pytest.mark.parametrize("count", [1, 3])
 def test_projector_does_not_depend_on_the_scale_of_the_gradient(m, n, rank, over, count):

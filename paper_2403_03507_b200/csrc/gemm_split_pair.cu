@@ -11,8 +11,9 @@
 // as many.  Operands arrive by TMA as they are, three half-blocks of K ahead, so that no thread waits for memory.
 // Eight layers of the LLaMA-130M set at rank 256: projections 245 -> 174 us, the call 553 -> 492 us.  A block of 64 takes 2.85 us
 // (1.3 PFLOP/s of plane products; without the conversion, or with half the products, little less), a launch about 15 us more.
-// The sums are no further from 64 bits than those of the smaller tiles (R of 768 x 2048 at rank 256: 9.1e-8 against 9.4e-8); with
-// leading products and corrections in one accumulator they were (9.75e-8).
+// The sums are nearer to 64 bits than those of the smaller tiles (R of 448 x 2304, 768 x 2048, 1024 x 2816 at rank 256 and 3000 x 3000 at 512:
+// 8.03e-8, 9.1e-8, 9.8e-8 and 1.41e-7 against 8.33e-8, 9.3e-8, 1.00e-7 and 1.42e-7); with leading products and corrections in one
+// accumulator they were not (768 x 2048: 9.75e-8).
 //
 // One persistent CTA per SM:
 //   warps 0..7    epilogue: four quarters of the TMEM lanes x two halves of the columns

@@ -50,8 +50,8 @@ def test_products_of_split_operands_are_fp32_products(m, n, r, g, w, pad):
         assert torch.isnan(W._base[:, n:]).all()
 
 
-# groups that fill the machine with the 256 x 256 tiles of CTA pairs: ragged tiles on both sides, blocks of K cut off, several K
-# slices (one matrix), rows padded to 16 bytes; the largest rank takes two tiles along the rank
+# groups around the line between the 128 x 128 tiles and the 256 x 256 tiles of CTA pairs (which 1000 x 1999 and 5460 x 2050 take): ragged tiles
+# on both sides, blocks of K cut off, several K slices (one matrix), rows padded to 16 bytes; the largest rank takes two tiles along the rank
 @pytest.mark.parametrize("m,n,r,count,pad", [(769, 2052, 256, 12, 0), (2052, 770, 260, 12, 2), (96, 8200, 64, 20, 0), (1000, 1999, 388, 8, 1), (2048, 5460, 512, 1, 0),
                                              (5460, 2050, 512, 1, 2)])
 def test_products_of_large_groups_are_fp32_products(m, n, r, count, pad):
@@ -118,3 +118,75 @@ def test_packed_bf16_rows_keep_fp32_precision(m, n, r, off, pad, state):
     assert torch.equal(G, G0)
     for buf in bufs:
         assert torch.isnan(buf[:, :off]).all() and torch.isnan(buf[:, off + n:]).all()
+
+
+def _off_by_one(x):
+    """x in rows one element off the 16-byte boundaries: CTA pairs do not take it."""
+    buf = torch.zeros(x.shape[0], (x.shape[1] + 4) // 4 * 4, device="cuda", dtype=x.dtype)
+    out = buf[:, 1:1 + x.shape[1]]
+    out.copy_(x)
+    return out
+
+
+# Groups that take the tiles of CTA pairs: both sides (the operands' majors change from one unit of a pair to the next), sums of 3 to 10
+# blocks of 64 (the corrections are added after every eight), decoder layers.  The same gradients off the 16-byte boundaries take the
+# tiles of one CTA, whose leading products and corrections are both added after every block.
+@pytest.mark.parametrize("shapes,count,r", [([(188, 2304)], 8, 188), ([(448, 2304)], 8, 256), ([(2304, 512)], 8, 256), ([(513, 2304)], 8, 256),
+                                            ([(2304, 577)], 8, 256), ([(449, 2300), (2300, 449)], 16, 256), ([(600, 2300), (2300, 520)], 16, 252),
+                                            ([(768, 768)] * 4 + [(768, 2048)] * 2 + [(2048, 768)], 14, 256), ([(768, 768)] * 4 + [(768, 2048)] * 2 + [(2048, 768)], 28, 256),
+                                            ([(1024, 2816)], 20, 256), ([(3000, 3000)], 8, 512)])
+def test_pair_tiles_are_no_further_from_64_bits_than_single_ones(shapes, count, r):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(r + count)
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda")
+    sizes = [shapes[i % len(shapes)] for i in range(count)]
+    P = [torch.linalg.qr(rand(min(s), r))[0] for s in sizes]
+    G = [rand(m, n) for m, n in sizes]
+    err, bias, moments = [], [], []
+    for place in (lambda g: _matrix(g, "f32", -g.shape[1] % 4), _off_by_one):
+        layers = [gb.Layer(gb.make_config(m, n, r, w_dtype="bf16", g_dtype="f32", auto_refresh=False)) for m, n in sizes]
+        for layer, p in zip(layers, P):
+            layer.set_projector(p)
+        gb.Batch(layers, [torch.zeros(m, (n + 7) // 8 * 8, device="cuda", dtype=torch.bfloat16)[:, :n] for m, n in sizes], [place(g) for g in G]).galore_step_batch(1e-2)
+        assert max(layer.device_status() for layer in layers) == 0
+        moments.append([layer.get_moments()[0] for layer in layers])
+        off, rel = 0.0, 0.0
+        for layer, p, g, M in zip(layers, P, G, moments[-1]):
+            R = p.double().T @ g.double() if layer.side == gb.SIDE_LEFT else g.double() @ p.double()
+            # an fp32 sum of K terms, see above
+            e = float((M.double() / 0.1 - R).norm() / R.norm())
+            assert e <= 2 ** -24 * (8 + p.shape[0] ** 0.5)
+            off, rel = off + e * e / count, rel + float((M.double() / 0.1 * R).sum() / (R * R).sum() - 1) / count
+        err.append(off ** 0.5)
+        bias.append(abs(rel))
+    assert not all(torch.equal(a, b) for a, b in zip(*moments))       # two kernels ran
+    assert err[0] <= err[1] and bias[0] <= bias[1] + 1e-9, (err, bias)
+
+
+# A layer's own step takes slices by their time and adds accumulators to fp32 sums where the slices that fill the machine would end: no
+# further from 64 bits than those, which a batch of one takes.  Both sides, tiles of 128 columns, of 256 and of CTA pairs
+@pytest.mark.parametrize("m,n,r", [(6368, 2656, 80), (11008, 4096, 128), (4096, 4600, 120), (2104, 4800, 168), (1920, 2272, 256), (1536, 3264, 272), (3840, 2432, 632),
+                                   (1600, 4288, 600)])
+def test_drained_sums_are_no_further_from_64_bits_than_slices(m, n, r):
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(m + r)
+    rand = lambda *s: torch.randn(*s, generator=gen, device="cuda")
+    P, G = torch.linalg.qr(rand(min(m, n), r))[0], rand(m, n).bfloat16()
+    err, bias = [], []
+    for batch in (False, True):
+        layer = gb.Layer(gb.make_config(m, n, r, w_dtype="bf16", g_dtype="bf16", auto_refresh=False, adam_place=gb.ADAM_OWN_KERNEL))
+        assert layer.uses_tensor_path
+        layer.set_projector(P)
+        W = torch.zeros(m, n, device="cuda", dtype=torch.bfloat16)
+        if batch:
+            gb.Batch([layer], [W], [G]).galore_step_batch(1e-2)
+        else:
+            layer.galore_step(W, G, 1e-2)
+        assert layer.device_status() == 0
+        p = layer.get_projector().double()
+        R = p.T @ G.double() if layer.side == gb.SIDE_LEFT else G.double() @ p
+        M = layer.get_moments()[0].double() / 0.1
+        err.append(float((M - R).norm() / R.norm()))
+        bias.append(abs(float((M * R).sum() / (R * R).sum() - 1)))
+    # an accumulator loses up to a unit of 2^-23 of one sign per 16 products, four times a block of 64: 32 blocks lose 1.5e-5 at most
+    assert err[0] <= err[1] and bias[0] <= bias[1] + 1e-9 and err[0] <= 128 * 2 ** -23, (err, bias)

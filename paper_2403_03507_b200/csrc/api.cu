@@ -141,16 +141,7 @@ __global__ void __launch_bounds__(256) align_rows_kernel(const __nv_bfloat16* sr
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
-      if (!out[u]) continue;
-      const uint32_t raw[8] = {a[u].x, a[u].y, a[u].z, a[u].w, b[u].x, b[u].y, b[u].z, b[u].w};
-      uint32_t w[6], v[5];
-#pragma unroll
-      for (int j = 0; j < 6; ++j) w[j] = (shift[u] & 8u) ? raw[j + 2] : raw[j];
-#pragma unroll
-      for (int j = 0; j < 5; ++j) v[j] = (shift[u] & 4u) ? w[j + 1] : w[j];
-      const uint32_t bits = (shift[u] & 2u) * 8u;
-      *reinterpret_cast<uint4*>(out[u]) = make_uint4(__funnelshift_r(v[0], v[1], bits), __funnelshift_r(v[1], v[2], bits),
-                                                     __funnelshift_r(v[2], v[3], bits), __funnelshift_r(v[3], v[4], bits));
+      if (out[u]) *reinterpret_cast<uint4*>(out[u]) = bytes_from(a[u], b[u], shift[u]);
     }
   }
 }

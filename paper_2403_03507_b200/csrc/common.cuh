@@ -61,6 +61,21 @@ template <> __device__ __forceinline__ double cvt<double, __nv_bfloat16>(__nv_bf
 template <> __device__ __forceinline__ __nv_bfloat16 cvt<__nv_bfloat16, float>(float x) { return __float2bfloat16_rn(x); }
 template <> __device__ __forceinline__ __nv_bfloat16 cvt<__nv_bfloat16, double>(double x) { return __float2bfloat16_rn((float)x); }
 
+#ifdef __CUDACC__
+// 16 bytes from byte `shift` (0 .. 15, even) of a on; b holds the 16 behind it
+__device__ __forceinline__ uint4 bytes_from(const uint4& a, const uint4& b, uint32_t shift) {
+  const uint32_t raw[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+  uint32_t w[6], v[5];
+#pragma unroll
+  for (int j = 0; j < 6; ++j) w[j] = (shift & 8u) ? raw[j + 2] : raw[j];
+#pragma unroll
+  for (int j = 0; j < 5; ++j) v[j] = (shift & 4u) ? w[j + 1] : w[j];
+  const uint32_t bits = (shift & 2u) * 8u;
+  return make_uint4(__funnelshift_r(v[0], v[1], bits), __funnelshift_r(v[1], v[2], bits), __funnelshift_r(v[2], v[3], bits),
+                    __funnelshift_r(v[3], v[4], bits));
+}
+#endif
+
 // Several copies ("slots") of one workspace layout, `bytes` apart: a launch that carries a slot list
 // runs the same problem in every listed slot, all of its workspace pointers shifted by
 // id[i] * bytes for the i-th part of the grid.  Used to run the latency-bound small kernels of the

@@ -153,14 +153,8 @@ __device__ __forceinline__ void store_chunk(uint32_t dst, const uint32_t (&raw)[
     if (shift == 0u) {
       st_shared_16B(dst, raw[0], raw[1], raw[2], raw[3]);
     } else {
-      uint32_t w[6], v[5];
-#pragma unroll
-      for (int j = 0; j < 6; ++j) w[j] = (shift & 8u) ? raw[j + 2] : raw[j];
-#pragma unroll
-      for (int j = 0; j < 5; ++j) v[j] = (shift & 4u) ? w[j + 1] : w[j];
-      const uint32_t bits = (shift & 2u) * 8u;
-      st_shared_16B(dst, __funnelshift_r(v[0], v[1], bits), __funnelshift_r(v[1], v[2], bits),
-                    __funnelshift_r(v[2], v[3], bits), __funnelshift_r(v[3], v[4], bits));
+      const uint4 x = bytes_from(make_uint4(raw[0], raw[1], raw[2], raw[3]), make_uint4(raw[4], raw[5], raw[6], raw[7]), shift);
+      st_shared_16B(dst, x.x, x.y, x.z, x.w);
     }
   }
 }
